@@ -45,7 +45,7 @@ def arithmetic_name(prec: int, field_dtype: str) -> str:
     io = f"{field_dtype} in/out"
     return {0: f"f64 (banded solve), {io}",
             1: f"bf16 hi/lo split, 3 products, fp32 accumulate, {io}",
-            2: f"bf16 digit slices, 15 exact-integer products in fp32, {io}",
+            2: f"f16 digit slices, 10 exact-integer products in fp32, {io}",
             3: f"tf32, 1 product, fp32 accumulate, {io}"}[prec]
 
 WORKLOADS = {
@@ -789,9 +789,9 @@ def main():
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         byts = algorithmic_bytes(nint, nf, nops, elem) * prof_steps
         achieved = byts / (tl * 1e-3) / 1e9
-        pairs = 15 if prec == PREC["tc_bf16_exact"] else 3
+        pairs = 10 if prec == PREC["tc_bf16_exact"] else 3
         tcf = tc_flops(mesh, nf, pairs) * prof_steps / (tl * 1e-3) / 1e12 if nops == 9 else None
-        roof = {"kernel": "k_dense (tcgen05 BF16 digit-slice GEMM)", "bound": "hbm", "achieved": round(achieved, 1),
+        roof = {"kernel": "k_dense_exact (tcgen05 digit-slice GEMM)", "bound": "hbm", "achieved": round(achieved, 1),
                 "peak": hbm, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic_bytes_per_point_op": round(elem * (1 + nops) / nops, 3),
@@ -1111,7 +1111,7 @@ def run_advect(args, spec):
         ach = per_pf * units * prof_steps / (tdl * 1e-3) / 1e9
         nhl, thl = prof["dense_halo"]
         comb_b = (3 + 1 + 3 / nf) * elem * units * prof_steps
-        roof = {"kernel": "k_dense (tcgen05 BF16 digit-slice GEMM, biased operators D+ and D-)", "bound": "hbm",
+        roof = {"kernel": "k_dense_exact (tcgen05 digit-slice GEMM, biased operators D+ and D-)", "bound": "hbm",
                 "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic_bytes_per_point_field": round(per_pf, 2),

@@ -76,8 +76,9 @@ typedef enum cfd_status {
  */
 typedef enum cfd_precision {
   CFD_FP64_BANDED = 0,   /* FP64 right-hand side + Thomas solve per pencil */
-  CFD_TC_BF16X3 = 1,     /* dense D on BF16 tensor cores, hi/lo split, 3 products */
-  CFD_TC_BF16_EXACT = 2, /* dense D on BF16 tensor cores, exact integer slices (FP64-level result) */
+  CFD_TC_BF16X3 = 1,     /* dense D on the tensor cores, BF16 hi/lo split, 3 products */
+  CFD_TC_BF16_EXACT = 2, /* dense D on the tensor cores, exact integer slices (FP64-level result): four
+                            10-bit digits per factor in FP16, 10 products, FP32 accumulators */
   CFD_TC_TF32 = 3        /* dense D on TF32 tensor cores, one product, FP32 accumulation:
                             each pencil and D rounded to TF32 (same per-pencil scale);
                             measured max relative error against FP64 (tuned Q schemes,

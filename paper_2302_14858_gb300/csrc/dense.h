@@ -47,6 +47,10 @@ struct DenseParams {
   // TMA staging of the tile's pencils (0: cp.async path): 1 x rows (SWIZZLE_128B boxes of 128
   // bytes along x), 2 y columns (box [t1][y][x]), 3 z columns (box [z][t1][x])
   int tma_kind, tma_boxes, tma_bytes, tma_zstep;  // zstep: z planes per job in the tensor map
+  int nstg, stg_bytes;       // exact form: staging buffers (1 or 2) and bytes of one
+  // exact form, x stages: bytes of an epilogue warp's output box ([32 pencils][8 values]; 0: stores
+  // straight to memory) and the output as a tensor of N-value rows
+  int out_box_bytes;
   // Intermediate written on interior pencils only: each value within g of an x (and, with
   // ghost_y, a y) face is also written into the face neighbour's ghost column of the same box.
   // nl: [nblk][4] local indices of the x-, x+, y-, y+ face neighbours.
@@ -56,6 +60,7 @@ struct DenseParams {
   // launch over some blocks of a group writes into the group's intermediate boxes.
   const int *sc_local;
   CUtensorMap tmap;          // (the type carries its own 128-byte alignment)
+  CUtensorMap tmap_out;
   int *status;
   long long wait_limit;      // clock cycles a main-loop wait may take before it latches CFD_ERR_TIMEOUT
   float inv_tpj, inv_nf, inv_n2;  // 1 / tiles_per_job, 1 / nf, 1 / n2 (set at launch)
@@ -75,6 +80,10 @@ void halo_rows_from(const std::vector<long double> &M, int cols, HaloRows &R);
 // addressing of P, as k_dense reads it), the 4 rows of R applied to the pencil (and, with
 // P.halo_in, to the neighbours' previous iterate), written to P.halo_out.
 cfd_status halo_rows_launch(const DenseParams &P, const HaloRows &R, bool f32_in, cudaStream_t st);
+
+// One launch of the exact form (dense_exact.cuh) for blocks of 16^3 / 32^3.
+cfd_status dense_exact_launch16(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);
+cfd_status dense_exact_launch32(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);
 
 cfd_status dense_bind(cfd_blocks_s *B);
 void dense_set_tuning(cfd_blocks_s *B, bool on);

@@ -1,0 +1,73 @@
+// Host side of the exact tensor-core kernel: shared-memory plan and instantiation choice.
+#pragma once
+#include <algorithm>
+#include <atomic>
+
+#include "dense_exact.cuh"
+
+namespace cfd {
+namespace {
+
+constexpr size_t kSmemMax = 227 * 1024;
+
+// Shared memory of a launch: two A digit buffers, the operator digits, the staging buffers (two where
+// they fit), the epilogue's output boxes (x stages), row exponents, the pencil-scale ring and the barriers.  At least 116 KB, so that one CTA
+// (holding all TMEM columns) occupies an SM.
+template <typename TI, int N>
+size_t plan_smem(DenseParams &P) {
+  constexpr int KP = N == 32 ? 48 : 32;
+  const int E = N + 2 * P.g;
+  const size_t fixed = ((2 * (size_t)kSl * kTile * KP * 2 + (size_t)kSl * P.rows * KP * 2 + 1023) & ~(size_t)1023) +
+                       (64 + kXEtau * kTile) * 4 + 28 * 8 + 16;
+  const size_t rows = P.axis == 2 ? (size_t)((E * (int)sizeof(TI) + kXRowBytes - 1) / kXRowBytes) * kTile * kXRowBytes
+                                  : (size_t)E * kTile * sizeof(TI);
+  P.stg_bytes = (int)((rows + 1023) & ~(size_t)1023);
+  const size_t out = (size_t)P.out_box_bytes * kXEpiWarps;
+  P.nstg = fixed + out + 2 * (size_t)P.stg_bytes <= kSmemMax ? 2 : 1;
+  return std::max(fixed + out + (size_t)P.nstg * P.stg_bytes, (size_t)116 * 1024);
+}
+
+template <typename TI, typename TO, int N, int AXIS, bool ITER>
+cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
+  const size_t smem = plan_smem<TI, N>(P);
+  // The shared-memory opt-in is made once per device and instantiation, for the most any launch may
+  // need, so later calls issue nothing but the launch (a stream under capture sees kernel nodes only).
+  static std::atomic<bool> opted[64];
+  int dev = 0;
+  cfd_status s = cuda_fail(cudaGetDevice(&dev), "cudaGetDevice");
+  if (s != CFD_OK) return s;
+  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER>;
+  if (dev < 0 || dev >= 64 || !opted[dev].load()) {
+    s = cuda_fail(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax),
+                  "cudaFuncSetAttribute");
+    if (s != CFD_OK) return s;
+    if (dev >= 0 && dev < 64) opted[dev].store(true);
+  }
+  if (smem > kSmemMax) { set_error("dense: shared memory plan too large"); return CFD_ERR_UNSUPPORTED; }
+  launch_begin(KF_DENSE, st);
+  fn<<<grid, kXThreads, smem, st>>>(P);
+  launch_end(KF_DENSE, st);
+  return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
+}
+
+// Ghost width 4 has the axis compiled in; other widths share one instantiation per type.
+template <typename TI, typename TO, int N>
+cfd_status launch_exact_types(const DenseParams &P, unsigned grid, cudaStream_t st) {
+  const bool it = P.halo_in != nullptr;
+  if (P.g == 4) {
+    if (P.axis == 2) return it ? launch_one<TI, TO, N, 2, true>(P, grid, st) : launch_one<TI, TO, N, 2, false>(P, grid, st);
+    if (P.axis == 1) return it ? launch_one<TI, TO, N, 1, true>(P, grid, st) : launch_one<TI, TO, N, 1, false>(P, grid, st);
+    return it ? launch_one<TI, TO, N, 0, true>(P, grid, st) : launch_one<TI, TO, N, 0, false>(P, grid, st);
+  }
+  return it ? launch_one<TI, TO, N, 3, true>(P, grid, st) : launch_one<TI, TO, N, 3, false>(P, grid, st);
+}
+
+template <int N>
+cfd_status launch_exact(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st) {
+  if (f32_in) return launch_exact_types<float, float, N>(P, grid, st);
+  if (f32_out) return launch_exact_types<double, float, N>(P, grid, st);
+  return launch_exact_types<double, double, N>(P, grid, st);
+}
+
+}  // namespace
+}  // namespace cfd

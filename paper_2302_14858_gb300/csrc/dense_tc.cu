@@ -7,26 +7,18 @@
 //     out[p, i] = sum_j f[p, j] D[i, j]      (p: pencil, j: ghost-extended index)
 // run as a GEMM with M = 128 pencils per tile, N = output rows, K = N + 2g.
 //
-// Precision ("exact integer slices").  D row i is scaled by a power of two
-// sigma_i >= max_j |D_ij| and written as 5 signed 8-bit digits
-//     D_ij / sigma_i = sum_t b_t 2^{-7-8t},  |b_t| <= 128,
-// each exact in BF16; every pencil p gets a power-of-two scale tau_p and the
-// same 5-digit split a_s of its values (done in the kernel from the IEEE bits).
-// A BF16 x BF16 product of digits is an integer below 2^14, a K <= 48 sum is
-// below 2^20, and the pairs (s, t) of one level k = s + t (at most 5 of them)
-// are accumulated in the same FP32 TMEM columns, staying below 2^22: every
-// accumulator is an exact integer.  Levels k <= L are kept; the epilogue forms
-// Y = sum_k acc_k 2^{8(L-k)} as a 64-bit integer and writes
-//     out = Y * 2^{e(sigma_i) + e(tau_p) - 14 - 8L}
-// by assembling the IEEE bits with integer instructions (no FP64 arithmetic).
-// (S, L) = (5, 4) keeps 15 slice pairs: the error is below ~2^-37 of
-// sum_j |D_ij f_j|, i.e. FP64-level for these operators.  (S, L) = (2, 1) is
-// the 3-product hi/lo split.
-//
-// Kernel structure: a persistent, warp-specialised CTA per SM (producers stage
-// and split the pencils of a tile, one thread issues tcgen05.mma, epilogue warps
-// read TMEM and rebuild the outputs), described at k_dense below.  The halo
-// passes of the hybrid iteration run on the CUDA cores (halo_rows.cu).
+// Three arithmetic forms share the planning in this file:
+//   - CFD_TC_BF16_EXACT: exact integer digit slices in FP16 (FP64-level results), the kernel of
+//     dense_exact.cuh;
+//   - CFD_TC_BF16X3: the hi/lo split, two balanced 8-bit digits per factor in BF16 (S = 2), the
+//     levels k = s + t <= 1 (L = 1, 3 products) as exact integers in FP32 accumulators;
+//   - CFD_TC_TF32: one TF32 product (S = 1, L = 0).
+// The last two run in k_dense below, a persistent, warp-specialised CTA per SM (producers stage and
+// split the pencils of a tile, one thread issues tcgen05.mma, epilogue warps read TMEM and rebuild the
+// outputs).  In both digit forms row i of D is scaled by a power of two sigma_i, every pencil p by a
+// power of two tau_p (taken from its values in the kernel), and the epilogue writes the integer sum
+// times 2^{e(sigma_i) + e(tau_p) - const} by assembling the IEEE bits.  The halo passes of the hybrid
+// iteration run on the CUDA cores (halo_rows.cu).
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -37,16 +29,13 @@
 #include <string>
 #include <vector>
 
-#include "dense.h"
+#include "dense_dev.cuh"
 
 namespace cfd {
 
 namespace {
 
-constexpr int kS = 5;              // digit slices kept for exact mode
-constexpr int kTile = 128;         // pencils per tile (MMA M)
-constexpr int kTmemCols = 512;
-constexpr long long kWaitLimit = 4000000000LL;  // clock cycles (~2 s) before giving up
+constexpr int kS = 2;              // digit slices of the hi/lo split
 
 // ------------------------------------------------------------------ host: wait limit of the main loop
 
@@ -134,7 +123,7 @@ uint16_t bf16_of_small_int(int a) {
   return (uint16_t)(u >> 16);
 }
 
-// Digit image of one operator: kS slices x rows x Kp columns (row-major D of
+// BF16 digit image of one operator (the leading kS of five balanced base-256 digits): kS slices x rows x Kp columns (row-major D of
 // `cols` columns, cols <= Kp, rows a multiple of 8), canonical K-major smem
 // layout per slice: [row/8][k/8][row%8][k%8] bf16.  Row i is scaled by
 // 2^rowexp[i] >= max_j |D_ij|.
@@ -150,8 +139,8 @@ void digit_image(const std::vector<ld> &D, int rows, int cols, int Kp, std::vect
     rowexp[i] = e;
     for (int j = 0; j < cols; ++j) {
       long long F = llrintl(ldexpl(D[(size_t)i * cols + j], 39 - e));  // |F| <= 2^39
-      int dig[kS];
-      for (int t = kS - 1; t >= 1; --t) {
+      int dig[5];
+      for (int t = 4; t >= 1; --t) {
         long long r = F & 0xFF;
         if (r >= 128) r -= 256;
         dig[t] = (int)r;
@@ -161,6 +150,50 @@ void digit_image(const std::vector<ld> &D, int rows, int cols, int Kp, std::vect
       for (int t = 0; t < kS; ++t) {
         const size_t off = (size_t)t * rows * Kp + ((size_t)(i / 8) * (Kp / 8) + j / 8) * 64 + (i % 8) * 8 + (j % 8);
         img[off] = bf16_of_small_int(dig[t]);
+      }
+    }
+  }
+}
+
+uint16_t fp16_of_small_int(int a) {  // |a| <= 2048: exact
+  if (a == 0) return 0;
+  int m = a < 0 ? -a : a, e = 0;
+  while ((m >> e) > 1) ++e;
+  return (uint16_t)((a < 0 ? 0x8000 : 0) | ((e + 15) << 10) | (((m << 10) >> e) & 0x3FF));
+}
+
+// FP16 digit image of the exact form (dense_exact.cuh): four balanced base-1024 digits of
+// D_ij / 2^rowexp[i] in 39-bit fixed point, laid out as above.  2^rowexp[i] >= max_j |D_ij|, and at
+// least sum_j |D_ij| / 7.8: with pencil digits up to 512 the level-0 sums then stay below
+// 512 x (512 x 7.8 + 24) < 2^21 - 2^14, so that x_0 2^10 + x_1 fits in 32 bits.  (A row with a sum
+// above 7.8 times its maximum keeps its accuracy relative to sum_j |D_ij|.)
+void exact_image(const std::vector<ld> &D, int rows, int cols, int Kp, std::vector<uint16_t> &img,
+                 std::vector<int> &rowexp) {
+  img.assign((size_t)4 * rows * Kp, 0);
+  rowexp.assign(rows, 0);
+  for (int i = 0; i < rows; ++i) {
+    ld mx = 0, sum = 0;
+    for (int j = 0; j < cols; ++j) {
+      mx = std::max(mx, fabsl(D[(size_t)i * cols + j]));
+      sum += fabsl(D[(size_t)i * cols + j]);
+    }
+    int e = 0;
+    if (mx > 0) frexpl(mx, &e);  // mx < 2^e
+    while (ldexpl(sum, -e) > 7.8L) ++e;
+    rowexp[i] = e;
+    for (int j = 0; j < cols; ++j) {
+      long long F = llrintl(ldexpl(D[(size_t)i * cols + j], 39 - e));  // |F| <= 2^39
+      int dig[4];
+      for (int t = 3; t >= 1; --t) {
+        long long r = F & 1023;
+        if (r >= 512) r -= 1024;
+        dig[t] = (int)r;
+        F = (F - r) >> 10;
+      }
+      dig[0] = (int)F;
+      for (int t = 0; t < 4; ++t) {
+        const size_t off = (size_t)t * rows * Kp + ((size_t)(i / 8) * (Kp / 8) + j / 8) * 64 + (i % 8) * 8 + (j % 8);
+        img[off] = fp16_of_small_int(dig[t]);
       }
     }
   }
@@ -235,20 +268,6 @@ void iterated_operator(const SchemeCoef &s, int N, int g, std::vector<ld> &D1, s
 
 // ------------------------------------------------------------------ device helpers
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-         ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-      "l"(da), "l"(db), "r"(idesc), "r"(acc));
-}
-
 __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -268,23 +287,7 @@ __device__ __forceinline__ uint32_t small_int_f32bits(int a) {
 // multiply-adds.
 constexpr uint32_t kAccBiasBits = 0x4B400000u;
 constexpr float kAccBias = 12582912.0f;
-constexpr int kBadTau = 1 << 20;  // pencil scale of a pencil holding a NaN or an infinity
 
-// Y * 2^E as an IEEE double (|Y| < 2^55).  The 64-bit conversion runs on the FP64 pipe,
-// which nothing else in this kernel uses; the power-of-two scale is an add to the exponent
-// field.  `checked`: results below the normal range flush to a signed zero, results above
-// it become infinities, and `bad` gives a NaN; without it the caller has established that
-// the exponent stays in range for every Y.
-template <bool checked>
-__device__ __forceinline__ double scaled_double(double d, int E, bool bad) {
-  const int hi = __double2hiint(d), lo = __double2loint(d);
-  if (!checked) return d == 0.0 ? 0.0 : __hiloint2double(hi + (E << 20), lo);
-  const int fe = (hi >> 20) & 0x7FF;  // 0 only for d = 0 here (d is an integer or an FP32 value)
-  if (bad) return __longlong_as_double(0x7FF8000000000000ll);
-  if (fe == 0 || fe + E <= 0) return __hiloint2double(hi & (int)0x80000000, 0);
-  if (fe + E >= 2047) return __hiloint2double((hi & (int)0x80000000) | 0x7FF00000, 0);
-  return __hiloint2double(hi + (E << 20), lo);
-}
 template <bool checked>
 __device__ __forceinline__ double scaled_int_to_double(long long Y, int E, bool bad) {
   return scaled_double<checked>(__ll2double_rn(Y), E, bad);
@@ -310,14 +313,6 @@ __device__ __forceinline__ uint32_t tf32_of(float v, int emax) {
   const int e = (int)((u >> 23) & 0xFF);
   if (e == 0 || e + 60 < emax) return 0u;
   return cvt_rna_tf32(__uint_as_float(u - ((uint32_t)(emax - 126) << 23)));
-}
-
-// y * 2^E in FP32 for |E| <= 300: two exact power-of-two factors (each a normal float),
-// so the only rounding is that of the final product (under- and overflow as IEEE).
-__device__ __forceinline__ float scale_pow2(float y, int E) {
-  E = max(-300, min(300, E));
-  const int e1 = E / 2, e2 = E - e1;
-  return y * __int_as_float((e1 + 127) << 23) * __int_as_float((e2 + 127) << 23);
 }
 
 // Signed fixed-point value F = round(v / tau * 2^39), |F| <= 2^39, of one input element;
@@ -362,45 +357,6 @@ __device__ __forceinline__ void digits_of(long long F, uint32_t (&out)[S]) {
     const uint32_t sel = 0x5440u | (uint32_t)(4 - t);  // byte 4-t of lo, then 0x00 0x00 0x4B
     out[t] = __float_as_uint(__uint_as_float(__byte_perm(lo, 0x4B00u, sel)) - 8388736.0f);
   }
-}
-
-__device__ __forceinline__ int biased_exp(double v) {
-  return (int)((((unsigned long long)__double_as_longlong(v)) >> 52) & 0x7FF);
-}
-__device__ __forceinline__ int biased_exp(float v) { return (int)((__float_as_uint(v) >> 23) & 0xFF); }
-__device__ __forceinline__ int tau_exp(int emax, double) { return emax - 1022; }
-__device__ __forceinline__ int tau_exp(int emax, float) { return emax - 126; }
-__device__ __forceinline__ int nonfinite_exp(double) { return 0x7FF; }
-__device__ __forceinline__ int nonfinite_exp(float) { return 0xFF; }
-
-// Wait for the phase `parity` of an mbarrier for at most `limit` clock cycles.  The main loop
-// uses the launch's limit (DenseParams::wait_limit); the exit path, which drains the CTA's own
-// copies and MMAs before it frees TMEM, always uses kWaitLimit.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar_addr, uint32_t parity, long long limit = kWaitLimit) {
-  const long long t0 = clock64();
-  uint32_t done = 0;
-  while (!done) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(mbar_addr), "r"(parity));
-    if (!done && clock64() - t0 > limit) return false;
-  }
-  return true;
-}
-
-__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src));
-}
-__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src));
-}
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src));
-}
-
-__device__ __forceinline__ long long stride_of(int axis, long long s0, long long s1) {
-  return axis == 0 ? s0 : (axis == 1 ? s1 : 1ll);
 }
 
 // ------------------------------------------------------------------ the kernel
@@ -474,19 +430,12 @@ __device__ __forceinline__ void epilogue_rows(uint32_t taddr, uint32_t lev_strid
     for (int u = 0; u < V; ++u) {
       const int c = c0 + u;
       const int ex = rowexp[c] + ebase;
-      // Y = sum_k a_k 2^(8 (LEV-1-k)), a_k = acc_k - kAccBiasBits (exact integers; the
-      // 32-bit partial sums are exact modulo 2^32 and their true values fit)
+      // Y = sum_k a_k 2^(8 (LEV-1-k)), a_k = acc_k - kAccBiasBits (exact integers)
       auto exact_y = [&]() -> long long {
-        if constexpr (LEV == 5) {
-          const int t1 = (int)(acc[0][c] * 256u + acc[1][c] - 257u * kAccBiasBits);
-          const int t2 = (int)(acc[2][c] * 256u + acc[3][c] - 257u * kAccBiasBits);
-          return (long long)t1 * 16777216ll + (long long)t2 * 256ll + (long long)(int)(acc[4][c] - kAccBiasBits);
-        } else {
-          long long Y = 0;
+        long long Y = 0;
 #pragma unroll
-          for (int k = 0; k < LEV; ++k) Y = Y * 256ll + (long long)(int)(acc[k][c] - kAccBiasBits);
-          return Y;
-        }
+        for (int k = 0; k < LEV; ++k) Y = Y * 256ll + (long long)(int)(acc[k][c] - kAccBiasBits);
+        return Y;
       };
       TO val;
       double dv = 0.0;  // the FP64 value the intermediates keep
@@ -577,16 +526,9 @@ __device__ __forceinline__ void epilogue_fast8(uint32_t taddr, uint32_t lev_stri
     } else if (sizeof(TO) == 8 || SC) {
       // Y = sum_k a_k 2^(8 (LEV-1-k)) as a 64-bit integer, one conversion, the scale as an
       // exponent-field add (Y = 0 gives 0)
-      long long Y;
-      if constexpr (LEV == 5) {
-        const int t1 = (int)(acc[0][c] * 256u + acc[1][c] - 257u * kAccBiasBits);
-        const int t2 = (int)(acc[2][c] * 256u + acc[3][c] - 257u * kAccBiasBits);
-        Y = (long long)t1 * 16777216ll + (long long)t2 * 256ll + (long long)(int)(acc[4][c] - kAccBiasBits);
-      } else {
-        Y = 0;
+      long long Y = 0;
 #pragma unroll
-        for (int k = 0; k < LEV; ++k) Y = Y * 256ll + (long long)(int)(acc[k][c] - kAccBiasBits);
-      }
+      for (int k = 0; k < LEV; ++k) Y = Y * 256ll + (long long)(int)(acc[k][c] - kAccBiasBits);
       const double d = __ll2double_rn(Y);
       const int hi = __double2hiint(d), lo = __double2loint(d);
       dv = __hiloint2double(hi ? hi + (ex << 20) : 0, lo);
@@ -623,12 +565,6 @@ __device__ __forceinline__ void epilogue_fast8(uint32_t taddr, uint32_t lev_stri
   }
 }
 
-__device__ __forceinline__ void mbar_init(uint32_t addr, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(addr), "r"(count));
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t addr) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(addr));
-}
 __device__ __forceinline__ void producer_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kProducers)); }
 
 // Barrier of the 256 producer threads that also ORs a flag over them.
@@ -641,58 +577,6 @@ __device__ __forceinline__ bool producer_any(bool v) {
   return r != 0;
 }
 
-struct TileCoord {
-  int lb, q, b, t1, t2;
-  bool valid;
-};
-
-// The tiles of this CTA: interleaved (tile = CTA + k * grid) or a contiguous run of
-// tiles_per_cta (tile_order 1; neighbouring tiles share input rows in L2).
-struct TileRange {
-  int first, end, step;
-};
-__device__ __forceinline__ TileRange tile_range(const DenseParams &P) {
-  TileRange r;
-  if (P.tile_order) {
-    r.first = blockIdx.x * P.tiles_per_cta;
-    r.end = min(P.ntiles, r.first + P.tiles_per_cta);
-    r.step = 1;
-  } else {
-    r.first = blockIdx.x;
-    r.end = P.ntiles;
-    r.step = gridDim.x;
-  }
-  return r;
-}
-
-__device__ __forceinline__ int dir_index_dev(int dz, int dy, int dx) {
-  const int r = 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1);
-  return r > 13 ? r - 1 : r;
-}
-
-// pencil index p (within the block and field) of pencil `pencil` of a tile
-// n / d for 0 <= n < 2^22 with inv = 1/d rounded to FP32: (n + 1/2) / d stays at least 1/(2d)
-// away from an integer, more than the two roundings can move it
-__device__ __forceinline__ int fdiv(int n, float inv) { return __float2int_rz(((float)n + 0.5f) * inv); }
-
-__device__ __forceinline__ int tile_pencil(const DenseParams &P, int tile, int pencil) {
-  const int job = fdiv(tile, P.inv_tpj), tj = tile - job * P.tiles_per_job;
-  return tj * kTile + pencil;
-}
-
-__device__ __forceinline__ TileCoord tile_coord(const DenseParams &P, int tile, int pencil) {
-  TileCoord c;
-  const int job = fdiv(tile, P.inv_tpj), tj = tile - job * P.tiles_per_job;
-  c.lb = fdiv(job, P.inv_nf);
-  c.q = job - c.lb * P.nf;
-  c.b = P.contig ? P.b0 + c.lb : P.blocks[c.lb];
-  const int p = tj * kTile + pencil;
-  c.valid = p < P.n1 * P.n2;
-  c.t1 = c.valid ? fdiv(p, P.inv_n2) : 0;
-  c.t2 = c.valid ? p - c.t1 * P.n2 : 0;
-  return c;
-}
-
 // TFM = 1: the one-product TF32 form (S = 1, L = 0): A = the pencils scaled by tau and rounded
 // to TF32, B = the TF32 image of D, one kind::tf32 MMA chain per pass, FP32 accumulators.
 //
@@ -700,11 +584,7 @@ __device__ __forceinline__ TileCoord tile_coord(const DenseParams &P, int tile, 
 // neighbours' previous iterate as 4 extra columns.  A separate instantiation keeps that code out
 // of the closed passes' producer loop (measured 5 % slower with it there).
 //
-// SPL = 1: a closed pass whose pencils fill an odd number of 8-value K chunks (E = N + 8 for
-// N = 16, 32), the last chunk all padding.  The two producer threads of a pencil then split
-// the last real chunk four values each instead of one of them taking it whole, so both do the
-// same digit work.
-template <typename TI, typename TO, int KP, int S, int L, int TFM, bool ITER, bool SPL>
+template <typename TI, typename TO, int KP, int S, int L, int TFM, bool ITER>
 __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ DenseParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr int EB = TFM ? 4 : 2;  // bytes per operand element (TF32 or BF16)
@@ -800,7 +680,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ D
     // kParts threads per pencil; part `half` splits K chunks half, half + kParts, ...
     const int pl = (warp & 3) * 32 + lane, half = warp >> 2;
     constexpr int CPP = (NCH + kParts - 1) / kParts;  // K chunks per producer thread
-    static_assert(!SPL || (!TFM && !ITER && kParts == 2 && NCH % 2 == 0), "split last chunk: two threads per pencil");
     const float inv_n2 = 1.0f / (float)P.n2;
     const int cpr = E / VE;  // 16-byte chunks per pencil row (x axis); E * sizeof(TI) is a multiple of 16
     const float inv_cpr = 1.0f / (float)cpr;
@@ -940,11 +819,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ D
       const int kv = c.valid ? P.kext : 0;  // values of this pencil (none for a pencil past the end)
 #pragma unroll
       for (int h = 0; h < CPP; ++h) {
-        // the last slot of a split pass: values 4 half .. 4 half + 3 of chunk NCH - 2
-        const bool sl = SPL && h == CPP - 1;
 #pragma unroll
-        for (int k = 0; k < (sl ? 4 : 8); ++k) {
-          const int j = sl ? (NCH - 2) * 8 + 4 * half + k : (half + kParts * h) * 8 + k;
+        for (int k = 0; k < 8; ++k) {
+          const int j = (half + kParts * h) * 8 + k;
           v[h][k] = j < kv ? stg[stg_index(j)] : TI(0);
           em = max(em, biased_exp(v[h][k]));
         }
@@ -988,26 +865,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ D
       } else {
 #pragma unroll
       for (int h = 0; h < CPP; ++h) {
-        if (SPL && h == CPP - 1) {
-          // half of chunk NCH - 2 (8-byte digit stores); the second thread also writes the
-          // zero digits of the padding chunk NCH - 1
-          uint32_t w2[S][2];
-#pragma unroll
-          for (int k = 0; k < 4; k += 2) {
-            uint32_t d0[S], d1[S];
-            digits_of<S>(fixed_of(v[h][k], emax), d0);
-            digits_of<S>(fixed_of(v[h][k + 1], emax), d1);
-#pragma unroll
-            for (int t = 0; t < S; ++t) w2[t][k / 2] = __byte_perm(d0[t], d1[t], 0x7632);
-          }
-#pragma unroll
-          for (int t = 0; t < S; ++t) {
-            uint16_t *row = Ab + (size_t)t * kTile * KP + (size_t)row_group * NCH * 64 + row_in * 8;
-            *reinterpret_cast<uint2 *>(row + (NCH - 2) * 64 + 4 * half) = make_uint2(w2[t][0], w2[t][1]);
-            if (half) *reinterpret_cast<uint4 *>(row + (NCH - 1) * 64) = make_uint4(0u, 0u, 0u, 0u);
-          }
-          continue;
-        }
         const int ch = half + kParts * h;
         if (ch >= NCH) break;
         uint32_t w[S][4];
@@ -1063,7 +920,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ D
             // every level column of the pass buffer starts at kAccBias (1 x kAccBias, K = 16)
             const uint32_t idesc_b = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(((L + 1) * R) >> 3) << 17) |
                                      ((uint32_t)(kTile >> 4) << 24);
-            mma_bf16(cbase, smem_desc(smem_u32(sOne), 128, 256), smem_desc(smem_u32(sBias), 128, 256), idesc_b, 0u);
+            mma_16bit(cbase, smem_desc(smem_u32(sOne), 128, 256), smem_desc(smem_u32(sBias), 128, 256), idesc_b, 0u);
           }
 #pragma unroll
           for (int s = 0; s < S; ++s) {
@@ -1075,7 +932,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_dense(const __grid_constant__ D
             for (int kk = 0; kk < KP / 16; ++kk) {
               const uint64_t da = smem_desc(a0 + (uint32_t)(s * kTile * KP * 2 + kk * 256), lbo, sbo);
               const uint64_t db = smem_desc(b0 + (uint32_t)(kk * 256), lbo, sbo);
-              mma_bf16(cbase + (uint32_t)(s * R), da, db, idesc_s, 1u);
+              mma_16bit(cbase + (uint32_t)(s * R), da, db, idesc_s, 1u);
             }
           }
           }
@@ -1240,21 +1097,14 @@ template <typename TI, typename TO, int KP>
 cfd_status launch_kp(const DenseParams &P, int S, int L, size_t smem, unsigned grid, cudaStream_t st) {
   void (*fn)(const __grid_constant__ DenseParams);
   const bool it = P.halo_in != nullptr;
-  // the exact slices' closed passes whose last K chunk is all padding split the last real one,
-  // except in the stages that also write an intermediate (measured 1-3 % slower there, 3 %
-  // faster in the others)
-  const bool spl = !it && P.scratch_out == nullptr && P.kext > KP - 16 && P.kext <= KP - 8;
-  if (S == 5 && L == 4)
-    fn = it ? k_dense<TI, TO, KP, 5, 4, 0, true, false>
-            : (spl ? k_dense<TI, TO, KP, 5, 4, 0, false, true> : k_dense<TI, TO, KP, 5, 4, 0, false, false>);
-  else if (S == 2 && L == 1) fn = it ? k_dense<TI, TO, KP, 2, 1, 0, true, false> : k_dense<TI, TO, KP, 2, 1, 0, false, false>;
-  else if (S == 1 && L == 0) fn = it ? k_dense<TI, TO, KP, 1, 0, 1, true, false> : k_dense<TI, TO, KP, 1, 0, 1, false, false>;
+  if (S == 2 && L == 1) fn = it ? k_dense<TI, TO, KP, 2, 1, 0, true> : k_dense<TI, TO, KP, 2, 1, 0, false>;
+  else if (S == 1 && L == 0) fn = it ? k_dense<TI, TO, KP, 1, 0, 1, true> : k_dense<TI, TO, KP, 1, 0, 1, false>;
   else { set_error("dense: unsupported slice configuration"); return CFD_ERR_UNSUPPORTED; }
   // The shared-memory opt-in is set once per device and instantiation (and raised when a
   // launch needs more), so that later calls issue nothing but the launch: a stream being
   // captured into a CUDA graph sees only kernel nodes.
-  static size_t opted[7][64] = {};  // [slice configuration, iterated or split][device]
-  const int v = (S == 5 ? 0 : (S == 2 ? 1 : 2)) + (it ? 3 : 0) + (S == 5 && spl ? 6 : 0);
+  static size_t opted[4][64] = {};  // [slice configuration, iterated][device]
+  const int v = (S == 2 ? 0 : 1) + (it ? 2 : 0);
   int dev = 0;
   cfd_status s = cuda_fail(cudaGetDevice(&dev), "cudaGetDevice");
   if (s != CFD_OK) return s;
@@ -1287,10 +1137,15 @@ cfd_status launch_types(const DenseParams &P, int KP, int S, int L, size_t smem,
 // ------------------------------------------------------------------ host planning
 
 struct DenseOp {        // one (group, axis, degree) operator
-  uint16_t *img = nullptr;    // device: kS x N x Kp digits
+  uint16_t *img = nullptr;    // device: kS x N x Kp BF16 digits (hi/lo split)
+  uint16_t *imgx = nullptr;   // device: 4 x N x Kp FP16 digits (the exact form)
   uint32_t *img32 = nullptr;  // device: N x Kp TF32 values (the one-product TF32 form)
-  int *rowexp = nullptr;      // device: N
-  const void *image(bool tf32) const { return tf32 ? (const void *)img32 : (const void *)img; }
+  int *rowexp = nullptr;      // device: N row exponents of img and img32
+  int *rowexpx = nullptr;     // device: N row exponents of imgx
+  const void *image(cfd_precision p) const {
+    return p == CFD_TC_TF32 ? (const void *)img32 : (p == CFD_TC_BF16X3 ? (const void *)img : (const void *)imgx);
+  }
+  const int *exps(cfd_precision p) const { return p == CFD_TC_BF16_EXACT ? rowexpx : rowexp; }
 };
 
 struct DenseGroup {
@@ -1339,22 +1194,31 @@ DenseState *state_of(cfd_blocks_s *B) { return reinterpret_cast<DenseState *>(B-
 }  // namespace
 
 static cfd_status upload_op(cfd_blocks_s *B, const std::vector<ld> &D, int rows, int cols, int Kp, DenseOp &o) {
-  std::vector<uint16_t> img;
+  std::vector<uint16_t> img, imgx;
   std::vector<uint32_t> img32;
-  std::vector<int> rexp;
+  std::vector<int> rexp, rexpx;
   digit_image(D, rows, cols, Kp, img, rexp);
+  exact_image(D, rows, cols, Kp, imgx, rexpx);
   tf32_image(D, rows, cols, Kp, img32);
-  cfd_status s = cuda_fail(cudaMalloc((void **)&o.img, img.size() * 2), "cudaMalloc");
-  if (s == CFD_OK) s = cuda_fail(cudaMemcpy(o.img, img.data(), img.size() * 2, cudaMemcpyHostToDevice), "cudaMemcpy");
-  if (s == CFD_OK) s = cuda_fail(cudaMalloc((void **)&o.img32, img32.size() * 4), "cudaMalloc");
-  if (s == CFD_OK)
-    s = cuda_fail(cudaMemcpy(o.img32, img32.data(), img32.size() * 4, cudaMemcpyHostToDevice), "cudaMemcpy");
-  if (o.img32) B->d_dense_ptrs.push_back(o.img32);
-  if (s == CFD_OK) s = cuda_fail(cudaMalloc((void **)&o.rowexp, rexp.size() * 4), "cudaMalloc");
-  if (s == CFD_OK) s = cuda_fail(cudaMemcpy(o.rowexp, rexp.data(), rexp.size() * 4, cudaMemcpyHostToDevice), "cudaMemcpy");
-  if (o.img) B->d_dense_ptrs.push_back(o.img);
-  if (o.rowexp) B->d_dense_ptrs.push_back(o.rowexp);
-  return s;
+  // one device allocation and one copy per operator: binding a mesh makes a few dozen of these
+  std::vector<unsigned char> all;
+  auto add = [&](const auto &v) {
+    const size_t at = (all.size() + 15) & ~(size_t)15;
+    all.resize(at + v.size() * sizeof(v[0]));
+    memcpy(all.data() + at, v.data(), v.size() * sizeof(v[0]));
+    return at;
+  };
+  const size_t a0 = add(img), a1 = add(imgx), a2 = add(img32), a3 = add(rexp), a4 = add(rexpx);
+  unsigned char *d = nullptr;
+  cfd_status s = cuda_fail(cudaMalloc((void **)&d, all.size()), "cudaMalloc");
+  if (s != CFD_OK) return s;
+  B->d_dense_ptrs.push_back(d);
+  o.img = reinterpret_cast<uint16_t *>(d + a0);
+  o.imgx = reinterpret_cast<uint16_t *>(d + a1);
+  o.img32 = reinterpret_cast<uint32_t *>(d + a2);
+  o.rowexp = reinterpret_cast<int *>(d + a3);
+  o.rowexpx = reinterpret_cast<int *>(d + a4);
+  return cuda_fail(cudaMemcpy(d, all.data(), all.size(), cudaMemcpyHostToDevice), "cudaMemcpy");
 }
 
 cfd_status dense_bind(cfd_blocks_s *B) {
@@ -1512,15 +1376,17 @@ cfd_status dense_bind(cfd_blocks_s *B) {
 
 namespace {
 
-// Digit slices S of the inputs and the highest level L kept: exact mode five slices and levels
-// 0..4 (15 slice pairs), for FP32 fields too -- four slices and levels 0..3 measured ~1e-6 on
-// second derivatives at fine spacing (the truncated fifth operator digit acts coherently on
-// smooth data), ten times the FP32 rounding of the outputs.
-int slices_of(cfd_precision p, int) { return p == CFD_TC_BF16_EXACT ? 5 : (p == CFD_TC_TF32 ? 1 : 2); }
-int levels_of(cfd_precision p, int) { return p == CFD_TC_BF16_EXACT ? 4 : (p == CFD_TC_TF32 ? 0 : 1); }
+// Digit slices S of the inputs and the highest level L kept (the exact form has its own kernel:
+// four digits, levels 0..3).  FP32 fields take all four digits too: with fewer, second derivatives at
+// fine spacing lose up to 1e-6 (a truncated operator digit acts coherently on smooth data), ten times
+// the FP32 rounding of the outputs.
+int slices_of(cfd_precision p) { return p == CFD_TC_BF16_EXACT ? 4 : (p == CFD_TC_TF32 ? 1 : 2); }
+int levels_of(cfd_precision p) { return p == CFD_TC_BF16_EXACT ? 3 : (p == CFD_TC_TF32 ? 0 : 1); }
+// operator rows of one MMA pass: the exact form's TMEM buffers hold both degrees (64 rows x 4 levels)
+int pass_rows(cfd_precision p) { return p == CFD_TC_BF16_EXACT ? 64 : 32; }
 bool tc_precision(cfd_precision p) { return p == CFD_TC_BF16_EXACT || p == CFD_TC_BF16X3 || p == CFD_TC_TF32; }
 
-// Shared memory per CTA: two A digit buffers, B digits of two passes, the
+// Shared memory of k_dense per CTA: two A digit buffers, B digits of two passes, the
 // input staging tile, row exponents, exponent exchange, etau ring, barriers.  At least 116 KB so that
 // one CTA (holding all 512 TMEM columns) occupies an SM.
 size_t dense_smem(int KP, int S, int rows, size_t elem, int tma_boxes) {
@@ -1554,12 +1420,14 @@ EncodeTiledFn tensor_map_encoder() {
 // TMA staging for a stage whose 128-pencil tiles are boxes of the input: pencils along x
 // (x rows, 128-byte swizzled boxes) or along y / z (one box of the whole columns).  Falls
 // back to the cp.async path (tma_kind 0) when a box or alignment rule does not hold.
-void plan_tma(DenseParams &P, size_t elem) {
+void plan_tma(DenseParams &P, size_t elem, bool exact) {
   P.tma_kind = 0;
   P.tma_boxes = 0;
-  // An iterated pass (halo_in) takes kext = E + 4 values per pencil: the boxes cover kext along
-  // the pencil axis, and the producers write the 4 halo columns into the staged tile.
-  const int n2 = P.n2, E = P.N + 2 * P.g, K = P.kext;
+  // An iterated pass (halo_in) of k_dense takes kext = E + 4 values per pencil: the boxes cover kext
+  // along the pencil axis, and the producers write the 4 halo columns into the staged tile.  (The
+  // exact form's producers take the halo columns in registers, and its layouts need n2 = N.)
+  const int n2 = P.n2, E = P.N + 2 * P.g, K = exact ? E : P.kext;
+  if (exact && n2 != P.N) return;
   if ((n2 != 16 && n2 != 32) || (P.n1 * n2) % kTile != 0) return;
   if (P.in_field && !P.contig) return;
   const int d0 = P.in_dims[0], d1 = P.in_dims[1], d2 = P.in_dims[2];
@@ -1576,12 +1444,12 @@ void plan_tma(DenseParams &P, size_t elem) {
   cuuint32_t box[3];
   int kind, boxes;
   CUtensorMapSwizzle swz = CU_TENSOR_MAP_SWIZZLE_NONE;
-  const int xb = (int)(128 / elem);
+  const int xb = (int)((exact ? 64 : 128) / elem);  // the exact form stages x rows in 64-byte boxes
   if (P.axis == 2) {  // t1 = z, t2 = y
     kind = 1;
     boxes = (K + xb - 1) / xb;
     box[0] = (cuuint32_t)xb; box[1] = (cuuint32_t)n2; box[2] = (cuuint32_t)(kTile / n2);
-    swz = CU_TENSOR_MAP_SWIZZLE_128B;
+    swz = exact ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
   } else if (P.axis == 1) {  // t1 = z, t2 = x
     kind = 2;
     boxes = 1;
@@ -1601,13 +1469,43 @@ void plan_tma(DenseParams &P, size_t elem) {
   P.tma_zstep = d0;
 }
 
+// The exact form's x stages write their outputs by TMA (boxes of 8 values x 32 pencils) where the
+// tile's pencils are consecutive rows of an output aligned to 16 bytes.
+void plan_out_tma(DenseParams &P, size_t elem) {
+  P.out_box_bytes = 0;
+  if (P.axis != 2 || !P.tma_kind || !P.contig || !P.xvec) return;
+  if (P.n1 != P.N || P.n2 != P.N || P.int_lo1 != 0 || P.int_lo2 != 0 || P.int_hi1 != P.N || P.int_hi2 != P.N) return;
+  const unsigned long long rows = (unsigned long long)P.nblk * P.nf * P.nops * P.N * P.N;
+  if (rows >= (1ull << 31)) return;
+  EncodeTiledFn enc = tensor_map_encoder();
+  if (!enc) return;
+  char *base = static_cast<char *>(P.out) + (size_t)P.nf * P.nops * P.int0 * elem;
+  const cuuint64_t gdim[2] = {(cuuint64_t)P.N, (cuuint64_t)rows}, gstr[1] = {(cuuint64_t)P.N * elem};
+  const cuuint32_t box[2] = {8, 32}, estr[2] = {1, 1};
+  if (enc(&P.tmap_out, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, gdim,
+          gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+          elem == 8 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return;
+  P.out_box_bytes = (int)(8 * 32 * elem);
+}
+
 // Launch one stage with the choices the autotuner made for it (TMA staging and interleaved
 // tiles by default); during cfd_autotune, launch every candidate three times, time the last two
 // with events on the stream, and keep the fastest.  Repeated launches of a stage are idempotent
 // (a stage never reads what it writes), and every candidate computes the same outputs.
 cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int L, size_t ein, bool f32,
                         unsigned grid, cudaStream_t st) {
-  auto launch = [&](const DenseParams &Q) -> cfd_status {
+  const bool exact = S == 4;
+  auto launch = [&](DenseParams Q) -> cfd_status {
+    if (exact) {
+      Q.wait_limit = dense_wait_limit();
+      Q.inv_tpj = 1.0f / (float)Q.tiles_per_job;
+      Q.inv_nf = 1.0f / (float)Q.nf;
+      Q.inv_n2 = 1.0f / (float)Q.n2;
+      return Q.N == 32 ? dense_exact_launch32(Q, Q.in_field && f32, f32, grid, st)
+                       : dense_exact_launch16(Q, Q.in_field && f32, f32, grid, st);
+    }
     const size_t smem = dense_smem(KP, S, Q.rows, ein, Q.tma_boxes);
     if (!Q.in_field)
       return f32 ? launch_types<double, float>(Q, KP, S, L, smem, grid, st)
@@ -1619,8 +1517,9 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
     DenseParams Q = P;
     Q.tile_order = order;
     Q.tiles_per_cta = (Q.ntiles + (int)grid - 1) / (int)grid;
-    if (staging == 0) plan_tma(Q, ein);
+    if (staging == 0) plan_tma(Q, ein, exact);
     else { Q.tma_kind = 0; Q.tma_boxes = 0; }
+    if (exact) plan_out_tma(Q, f32 ? 4 : 8);
     return Q;
   };
   const int idx = ds->launch++;
@@ -1702,7 +1601,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
   ds->key = "apply nf=" + std::to_string(nf) + " ops=" + std::to_string(mask) + " prec=" + std::to_string((int)prec) +
             " n_iter=" + std::to_string(n_iter);
   ds->launch = 0;
-  const int S = slices_of(prec, B->dtype), L = levels_of(prec, B->dtype);
+  const int S = slices_of(prec), L = levels_of(prec);
   const DensePlanSizes z = dense_sizes(B, nf, mask, n_iter);
   double *gy = (double *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   double *gz = gy + bytes256(z.gy) / 8;
@@ -1777,7 +1676,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
       int deg[2], mode[2], op[2], n = 0;
       if (m1 >= 0) { deg[n] = 1; mode[n] = m1; op[n] = op1; ++n; }
       if (m2 >= 0) { deg[n] = 2; mode[n] = m2; op[n] = op2; ++n; }
-      const int per_pass = (n * N <= 32) ? n : 1;
+      const int per_pass = (n * N <= pass_rows(prec)) ? n : 1;
       P.passes = n / per_pass;
       P.rows = per_pass * N;
       for (int ps = 0; ps < P.passes; ++ps) {
@@ -1785,8 +1684,8 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
         for (int k = 0; k < per_pass; ++k) {
           const int sgi = ps * per_pass + k;
           const DenseOp &o = iterating(box) ? G.opI[box][deg[sgi] - 1] : G.op[box][deg[sgi] - 1];
-          P.seg_img[ps][k] = o.image(prec == CFD_TC_TF32);
-          P.seg_exp[ps][k] = o.rowexp;
+          P.seg_img[ps][k] = o.image(prec);
+          P.seg_exp[ps][k] = o.exps(prec);
           P.seg_mode[ps][k] = mode[sgi];
           P.seg_op[ps][k] = op[sgi];
         }
@@ -1982,7 +1881,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
   ds->launch = 0;
   const size_t need = dense_biased_workspace(B, nf, n_iter, mode == 2);
   if (!work || work_bytes < need) { set_error("biased path: workspace too small (see cfd_biased_workspace)"); return CFD_ERR_ARG; }
-  const int S = slices_of(prec, B->dtype), L = levels_of(prec, B->dtype);
+  const int S = slices_of(prec), L = levels_of(prec);
   const DensePlanSizes z = dense_sizes(B, nf, 0, n_iter);
   char *base_w = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   void *tmp6 = nullptr;
@@ -2062,7 +1961,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       int side[2], op[2], n = 0;
       if (mode == 2) { side[0] = 0; op[0] = 2 * i; side[1] = 1; op[1] = 2 * i + 1; n = 2; }
       else { side[0] = mode; op[0] = i; n = 1; }
-      const int per_pass = (n * N <= 32) ? n : 1;
+      const int per_pass = (n * N <= pass_rows(prec)) ? n : 1;
       P.passes = n / per_pass;
       P.rows = per_pass * N;
       for (int ps = 0; ps < P.passes; ++ps) {
@@ -2070,8 +1969,8 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
         for (int k = 0; k < per_pass; ++k) {
           const int sgi = ps * per_pass + k;
           const DenseOp &o = iter ? G.bopI[box][side[sgi]] : G.bop[box][side[sgi]];
-          P.seg_img[ps][k] = o.image(prec == CFD_TC_TF32);
-          P.seg_exp[ps][k] = o.rowexp;
+          P.seg_img[ps][k] = o.image(prec);
+          P.seg_exp[ps][k] = o.exps(prec);
           P.seg_mode[ps][k] = 0;
           P.seg_op[ps][k] = op[sgi];
         }

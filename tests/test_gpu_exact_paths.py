@@ -1,0 +1,118 @@
+"""The exact tensor-core kernel's dispatch: every form it accepts against the FP64 banded solve.
+
+The kernel has compiled-in addressing for four ghost layers and a general form for other widths, TMA
+staging where a tile is an aligned box of the input and element copies elsewhere, row boxes for the
+x outputs where they are aligned, and one or two operators (16, 32 or 64 rows) per launch.  Tolerances:
+1e-7 of the largest output for FP64 fields (the contract of the exact slices; 2^-37 of sum |D f| times
+the cancellation of the operator) and 2e-6 for FP32 fields (their rounding).
+"""
+import numpy as np
+import pytest
+
+from paper_2302_14858_gb300 import workloads as W
+from tests.helpers import desc, rel_max
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2302_14858_gb300 import build
+    build.build()
+    from paper_2302_14858_gb300 import cfd
+    return cfd
+
+
+def run(lib, B, fields, nf, mask, prec, n_iter, out_offset):
+    import torch
+    nops, nint = bin(mask).count("1"), sum(int(n) ** 3 for n in B.block_n)
+    buf = torch.full((nint * nf * nops + 8,), float("nan"), dtype=fields.dtype, device=fields.device)
+    out = buf[out_offset:out_offset + nint * nf * nops]
+    work = torch.empty(max(lib.cfd_apply_workspace(B, nf, mask, prec, n_iter), 256), dtype=torch.uint8,
+                       device=fields.device)
+    lib.cfd_apply(B, fields, nf, mask, prec, n_iter, out, work)
+    lib.cfd_sync_status(B)
+    return out.cpu().numpy().reshape(len(B.block_n), nf, nops, -1)
+
+
+@pytest.mark.parametrize("nb,N,g,dtype,nf,ops,n_iter,offset", [
+    ((2, 1, 3), 16, 4, "f64", 1, ("dx",), 0, 0),                     # 16 operator rows; a cyclic axis
+    ((2, 1, 3), 16, 4, "f64", 3, ("dx", "dxx", "dyz"), 1, 0),
+    ((3, 2, 2), 16, 4, "f32", 2, ("dx", "dy", "dz", "dxx", "dyy", "dzz", "dxy", "dxz", "dyz"), 2, 0),
+    ((2, 2, 2), 32, 4, "f64", 1, ("dx", "dxy"), 1, 1),               # unaligned buffers: element copies
+    ((2, 2, 1), 32, 4, "f32", 3, ("dxx", "dz", "dxz", "dyz"), 0, 1),
+    ((2, 2, 2), 32, 4, "f32", 1, ("dy", "dyy"), 1, 2),
+    ((2, 2, 2), 16, 5, "f64", 2, ("dx", "dyy", "dzz", "dxy", "dxz", "dyz"), 0, 0),   # other ghost widths
+    ((2, 3, 2), 16, 5, "f32", 1, ("dx", "dy", "dz", "dxy"), 1, 0),
+    ((2, 2, 2), 16, 8, "f64", 1, ("dx", "dz", "dyy", "dyz"), 0, 0),  # no padding column left
+    ((2, 2, 2), 32, 6, "f64", 1, ("dx", "dy", "dz", "dxx", "dxz"), 1, 0),
+    ((2, 2, 2), 32, 8, "f32", 1, ("dx", "dyy", "dz"), 0, 1),
+])
+def test_every_form_matches_the_banded_solve(lib, nb, N, g, dtype, nf, ops, n_iter, offset):
+    import torch
+    mesh = W.periodic_box_mesh(*nb, N, g)
+    # wave numbers in units of the box: every axis is periodic
+    L = [nb[a] * N * mesh.dx[0, a] for a in range(3)]
+    r = W.rng(77 + N + g + n_iter)
+    fs = []
+    for _ in range(nf):
+        s = W.sine_sum(r, 6, 1, 4)
+        s.k = 2 * np.pi * s.k / np.asarray(L)
+        fs.append(s)
+    flat = W.pack(W.sample(mesh, fs, np.float32 if dtype == "f32" else np.float64))
+    dev = torch.device("cuda", 0)
+    hold = torch.zeros(flat.size + 8, dtype=torch.float32 if dtype == "f32" else torch.float64, device=dev)
+    fields = hold[offset:offset + flat.size]
+    fields.copy_(torch.from_numpy(flat))
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), desc("Q13_1_d2"))
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F32 if dtype == "f32" else lib.CFD_F64)
+    mask = lib.op_mask(ops)
+    got = run(lib, B, fields, nf, mask, lib.CFD_TC_BF16_EXACT, n_iter, offset)
+    want = run(lib, B, fields, nf, mask, lib.CFD_FP64_BANDED, n_iter, 0)
+    tol = 2e-6 if dtype == "f32" else 1e-7
+    for i, op in enumerate(lib.ops_in_mask(mask)):
+        for q in range(nf):
+            e = rel_max(got[:, q, i], want[:, q, i])
+            assert e < tol, (op, q, e)
+
+
+@pytest.mark.parametrize("nblk", [1, 3])
+def test_rows_with_a_flat_operator_keep_their_accuracy(lib, nblk):
+    """A scheme whose interior stencil is nearly flat (its rows sum to several times their largest
+    entry): the row scale makes room for the level-0 sums.  Random fields, closed blocks, d_x."""
+    import torch
+    N, g = 32, 6
+    mesh = W.periodic_box_mesh(nblk, 1, 1, N, g)
+    M = 5
+    rhs = [0.0] * (2 * M + 1)
+    for m in range(1, M + 1):          # antisymmetric, consistent: sum m a_m = (1 + 2a) / 2
+        rhs[M + m] = 1.0
+    c = (1 + 2 * 0.45) / (2.0 * sum(m * rhs[M + m] for m in range(1, M + 1)))
+    for m in range(1, M + 1):
+        rhs[M + m] *= c
+        rhs[M - m] = -rhs[M + m]
+    d1 = {"deriv": 1, "order": 2, "a": 0.45, "rhs": rhs, "closure": rhs}
+    s = lib.cfd_scheme_create(d1, None)
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F64)
+    E = N + 2 * g
+    f = W.rng(5).uniform(-1, 1, size=(nblk, 1, E, E, E))
+    dev = torch.device("cuda", 0)
+    fields = torch.from_numpy(f.reshape(-1).copy()).to(dev)
+    got = run(lib, B, fields, 1, lib.CFD_OP_DX, lib.CFD_TC_BF16_EXACT, 0, 0).reshape(nblk, N, N, N)
+    # the closed (cyclic where the block is its own neighbour) system, solved in FP64
+    A, Bm = np.eye(N), np.zeros((N, E))
+    for k in range(N):
+        if nblk == 1:
+            A[k, (k - 1) % N] += 0.45
+            A[k, (k + 1) % N] += 0.45
+            for m in range(-M, M + 1):
+                Bm[k, g + (k + m) % N] += rhs[m + M]
+        else:
+            if 0 < k < N - 1:
+                A[k, k - 1] = A[k, k + 1] = 0.45
+            Bm[k, g + k - M:g + k + M + 1] = rhs
+    D = np.linalg.solve(A, Bm) / mesh.dx[0, 0]
+    I = slice(g, g + N)
+    want = np.einsum("ij,bzyj->bzyi", D, f[:, 0, I, I, :])
+    bound = 2.0 ** -36 * np.abs(D).sum(1)      # |f| < 1 = tau; 2^-37 sum |D f| is the design bound
+    assert np.all(np.abs(got - want) <= bound[None, None, None, :])
