@@ -38,6 +38,9 @@ struct DenseParams {
   double *halo_out;          // same layout, written by a halo pass (k_halo_rows)
   const int *nbr;            // [nblocks][26] neighbour table
   int halo_deg_mask;         // degrees whose halo columns are filled (bit d-1)
+  // exact form: halo_in / halo_out are [block][field][side: row 1, row N-2][pencil][halo_nd], halo_nd
+  // the degrees kept (2, or 1: the one of halo_deg_mask)
+  int halo_nd;
   int xrow;                  // x-axis stage with 16-byte aligned pencil rows: chunked row copies
   int xvec;                  // x-axis stage with a 16-byte aligned output: vector stores
   // Consecutive block ids (blocks[lb] = b0 + lb): offsets follow from the job index
@@ -81,6 +84,7 @@ void halo_rows_from(const std::vector<long double> &M, int cols, HaloRows &R);
 // P.halo_in, to the neighbours' previous iterate), written to P.halo_out.
 cfd_status halo_rows_launch(const DenseParams &P, const HaloRows &R, bool f32_in, cudaStream_t st);
 
+cfd_status dense_exact_halo(const DenseParams &P, bool f32_in, unsigned grid, cudaStream_t st);
 // One launch of the exact form (dense_exact.cuh) for blocks of 16^3 / 32^3.
 cfd_status dense_exact_launch16(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);
 cfd_status dense_exact_launch32(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);

@@ -240,9 +240,13 @@ __device__ __noinline__ void rows_any(uint32_t taddr, uint32_t lev, int etau, co
 // ---------------------------------------------------------------- the kernel
 
 // N: block size (16, 32).  AXIS 0, 1, 2: pencils along z, y, x with ghost width 4 (every stride and
-// the split of a pencil's columns are constants); AXIS 3: any axis and ghost width.  ITER: the final
-// pass of an iterated stage, four more columns per pencil with the neighbours' previous iterate.
-template <typename TI, typename TO, int N, int AXIS, bool ITER>
+// the split of a pencil's columns are constants); AXIS 3: any axis and ghost width.  ITER: a pass of
+// an iterated stage that takes the neighbours' previous iterate as four more columns per pencil.
+// HALO: a halo pass of the hybrid iteration (Eq. iter_center_P): four operator rows (16 with their
+// zero padding), whose outputs are the values the neighbours read at their k^c nodes.  It costs the
+// producers' share of a stage, against ~11 FP32 operations per coefficient and row in compensated
+// FP32 on the CUDA cores (256^3, 4 fields: see halo_pass in dense_tc.cu).
+template <typename TI, typename TO, int N, int AXIS, bool ITER, bool HALO>
 __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_constant__ DenseParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr bool GEN = AXIS == 3;
@@ -253,6 +257,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   const int g = GEN ? P.g : 4;
   const int E = N + 2 * g;
   const int R = P.rows;
+  constexpr int SR = HALO ? 16 : N;  // operator rows of a segment
   const int B_BYTES = kSl * R * KP * 2;
   const int kind = P.tma_kind, nstg = P.nstg, stg_bytes = P.stg_bytes;
   const int nbuf = R > 32 ? 2 : 4, buf_cols = kTmemCols / nbuf;
@@ -289,8 +294,10 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       mbar_init(s_full(i), kind ? 1 : kXProd);
       mbar_init(s_empty(i), kXProdWarps);
     }
-    // 16 units of 8 rows in a tile (N = 16, one operator: 8, and two warps of a quadrant sit it out)
-    for (int i = 0; i < 4; ++i) { mbar_init(t_full(i), 1); mbar_init(t_empty(i), R < 32 ? kXEpiWarps / 2 : kXEpiWarps); }
+    // warps that read a TMEM buffer: all, with 16 rows (N = 16, one operator) half of them in turn, in
+    // a halo pass one per lane quadrant in turn
+    const int readers = HALO ? kXEpiWarps / 4 : (R < 32 ? kXEpiWarps / 2 : kXEpiWarps);
+    for (int i = 0; i < 4; ++i) { mbar_init(t_full(i), 1); mbar_init(t_empty(i), readers); }
     for (int i = 0; i < kXEtau; ++i) mbar_init(meta_full(i), kXProdWarps);
     mbar_init(drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;");
@@ -298,12 +305,12 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   // operator digits: slices stacked along the MMA's N rows, [t][segment][N]
   for (int sg = 0; sg < P.nseg[0]; ++sg) {
     const uint4 *src = reinterpret_cast<const uint4 *>(P.seg_img[0][sg]);
-    constexpr int U = N * KP * 2 / 16;
+    constexpr int U = SR * KP * 2 / 16;
     for (int i = tid; i < kSl * U; i += kXThreads) {
       const int t = i / U, r = i - t * U;
-      reinterpret_cast<uint4 *>(sB + (t * R + sg * N) * KP * 2)[r] = __ldg(src + i);
+      reinterpret_cast<uint4 *>(sB + (t * R + sg * SR) * KP * 2)[r] = __ldg(src + i);
     }
-    for (int i = tid; i < N; i += kXThreads) s_rowexp[sg * N + i] = P.seg_exp[0][sg][i];
+    for (int i = tid; i < SR; i += kXThreads) s_rowexp[sg * SR + i] = P.seg_exp[0][sg][i];
   }
   if constexpr (!GEN) {
     // the columns behind the pencil (K padding; the halo columns are rewritten per tile) stay zero
@@ -394,33 +401,49 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       }
       asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(s_full(sb)) : "memory");
     };
-    // the neighbours' previous iterate at k^c, as columns E + m of the pencil: m = 2d from the lower
-    // neighbour's row N-2, m = 2d + 1 from the upper neighbour's row 1 (degree slot d)
-    auto halo = [&](int tile, int m) -> TI {
+    // The neighbours' previous iterate at k^c, as columns E + m of the pencil: m = 2d from the lower
+    // neighbour's row N-2 (side 1), m = 2d + 1 from the upper neighbour's row 1 (side 0), degree slot d.
+    // Layout [block][field][side][pencil][halo_nd]: a stage of one degree holds (and moves) only its own.
+    // The neighbour of tile t + 2 is looked up, and the values of tile t + 1 are loaded, while tile t is
+    // split: neither load is waited for (T stages at 256^3 with the lookup in the chain: 0.34 ms).
+    auto halo_block = [&](int tile, int up) -> int {
+      if (tile >= tr.end) return -1;
       const TileCoord c = tile_coord(P, tile, pl);
-      const int d = m >> 1, up = m & 1;
-      if (!c.valid || !((P.halo_deg_mask >> d) & 1)) return TI(0);
       const int sg = up ? 1 : -1;
-      const int nb = P.nbr[c.b * 26 + dir_index_dev(axis == 0 ? sg : 0, axis == 1 ? sg : 0, axis == 2 ? sg : 0)];
-      const long long hp = ((long long)nb * P.nf + c.q) * (long long)(P.n1 * P.n2) + tile_pencil(P, tile, pl);
-      return TI(P.halo_in[hp * 4 + 2 * d + (up ? 0 : 1)]);
+      return !c.valid ? -1 : P.nbr[c.b * 26 + dir_index_dev(axis == 0 ? sg : 0, axis == 1 ? sg : 0, axis == 2 ? sg : 0)];
+    };
+    const int np = P.n1 * P.n2;
+    auto halo = [&](int tile, int nb, int m) -> TI {
+      const int d = m >> 1, up = m & 1;
+      if (nb < 0 || !((P.halo_deg_mask >> d) & 1)) return TI(0);
+      const int job = fdiv(tile, P.inv_tpj), q = job - fdiv(job, P.inv_nf) * P.nf;
+      const long long hp = (((long long)nb * P.nf + q) * 2 + (up ? 0 : 1)) * np + tile_pencil(P, tile, pl);
+      return TI(P.halo_in[hp * P.halo_nd + (P.halo_nd == 2 ? d : 0)]);
     };
     constexpr int NFULL = GEN ? (NCH + 1) / 2 : N / 16;          // whole chunks of this lane
     constexpr int NV = NFULL * 8 + (GEN ? 0 : 4 + (ITER ? 2 : 0));  // values of this lane
     if (!kind)
       for (int k = 0, t = tr.first; k < nstg && t < tr.end; ++k, t += tr.step) prefetch(t, k);
     TI hq[4] = {TI(0), TI(0), TI(0), TI(0)};
+    int nb[2] = {-1, -1};  // lower and upper neighbour of the next tile to load
     auto load_halo = [&](int tile) {
       if constexpr (ITER) {
+        const int lo = nb[0], hi = nb[1];
+        nb[0] = halo_block(tile + tr.step, 0);
+        nb[1] = halo_block(tile + tr.step, 1);
         if constexpr (GEN) {
 #pragma unroll
-          for (int m = 0; m < 4; ++m) hq[m] = halo(tile, m);
-        } else {  // both lanes of a pencil take one degree slot
-          hq[0] = halo(tile, 2 * half);
-          hq[1] = halo(tile, 2 * half + 1);
+          for (int m = 0; m < 4; ++m) hq[m] = halo(tile, m & 1 ? hi : lo, m);
+        } else {  // the two lanes of a pencil take one degree slot each
+          hq[0] = halo(tile, lo, 2 * half);
+          hq[1] = halo(tile, hi, 2 * half + 1);
         }
       }
     };
+    if (ITER) {
+      nb[0] = halo_block(tr.first, 0);
+      nb[1] = halo_block(tr.first, 1);
+    }
     int it = 0;
     if (tr.first < tr.end) load_halo(tr.first);
     for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
@@ -518,6 +541,38 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     // |Y| < 2^47: Y 2^E is normal; FP32: the scale itself is a normal float
     constexpr int kLo = sizeof(TO) == 8 ? -1022 + kYUnit : -126 + kFUnit;
     constexpr int kHi = sizeof(TO) == 8 ? 976 + kYUnit : 127 + kFUnit;
+    if constexpr (HALO) {
+      // rows 0..3: row 1 and row N-2 of degree slot 0, then of slot 1 (biased schemes: rows 1 and 2);
+      // the tiles go round the four warps of a lane quadrant
+      const int np = P.n1 * P.n2;
+      int it = 0;
+      for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
+        if ((it & 3) != ew) continue;
+        const TileCoord c = tile_coord(P, tile, pl);
+        if (!wait(meta_full(it & (kXEtau - 1)), (uint32_t)((it / kXEtau) & 1))) { failed = true; break; }
+        const int etau = s_etau[(it & (kXEtau - 1)) * kTile + pl];
+        if (!wait(t_full(ew), (uint32_t)((it >> 2) & 1))) { failed = true; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        uint32_t acc[kSl][8];
+        load_levels(acc, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(ew * buf_cols), R);
+        release_levels(t_empty(ew));
+        double h[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          h[r] = scaled_double<true>(__ll2double_rn(exact_y(acc, r)), s_rowexp[r] + etau - kYUnit, etau == kBadTau);
+        if (!c.valid) continue;
+        double *o = P.halo_out + (((long long)c.b * P.nf + c.q) * 2 * np + tile_pencil(P, tile, pl)) * P.halo_nd;
+        const long long side = (long long)np * P.halo_nd;
+        if (P.halo_nd == 2) {
+          *reinterpret_cast<double2 *>(o) = make_double2(h[0], h[2]);
+          *reinterpret_cast<double2 *>(o + side) = make_double2(h[1], h[3]);
+        } else {
+          const bool second = P.halo_deg_mask == 2;
+          o[0] = second ? h[2] : h[0];
+          o[side] = second ? h[3] : h[1];
+        }
+      }
+    } else {
     const int units = P.nseg[0] * UPS;
     const bool rows_out = axis == 2 && P.out_box_bytes != 0;
     unsigned char *box = s_out + (warp - kXProdWarps) * P.out_box_bytes;
@@ -603,6 +658,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     }
     // the output boxes must have been read before the CTA leaves
     if (rows_out && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    }
   } else if (warp == kXProdWarps + kXEpiWarps) {
     // ================================================================ MMA issue
     asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");

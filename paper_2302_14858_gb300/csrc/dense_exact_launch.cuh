@@ -27,7 +27,7 @@ size_t plan_smem(DenseParams &P) {
   return std::max(fixed + out + (size_t)P.nstg * P.stg_bytes, (size_t)116 * 1024);
 }
 
-template <typename TI, typename TO, int N, int AXIS, bool ITER>
+template <typename TI, typename TO, int N, int AXIS, bool ITER, bool HALO = false>
 cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   const size_t smem = plan_smem<TI, N>(P);
   // The shared-memory opt-in is made once per device and instantiation, for the most any launch may
@@ -36,7 +36,7 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   int dev = 0;
   cfd_status s = cuda_fail(cudaGetDevice(&dev), "cudaGetDevice");
   if (s != CFD_OK) return s;
-  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER>;
+  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER, HALO>;
   if (dev < 0 || dev >= 64 || !opted[dev].load()) {
     s = cuda_fail(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax),
                   "cudaFuncSetAttribute");
@@ -44,9 +44,9 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
     if (dev >= 0 && dev < 64) opted[dev].store(true);
   }
   if (smem > kSmemMax) { set_error("dense: shared memory plan too large"); return CFD_ERR_UNSUPPORTED; }
-  launch_begin(KF_DENSE, st);
+  launch_begin(HALO ? KF_HALO : KF_DENSE, st);
   fn<<<grid, kXThreads, smem, st>>>(P);
-  launch_end(KF_DENSE, st);
+  launch_end(HALO ? KF_HALO : KF_DENSE, st);
   return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
 }
 
@@ -60,6 +60,17 @@ cfd_status launch_exact_types(const DenseParams &P, unsigned grid, cudaStream_t 
     return it ? launch_one<TI, TO, N, 0, true>(P, grid, st) : launch_one<TI, TO, N, 0, false>(P, grid, st);
   }
   return it ? launch_one<TI, TO, N, 3, true>(P, grid, st) : launch_one<TI, TO, N, 3, false>(P, grid, st);
+}
+
+// Halo passes: the first one (closed operator rows) has the axis compiled in for ghost width 4; the
+// further iterates, which only n_iter > 1 needs, take the general form.
+template <typename TI, int N>
+cfd_status launch_exact_halo(const DenseParams &P, unsigned grid, cudaStream_t st) {
+  if (P.halo_in) return launch_one<TI, double, N, 3, true, true>(P, grid, st);
+  if (P.g != 4) return launch_one<TI, double, N, 3, false, true>(P, grid, st);
+  if (P.axis == 2) return launch_one<TI, double, N, 2, false, true>(P, grid, st);
+  if (P.axis == 1) return launch_one<TI, double, N, 1, false, true>(P, grid, st);
+  return launch_one<TI, double, N, 0, false, true>(P, grid, st);
 }
 
 template <int N>

@@ -1171,6 +1171,9 @@ struct DenseGroup {
   bool biased = false;
   DenseOp bop[3][2], bopI[3][2];
   HaloRows bhr0[3], bhrI[3];
+  // the same rows (16 with zero padding) as digit images, for the exact form's halo passes:
+  // [box][0 closed, 1 iterated], centred and biased
+  DenseOp hop[3][2], bhop[3][2];
 };
 
 // Launch choices of the autotuner: per request (fields, ops, precision, iterations, entry
@@ -1193,19 +1196,23 @@ DenseState *state_of(cfd_blocks_s *B) { return reinterpret_cast<DenseState *>(B-
 
 }  // namespace
 
-static cfd_status upload_op(cfd_blocks_s *B, const std::vector<ld> &D, int rows, int cols, int Kp, DenseOp &o) {
+// Device images of one operator; halo rows (all = false) only ever run in the exact form.
+static cfd_status upload_op(cfd_blocks_s *B, const std::vector<ld> &D, int rows, int cols, int Kp, DenseOp &o,
+                            bool all_forms = true) {
   std::vector<uint16_t> img, imgx;
   std::vector<uint32_t> img32;
   std::vector<int> rexp, rexpx;
-  digit_image(D, rows, cols, Kp, img, rexp);
   exact_image(D, rows, cols, Kp, imgx, rexpx);
-  tf32_image(D, rows, cols, Kp, img32);
+  if (all_forms) {
+    digit_image(D, rows, cols, Kp, img, rexp);
+    tf32_image(D, rows, cols, Kp, img32);
+  }
   // one device allocation and one copy per operator: binding a mesh makes a few dozen of these
   std::vector<unsigned char> all;
   auto add = [&](const auto &v) {
     const size_t at = (all.size() + 15) & ~(size_t)15;
     all.resize(at + v.size() * sizeof(v[0]));
-    memcpy(all.data() + at, v.data(), v.size() * sizeof(v[0]));
+    if (!v.empty()) memcpy(all.data() + at, v.data(), v.size() * sizeof(v[0]));
     return at;
   };
   const size_t a0 = add(img), a1 = add(imgx), a2 = add(img32), a3 = add(rexp), a4 = add(rexpx);
@@ -1252,6 +1259,25 @@ cfd_status dense_bind(cfd_blocks_s *B) {
       const bool cyc = ncyc == (int)B->groups[gi].size();
       if (ncyc && !cyc) { G.ok = false; break; }
       G.cyc[box] = cyc;
+      // an axis with the spacing and kind of an earlier one has its operators
+      int same = -1;
+      for (int pb = 0; pb < box; ++pb)
+        if (G.cyc[pb] == cyc && B->dx[b0 * 3 + 2 - pb] == B->dx[b0 * 3 + ax]) same = pb;
+      if (same >= 0) {
+        for (int d = 0; d < 2; ++d) {
+          G.op[box][d] = G.op[same][d];
+          G.opI[box][d] = G.opI[same][d];
+          G.hop[box][d] = G.hop[same][d];
+          G.bop[box][d] = G.bop[same][d];
+          G.bopI[box][d] = G.bopI[same][d];
+          G.bhop[box][d] = G.bhop[same][d];
+        }
+        G.hr0[box] = G.hr0[same];
+        G.hrI[box] = G.hrI[same];
+        G.bhr0[box] = G.bhr0[same];
+        G.bhrI[box] = G.bhrI[same];
+        continue;
+      }
       std::vector<ld> H0(16 * E, 0), HI(16 * G.Kp, 0);
       for (int d = 1; d <= 2; ++d) {
         if (!B->s[d - 1].present) continue;
@@ -1291,6 +1317,9 @@ cfd_status dense_bind(cfd_blocks_s *B) {
       if (!cyc && G.iter_ok) {
         halo_rows_from(H0, E, G.hr0[box]);
         halo_rows_from(HI, G.Kp, G.hrI[box]);
+        cfd_status s = upload_op(B, H0, 16, E, G.Kp, G.hop[box][0], false);
+        if (s == CFD_OK) s = upload_op(B, HI, 16, G.Kp, G.Kp, G.hop[box][1], false);
+        if (s != CFD_OK) return s;
       }
       if (B->biased.present && B->biased.kc <= N) {
         const BiasedCoef &bc = B->biased;
@@ -1320,6 +1349,9 @@ cfd_status dense_bind(cfd_blocks_s *B) {
         if (!cyc && G.iter_ok) {
           halo_rows_from(BH0, E, G.bhr0[box]);
           halo_rows_from(BHI, G.Kp, G.bhrI[box]);
+          cfd_status s = upload_op(B, BH0, 16, E, G.Kp, G.bhop[box][0], false);
+          if (s == CFD_OK) s = upload_op(B, BHI, 16, G.Kp, G.Kp, G.bhop[box][1], false);
+          if (s != CFD_OK) return s;
         }
         G.biased = true;
       }
@@ -1490,6 +1522,13 @@ void plan_out_tma(DenseParams &P, size_t elem) {
   P.out_box_bytes = (int)(8 * 32 * elem);
 }
 
+void set_launch_constants(DenseParams &P) {
+  P.wait_limit = dense_wait_limit();
+  P.inv_tpj = 1.0f / (float)P.tiles_per_job;
+  P.inv_nf = 1.0f / (float)P.nf;
+  P.inv_n2 = 1.0f / (float)P.n2;
+}
+
 // Launch one stage with the choices the autotuner made for it (TMA staging and interleaved
 // tiles by default); during cfd_autotune, launch every candidate three times, time the last two
 // with events on the stream, and keep the fastest.  Repeated launches of a stage are idempotent
@@ -1499,10 +1538,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
   const bool exact = S == 4;
   auto launch = [&](DenseParams Q) -> cfd_status {
     if (exact) {
-      Q.wait_limit = dense_wait_limit();
-      Q.inv_tpj = 1.0f / (float)Q.tiles_per_job;
-      Q.inv_nf = 1.0f / (float)Q.nf;
-      Q.inv_n2 = 1.0f / (float)Q.n2;
+      set_launch_constants(Q);
       return Q.N == 32 ? dense_exact_launch32(Q, Q.in_field && f32, f32, grid, st)
                        : dense_exact_launch16(Q, Q.in_field && f32, f32, grid, st);
     }
@@ -1557,6 +1593,34 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
 }
 
 }  // namespace
+
+// One halo pass of the hybrid iteration along the stage's axis: the four rows of every pencil that the
+// neighbours read, from the pencils (first iterate) or with the previous iterate's halo columns.
+//   exact: four of 16 operator rows through the tensor cores (dense_exact.cuh).  256^3, 4 FP64 fields,
+//     six passes: HALO_NEW ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
+//     coefficient and row where the digit split costs ~20 instructions per value for all rows;
+//   otherwise compensated FP32 on the CUDA cores (halo_rows.cu), whose cost does not depend on the form.
+static cfd_status halo_pass(DenseParams H, const DenseOp &op, const HaloRows &rows, bool exact, bool f32, int sms,
+                            cudaStream_t st) {
+  const bool f32_in = H.in_field && f32;
+  if (!exact) return halo_rows_launch(H, rows, f32_in, st);
+  const int E = H.N + 2 * H.g, np = H.n1 * H.n2;
+  const size_t ein = f32_in ? 4 : 8;
+  H.scratch_out = nullptr;
+  H.nseg[0] = 1;
+  H.passes = 1;
+  H.rows = 16;
+  H.seg_img[0][0] = op.imgx;
+  H.seg_exp[0][0] = op.rowexpx;
+  H.xrow = H.axis == 2 && (E * ein) % 16 == 0 && ((uintptr_t)H.in & 15) == 0;
+  H.tiles_per_job = (np + kTile - 1) / kTile;
+  H.ntiles = H.tiles_per_job * H.nblk * H.nf;
+  H.tile_order = 0;
+  H.out_box_bytes = 0;
+  plan_tma(H, ein, true);
+  set_launch_constants(H);
+  return dense_exact_halo(H, f32_in, (unsigned)std::min(H.ntiles, sms), st);
+}
 
 struct DensePlanSizes {
   size_t gy = 0, gz = 0;  // elements per group (max over groups) of the two intermediates
@@ -1690,6 +1754,8 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
           P.seg_op[ps][k] = op[sgi];
         }
       }
+      // the halo values of a degree that the stage does not apply are not computed
+      if (prec == CFD_TC_BF16_EXACT) P.halo_deg_mask = (m1 >= 0 ? 1 : 0) | (m2 >= 0 ? 2 : 0);
       return n > 0;
     };
     // A stage along a decomposed axis with n_iter > 0 (Eq. iter_center_P): halo
@@ -1697,19 +1763,18 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
     // [n_iter-1] (the values the neighbours need at their k^c nodes) into a
     // ping-pong buffer; the final pass applies the iterated operator with
     // those values as four extra K columns.  Each pass is one launch: all
-    // blocks of iterate i are complete before any block reads them.  The halo
-    // passes are four dot products per pencil and run on the CUDA cores in
-    // compensated FP32 (halo_rows.cu), at a fraction of a tensor-core pass.
+    // blocks of iterate i are complete before any block reads them.
     auto run_stage = [&](DenseParams P, int box) -> cfd_status {
       if (!iterating(box)) return run(P);
+      P.halo_nd = P.halo_deg_mask == 3 ? 2 : 1;
       DenseParams H = P;
       H.scratch_out = nullptr;
       for (int it = 0; it < n_iter; ++it) {
         H.halo_in = it == 0 ? nullptr : halo[(it - 1) & 1];
         H.halo_out = halo[it & 1];
         H.kext = it == 0 ? E : E + 4;
-        cfd_status r = halo_rows_launch(H, it == 0 ? G.hr0[box] : G.hrI[box],
-                                        H.in_field && B->dtype == CFD_F32, st);
+        cfd_status r = halo_pass(H, G.hop[box][it > 0], it == 0 ? G.hr0[box] : G.hrI[box], prec == CFD_TC_BF16_EXACT,
+                                 B->dtype == CFD_F32, sms, st);
         if (r != CFD_OK) return r;
       }
       P.halo_in = halo[(n_iter - 1) & 1];
@@ -1976,13 +2041,14 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
         }
       }
       if (iter) {
-        // halo passes on the CUDA cores (halo_rows.cu), as for the centred operators
+        P.halo_nd = 2;
         DenseParams H = P;
         for (int it = 0; it < n_iter; ++it) {
           H.halo_in = it == 0 ? nullptr : halo[(it - 1) & 1];
           H.halo_out = halo[it & 1];
           H.kext = it == 0 ? E : E + 4;
-          if ((s = halo_rows_launch(H, it == 0 ? G.bhr0[box] : G.bhrI[box], B->dtype == CFD_F32, st)) != CFD_OK)
+          if ((s = halo_pass(H, G.bhop[box][it > 0], it == 0 ? G.bhr0[box] : G.bhrI[box], prec == CFD_TC_BF16_EXACT,
+                             B->dtype == CFD_F32, sms, st)) != CFD_OK)
             return s;
         }
         P.halo_in = halo[(n_iter - 1) & 1];
