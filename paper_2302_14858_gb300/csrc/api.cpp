@@ -12,6 +12,7 @@
 
 #include "cfd_internal.h"
 #include "dense.h"
+#include "line.h"
 
 namespace cfd {
 
@@ -186,76 +187,6 @@ cfd_status copy_desc(const cfd_scheme_desc *d, int deg, SchemeCoef &s) {
   return CFD_OK;
 }
 
-// Thomas factors of a tridiagonal system with rows (lo_k, 1, up_k), computed
-// in FP64 in the textbook order: den_k = 1 - lo_k c_{k-1}, c_k = up_k / den_k.
-void thomas_factors(int n, const double *lo, const double *up, double *c, double *inv) {
-  double cprev = 0;
-  for (int k = 0; k < n; ++k) {
-    const double den = 1.0 - lo[k] * cprev;
-    c[k] = (k < n - 1) ? up[k] / den : 0.0;
-    inv[k] = 1.0 / den;
-    cprev = c[k];
-  }
-}
-
-void build_tables(const SchemeCoef &s, int N, LineTables &T) {
-  memset(&T, 0, sizeof(T));
-  T.N = N;
-  T.M = s.M;
-  T.h = s.h;
-  T.d = s.d;
-  T.a = s.a;
-  for (int i = 0; i < 2 * s.M + 1; ++i) T.rhs[i] = s.rhs[i];
-  for (int i = 0; i < 2 * s.h + 1; ++i) T.clo[i] = s.clo[i];
-  // closed system: unit rows at k = 0 and N-1
-  double up[kMaxIter];
-  for (int k = 0; k < N; ++k) {
-    const bool unit = (k == 0 || k == N - 1);
-    T.lo[k] = unit ? 0.0 : s.a;
-    up[k] = unit ? 0.0 : s.a;
-  }
-  thomas_factors(N, T.lo, up, T.c, T.inv);
-  // iterated system: rows k = -2..N+1 at k + 2; unit rows at both ends
-  const int n = N + 4;
-  for (int i = 0; i < n; ++i) {
-    const bool unit = (i == 0 || i == n - 1);
-    T.ilo[i] = unit ? 0.0 : s.a;
-    up[i] = unit ? 0.0 : s.a;
-  }
-  thomas_factors(n, T.ilo, up, T.ic, T.iinv);
-  // cyclic: A = T + u v^T, gamma = -1, u = (gamma, 0.., a), v = (1, 0.., -a)
-  //   T_00 = 1 - gamma = 2, T_{N-1,N-1} = 1 + a^2 (rows of T scaled to unit
-  //   diagonal for the Thomas factors below).
-  {
-    double dl[kMaxN], dd[kMaxN], du[kMaxN];
-    for (int k = 0; k < N; ++k) {
-      dl[k] = (k == 0) ? 0.0 : s.a;
-      du[k] = (k == N - 1) ? 0.0 : s.a;
-      dd[k] = 1.0;
-    }
-    dd[0] = 2.0;
-    dd[N - 1] = 1.0 + s.a * s.a;
-    // general Thomas with diagonal: den_k = dd_k - dl_k c_{k-1}
-    double cprev = 0;
-    for (int k = 0; k < N; ++k) {
-      const double den = dd[k] - dl[k] * cprev;
-      T.yc[k] = (k < N - 1) ? du[k] / den : 0.0;
-      T.yinv[k] = 1.0 / den;
-      T.ylo[k] = dl[k];
-      cprev = T.yc[k];
-    }
-    // z = T^-1 u
-    double u[kMaxN] = {};
-    u[0] = -1.0;
-    u[N - 1] = s.a;
-    double y[kMaxN];
-    for (int k = 0; k < N; ++k) y[k] = (u[k] - (k ? T.ylo[k] * y[k - 1] : 0.0)) * T.yinv[k];
-    for (int k = N - 2; k >= 0; --k) y[k] -= T.yc[k] * y[k + 1];
-    for (int k = 0; k < N; ++k) T.z[k] = y[k];
-    T.vfac = 1.0 / (1.0 + (T.z[0] - s.a * T.z[N - 1]));
-  }
-}
-
 int dir_index(int dz, int dy, int dx) {
   int r = 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1);
   return r > 13 ? r - 1 : r;
@@ -286,12 +217,6 @@ OpList ops_of(unsigned mask) {
 const int kAxisOfOp1[3] = {2, 1, 0};                 // dx, dy, dz
 const int kMixed[3][2] = {{2, 1}, {2, 0}, {1, 0}};   // (i, j): dxy, dxz, dyz
 
-struct Workspace {
-  double *scratch = nullptr;
-  double *halo[2] = {nullptr, nullptr};
-  size_t scratch_elems = 0, halo_elems = 0;
-};
-
 void banded_workspace_sizes(const cfd_blocks_s *B, int nf, unsigned mask, int n_iter, size_t *scratch,
                             size_t *halo) {
   size_t sc = 0, hp = 0;
@@ -305,114 +230,186 @@ void banded_workspace_sizes(const cfd_blocks_s *B, int nf, unsigned mask, int n_
   *halo = n_iter > 0 ? (size_t)B->nblocks * nf * hp * 2 : 0;
 }
 
-cfd_status run_stage(cfd_blocks_s *B, LineParams P, const LineTables &T, int n_iter, Workspace &ws,
-                     cudaStream_t st) {
-  for (int pass = 0; pass <= n_iter; ++pass) {
-    P.pass = pass;
-    P.last = pass == n_iter;
-    P.halo_in = pass > 0 ? ws.halo[(pass - 1) & 1] : nullptr;
-    P.halo_out = ws.halo[pass & 1];
-    cfd_status s = launch_line(P, T, st, B->dtype);
-    if (s != CFD_OK) return s;
-  }
-  return CFD_OK;
-}
+// table of (degree, box axis, half) among a size's tables
+int ptab_index(int deg, int box, bool half) { return deg == 1 ? 2 * box + (half ? 1 : 0) : 6 + box; }
 
+// FP64 banded apply.  `region`: the mixed ops' scratch (region_elems doubles), `halo`: the halo values of
+// the iteration (halo_elems doubles); where both exist the halo space follows the scratch directly.
+//
+// Launches (all blocks, fields and axes of a size together): the single derivatives; then per inner axis
+// j of the mixed ops the ghost strips of D_j (local evaluation on the ghost rows of the outer axes) and
+// D_i on [strip | own points | strip].  Own points of D_j come from its output slot (FP64 fields with d_j
+// requested) or from one scratch copy.  Each launch is preceded by n_iter halo passes.
 cfd_status apply_banded(cfd_blocks_s *B, const void *fields, int nf, unsigned mask, int n_iter, void *out,
-                        Workspace &ws, cudaStream_t st) {
+                        double *region, size_t region_elems, double *halo, size_t halo_elems, cudaStream_t st) {
   const OpList ol = ops_of(mask);
+  auto slot = [&](int bit) {
+    for (int i = 0; i < ol.n; ++i)
+      if (ol.bit[i] == bit) return i;
+    return -1;
+  };
+  if (((mask & 0x1C7) && !B->s[0].present) || ((mask & 0x38) && !B->s[1].present)) {
+    set_error((mask & 0x1C0) && !B->s[0].present ? "mixed ops need the first-degree scheme"
+                                                 : "op needs a scheme that was not given");
+    return CFD_ERR_ARG;
+  }
+  for (int d = 0; d < 2; ++d) {
+    const SchemeCoef &s = B->s[d];
+    if (!(mask & (d ? 0x38 : 0x1C7))) continue;
+    if (!((s.M == 3 && (s.h == 4 || s.h == 5)) || (s.M == 2 && s.h == 4) || (s.M == 1 && s.h == 3))) {
+      set_error("banded path: unsupported stencil widths (M, closure half-width)");
+      return CFD_ERR_UNSUPPORTED;
+    }
+  }
+  const bool f32 = B->dtype == CFD_F32;
+  const size_t all_elems = region_elems + halo_elems;
+  double *all = region_elems ? region : halo;
   for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
-    const int N = B->sizes[gi], g = B->ng, E = N + 2 * g;
-    LineParams P;
-    memset(&P, 0, sizeof(P));
-    P.blocks = B->d_groups[gi];
-    P.extpre = B->d_extpre;
-    P.intpre = B->d_intpre;
-    P.nbr = B->d_nbr;
-    P.scale = B->d_scale;
-    P.nblk = (int)B->groups[gi].size();
-    P.nf = nf;
-    P.nops = ol.n;
-    P.g = g;
-    P.status = B->d_status;
-    for (int oi = 0; oi < ol.n; ++oi) {
-      const int bit = ol.bit[oi];
-      P.opidx = oi;
-      if (bit < 6) {
-        const int a = kAxisOfOp1[bit % 3];
-        const int deg = bit < 3 ? 1 : 2;
-        const OpSet &os = B->ops[gi];
-        if (!B->s[deg - 1].present) { set_error("op needs a scheme that was not given"); return CFD_ERR_ARG; }
-        LineParams Q = P;
-        Q.in = fields;
-        Q.in_field = 1;
-        Q.out = out;
-        Q.out_mode = 0;
-        Q.axis = a;
-        Q.t1 = a == 0 ? 1 : 0;
-        Q.t2 = a == 2 ? 1 : 2;
-        for (int t = 0; t < 3; ++t) {
-          Q.in_dims[t] = E;
-          Q.out_dims[t] = N;
-          Q.in_start[t] = (t == a) ? 0 : g;
-          Q.out_start[t] = 0;
+    const int N = B->sizes[gi], g = B->ng;
+    const std::vector<int> &blocks = B->groups[gi];
+    const long long per = (long long)blocks.size() * nf, n3 = (long long)N * N * N;
+    const PencilTab *tabs = static_cast<const PencilTab *>(B->d_ptab[gi]);
+    PencilArgs A;
+    memset(&A, 0, sizeof(A));
+    A.field = fields;
+    A.out = out;
+    A.region = region;
+    A.blocks = B->d_groups[gi];
+    A.lidx = B->d_lidx;
+    A.nbr = B->d_nbr;
+    A.extpre = B->d_extpre;
+    A.intpre = B->d_intpre;
+    A.scale = B->d_scale;
+    A.nblk = (int)blocks.size();
+    A.nf = nf;
+    A.nops = ol.n;
+    A.g = g;
+    // blocks that are their own neighbour along an axis (no halo passes there): all, none or some
+    bool cyc[3], some[3];
+    for (int a = 0; a < 3; ++a) {
+      size_t n = 0;
+      for (int b : blocks)
+        if (B->nbr[b * 26 + dir_index(-(a == 0), -(a == 1), -(a == 2))] == b &&
+            B->nbr[b * 26 + dir_index(a == 0, a == 1, a == 2)] == b)
+          ++n;
+      cyc[a] = n == blocks.size();
+      some[a] = n > 0 && !cyc[a];
+    }
+    int W = 0;
+    for (int d = 0; d < 2; ++d)
+      if (B->s[d].present) W = std::max(W, std::max(B->s[d].h, B->s[d].M + 1));
+    auto half_width = [&](const PencilTask &t) { return B->s[t.tab - tabs >= 6 ? 1 : 0].M; };
+    // tasks in as few launches as their number and the halo space allow
+    auto run = [&](std::vector<PencilTask> ts, double *hbase, size_t hcap) -> cfd_status {
+      const int bufs = n_iter > 1 ? 2 : 1;
+      for (size_t k = 0, n = ts.size(); k < n; ++k)
+        if (some[ts[k].axis]) {  // cyclic and other blocks in two tasks
+          ts[k].only = 2;
+          ts.push_back(ts[k]);
+          ts.back().only = 1;
         }
-        Q.n1 = N;
-        Q.n2 = N;
-        Q.deg = deg;
-        cfd_status s = run_stage(B, Q, os.tab[deg - 1], n_iter, ws, st);
-        if (s != CFD_OK) return s;
-      } else {
-        if (!B->s[0].present) { set_error("mixed ops need the first-degree scheme"); return CFD_ERR_ARG; }
-        const int mi = bit - 6;
-        const int norders = B->mixed_one_order ? 1 : 2;  // one order: written directly (out_mode 0)
-        for (int order = 0; order < norders; ++order) {
-          const int ai = order == 0 ? kMixed[mi][0] : kMixed[mi][1];  // outer (applied last)
-          const int aj = order == 0 ? kMixed[mi][1] : kMixed[mi][0];  // inner
-          const int ak = 3 - ai - aj;
-          // stage 1: D_j on rows extended along i
-          LineParams S1 = P;
-          S1.in = fields;
-          S1.in_field = 1;
-          S1.out = ws.scratch;
-          S1.out_mode = 2;
-          S1.axis = aj;
-          S1.t1 = std::min(ai, ak);
-          S1.t2 = std::max(ai, ak);
-          for (int t = 0; t < 3; ++t) {
-            S1.in_dims[t] = E;
-            S1.in_start[t] = (t == ak) ? g : 0;
-            S1.out_dims[t] = (t == ai) ? E : N;
-            S1.out_start[t] = 0;
+      for (size_t i = 0; i < ts.size();) {
+        size_t used = 0, j = i;
+        std::vector<long long> off;
+        // (one launch has one interior half-width: degrees of different widths go apart)
+        while (j < ts.size() && j - i < (size_t)kMaxTasks && half_width(ts[j]) == half_width(ts[i])) {
+          const size_t need = n_iter && !cyc[ts[j].axis] && ts[j].only != 1 ? (size_t)ts[j].n1 * ts[j].n2 * per * 2 : 0;
+          if (used + bufs * need > hcap && need) {
+            if (j == i) { set_error("banded path: halo space too small"); return CFD_ERR_ARG; }
+            break;
           }
-          S1.n1 = (S1.t1 == ai) ? E : N;
-          S1.n2 = (S1.t2 == ai) ? E : N;
-          S1.out_box = (unsigned long long)E * N * N;
-          S1.deg = 1;
-          cfd_status s = run_stage(B, S1, B->ops[gi].tab[0], n_iter, ws, st);
-          if (s != CFD_OK) return s;
-          // stage 2: D_i on the intermediate
-          LineParams S2 = P;
-          S2.in = ws.scratch;
-          S2.in_field = 0;
-          S2.in_box = (unsigned long long)E * N * N;
-          S2.out = out;
-          S2.out_mode = order == 0 ? 0 : 1;
-          S2.axis = ai;
-          S2.t1 = std::min(aj, ak);
-          S2.t2 = std::max(aj, ak);
-          for (int t = 0; t < 3; ++t) {
-            S2.in_dims[t] = S1.out_dims[t];
-            S2.in_start[t] = 0;
-            S2.out_dims[t] = N;
-            S2.out_start[t] = 0;
+          off.push_back((long long)used);
+          used += bufs * need;
+          ++j;
+        }
+        A.halo = hbase;
+        for (int pass = 0; pass <= n_iter; ++pass) {
+          const bool hp = pass < n_iter;
+          A.pass = pass;
+          A.ntask = 0;
+          for (size_t k = i; k < j; ++k) {
+            if (hp && (cyc[ts[k].axis] || ts[k].only == 1)) continue;
+            PencilTask t = ts[k];
+            const long long len = (long long)t.n1 * t.n2 * per * 2;
+            t.halo_in = off[k - i] + (bufs == 2 ? ((pass - 1) & 1) * len : 0);
+            t.halo_out = off[k - i] + (bufs == 2 ? (pass & 1) * len : 0);
+            A.task[A.ntask++] = t;
           }
-          S2.n1 = N;
-          S2.n2 = N;
-          S2.deg = 1;
-          s = run_stage(B, S2, B->ops[gi].tab[0], n_iter, ws, st);
+          cfd_status s = launch_pencils(A, hp, f32, N, half_width(ts[i]), W, st);
           if (s != CFD_OK) return s;
         }
+        i = j;
+      }
+      return CFD_OK;
+    };
+    auto pencils = [&](int axis, int deg, bool half) {
+      PencilTask t;
+      memset(&t, 0, sizeof(t));
+      t.tab = tabs + ptab_index(deg, axis, half);
+      t.axis = axis;
+      t.t1 = axis == 0 ? 1 : 0;
+      t.t2 = axis == 2 ? 1 : 2;
+      t.n1 = t.n2 = N;
+      t.out_op = -1;
+      t.sc_off = -1;
+      t.in_op = -1;
+      return t;
+    };
+    // outer axes that follow each inner axis, and their ops
+    std::vector<std::pair<int, int>> outer[3];  // [inner axis]: (outer axis, op slot)
+    for (int mi = 0; mi < 3; ++mi) {
+      const int o = slot(6 + mi);
+      if (o < 0) continue;
+      outer[kMixed[mi][1]].push_back({kMixed[mi][0], o});
+      if (!B->mixed_one_order) outer[kMixed[mi][0]].push_back({kMixed[mi][1], o});
+    }
+    std::vector<PencilTask> ts;
+    for (int bit = 0; bit < 6; ++bit) {
+      const int o = slot(bit), a = kAxisOfOp1[bit % 3];
+      if (o < 0 || (bit < 3 && f32 && !outer[a].empty())) continue;  // (computed with its FP64 copy below)
+      PencilTask t = pencils(a, bit < 3 ? 1 : 2, false);
+      t.out_op = o;
+      ts.push_back(t);
+    }
+    cfd_status s = run(ts, all, all_elems);
+    if (s != CFD_OK) return s;
+    bool written[9] = {};
+    for (int j = 0; j < 3; ++j) {
+      const int oj = slot(2 - j);  // op bit of d_j: x (box axis 2) is bit 0
+      const bool in_out = oj >= 0 && !f32;
+      const long long strip = 2ll * g * N * N * per, base = in_out ? 0 : n3 * per;
+      for (size_t k = 0; k < outer[j].size();) {
+        size_t n = std::min(outer[j].size() - k, (size_t)((region_elems - base) / strip));
+        if (n == 0) { set_error("banded path: scratch too small"); return CFD_ERR_ARG; }
+        ts.clear();
+        if (k == 0 && !in_out) {
+          PencilTask t = pencils(j, 1, false);
+          t.out_op = oj;
+          t.sc_off = 0;
+          ts.push_back(t);
+        }
+        for (size_t u = 0; u < n; ++u) {
+          PencilTask t = pencils(j, 1, false);
+          t.strip = outer[j][k + u].first == t.t1 ? 1 : 2;
+          (t.strip == 1 ? t.n1 : t.n2) = 2 * g;
+          t.sc_off = base + (long long)u * strip;
+          ts.push_back(t);
+        }
+        if ((s = run(ts, halo, halo_elems)) != CFD_OK) return s;
+        ts.clear();
+        for (size_t u = 0; u < n; ++u) {
+          const int op = outer[j][k + u].second;
+          PencilTask t = pencils(outer[j][k + u].first, 1, !B->mixed_one_order);
+          t.gather = 1;
+          t.in_op = in_out ? oj : -1;
+          t.strip_off = base + (long long)u * strip;
+          t.out_op = op;
+          t.accum = written[op];
+          written[op] = true;
+          ts.push_back(t);
+        }
+        if ((s = run(ts, halo, halo_elems)) != CFD_OK) return s;
+        k += n;
       }
     }
   }
@@ -466,6 +463,8 @@ void cfd_blocks_destroy(cfd_blocks_t B) {
   cudaFree(B->d_nvec);
   cudaFree(B->d_status);
   for (int *p : B->d_groups) cudaFree(p);
+  for (void *p : B->d_ptab) cudaFree(p);
+  cudaFree(B->d_lidx);
   for (void *p : B->d_dense_ptrs) cudaFree(p);
   if (B->dense_state && B->dense_free) B->dense_free(B->dense_state);
   cudaSetDevice(prev);
@@ -539,12 +538,6 @@ cfd_status cfd_blocks_bind(cfd_scheme_t scheme, int nblocks, const int *block_n,
   for (auto &kv : gm) {
     B->sizes.push_back(kv.first);
     B->groups.push_back(kv.second);
-    OpSet os;
-    memset(&os, 0, sizeof(os));
-    os.N = kv.first;
-    for (int d = 0; d < 2; ++d)
-      if (B->s[d].present) build_tables(B->s[d], kv.first, os.tab[d]);
-    B->ops.push_back(os);
     if (B->biased.present) {
       BiasedTables bt;
       build_biased_tables(B->biased, kv.first, ng, bt);
@@ -574,6 +567,35 @@ cfd_status cfd_blocks_bind(cfd_scheme_t scheme, int nblocks, const int *block_n,
       if (grp[k] != grp[0] + (int)k) consecutive = false;
     B->group_b0.push_back(consecutive ? grp[0] : -1);
   }
+  // FP64 banded tables: spacing equal in a group is folded into them
+  std::vector<int> lidx(nblocks);
+  for (size_t gi = 0; gi < B->groups.size(); ++gi) {
+    const std::vector<int> &grp = B->groups[gi];
+    for (size_t k = 0; k < grp.size(); ++k) lidx[grp[k]] = (int)k;
+    std::vector<PencilTab> tabs(9);
+    for (int box = 0; box < 3; ++box) {
+      const double h = B->dx[grp[0] * 3 + 2 - box];
+      bool equal = true;
+      for (int b : grp)
+        if (B->dx[b * 3 + 2 - box] != h) equal = false;
+      for (int d = 1; d <= 2; ++d) {
+        if (!B->s[d - 1].present) continue;
+        const ld scale = d == 1 ? 1.0L / h : 1.0L / ((ld)h * h);
+        for (int half = 0; half < (d == 1 ? 2 : 1); ++half) {
+          int same = -1;  // an axis with the same spacing has the same table
+          for (int pb = 0; pb < box; ++pb)
+            if (equal && B->dx[grp[0] * 3 + 2 - pb] == h && !tabs[ptab_index(d, pb, half != 0)].unscaled) same = pb;
+          PencilTab &T = tabs[ptab_index(d, box, half != 0)];
+          if (same >= 0) T = tabs[ptab_index(d, same, half != 0)];
+          else build_pencil_tab(B->s[d - 1], grp.empty() ? 0 : B->n[grp[0]], scale, !equal, half ? 0.5 : 1.0, T);
+        }
+      }
+    }
+    PencilTab *p = nullptr;
+    if ((s = upload(&p, tabs.data(), tabs.size())) != CFD_OK) return fail(s, nullptr);
+    B->d_ptab.push_back(p);
+  }
+  if ((s = upload(&B->d_lidx, lidx.data(), lidx.size())) != CFD_OK) return fail(s, nullptr);
   {
     std::vector<long long> exch((size_t)nblocks * 27);
     for (int b = 0; b < nblocks; ++b) {
@@ -638,14 +660,9 @@ cfd_status cfd_apply(cfd_blocks_t B, const void *fields, int nfields, unsigned o
   if (prec == CFD_FP64_BANDED) {
     size_t sc, ha;
     banded_workspace_sizes(B, nfields, op_mask, n_iter, &sc, &ha);
-    Workspace ws;
-    char *base = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
-    ws.scratch = sc ? (double *)base : nullptr;
-    base += align256(sc * 8);
-    ws.halo[0] = ha ? (double *)base : nullptr;
-    base += align256(ha * 8);
-    ws.halo[1] = ha ? (double *)base : nullptr;
-    return apply_banded(B, fields, nfields, op_mask, n_iter, out, ws, st);
+    double *scratch = (double *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
+    const size_t sc_elems = align256(sc * 8) / 8, ha_elems = 2 * align256(ha * 8) / 8;
+    return apply_banded(B, fields, nfields, op_mask, n_iter, out, scratch, sc_elems, scratch + sc_elems, ha_elems, st);
   }
   return dense_apply(B, fields, nfields, op_mask, prec, n_iter, out, work, work_bytes, st);
 }
@@ -715,9 +732,8 @@ size_t banded_closed_scratch_bytes(const cfd_blocks_s *B, int nf, unsigned mask)
 
 cfd_status apply_banded_closed(cfd_blocks_s *B, const void *fields, int nf, unsigned mask, void *out,
                                double *scratch, cudaStream_t st) {
-  Workspace ws;
-  ws.scratch = scratch;
-  return apply_banded(B, fields, nf, mask, 0, out, ws, st);
+  return apply_banded(B, fields, nf, mask, 0, out, scratch, banded_closed_scratch_bytes(B, nf, mask) / sizeof(double),
+                      nullptr, 0, st);
 }
 
 }  // namespace cfd

@@ -1597,7 +1597,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
 // One halo pass of the hybrid iteration along the stage's axis: the four rows of every pencil that the
 // neighbours read, from the pencils (first iterate) or with the previous iterate's halo columns.
 //   exact: four of 16 operator rows through the tensor cores (dense_exact.cuh).  256^3, 4 FP64 fields,
-//     six passes: HALO_NEW ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
+//     six passes: 0.95 ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
 //     coefficient and row where the digit split costs ~20 instructions per value for all rows;
 //   otherwise compensated FP32 on the CUDA cores (halo_rows.cu), whose cost does not depend on the form.
 static cfd_status halo_pass(DenseParams H, const DenseOp &op, const HaloRows &rows, bool exact, bool f32, int sms,
