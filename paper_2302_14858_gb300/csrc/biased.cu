@@ -506,87 +506,182 @@ cfd_status check_work(cfd_blocks_s *B, int nf, cfd_precision prec, int n_iter, v
   return CFD_OK;
 }
 
-// Upwind blend of the two biased derivatives of every axis (tensor-core path): one thread per
-// interior point of one block, looping over the fields (the shift is read once per point);
-// axes added in the order x, y, z, in the field precision (FP32 fields in FP32: GB300's FP64
-// pipe, not memory, bounded this kernel when FP32 values were widened to FP64).
-template <typename T, int NC>
+// Upwind blend of the biased derivatives of every axis (tensor-core path): one thread per V
+// consecutive interior points of one block (V values = 16 bytes where alignment allows), looping over the
+// fields (the shift is read once per point); axes added in the order x, y, z, in the field precision
+// (FP32 fields in FP32: GB300's FP64 pipe, not memory, bounded this kernel when FP32 values were widened
+// to FP64).  BOTH: tmp holds S+ and S- of every axis; otherwise the one the shift selects.
+template <typename T, int NC, int V, bool BOTH>
 __global__ void __launch_bounds__(256) k_advect_combine(const T *__restrict__ tmp, const T *__restrict__ beta, T *out,
                                  const int *__restrict__ blocks, const long long *__restrict__ extpre,
                                  const long long *__restrict__ intpre, int N_, int g, int nf, int out_nops,
                                  int out_opidx, int accum_all) {
+  struct alignas(V * sizeof(T)) Vec { T v[V]; };
   const int N = NC ? NC : N_;
   const int n3 = N * N * N;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   if (i >= n3) return;
   const int b = blocks[blockIdx.y];
   const int x = i % N, y = (i / N) % N, z = i / (N * N);
   const int E = N + 2 * g;
   const long long E3 = (long long)E * E * E;
   const T *bt = beta + 3 * extpre[b] + ((long long)(z + g) * E + (y + g)) * E + (x + g);
+  constexpr int S = BOTH ? 6 : 3;
   // the shift and, per axis, which biased derivative it takes: beta > 0 the right-biased one
   // (slot 2c+1), beta < 0 the left-biased one (slot 2c), beta = 0 none
-  T bv[3];
-  int slot[3];
+  Vec bv[3];
+  int slot[3][V];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    bv[c] = __ldg(bt + c * E3);
-    const int sg = sign_bits(bv[c]);
-    slot[c] = 2 * c + (sg == 1 ? 1 : 0);
-    if (sg == 0) bv[c] = T(0);  // a zero shift adds nothing (+0 times a finite derivative)
+    bv[c] = *reinterpret_cast<const Vec *>(bt + c * E3);
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      const int sg = sign_bits(bv[c].v[k]);
+      slot[c][k] = BOTH ? 2 * c + (sg == 1 ? 1 : 0) : c;
+      if (sg == 0) bv[c].v[k] = T(0);  // a zero shift adds nothing (+0 times a finite derivative)
+    }
   }
-  const T *tp = tmp + (long long)nf * 6 * intpre[b] + i;
+  const T *tp = tmp + (long long)nf * S * intpre[b] + i;
   T *o = out + (long long)nf * out_nops * intpre[b] + (long long)out_opidx * n3 + i;
   // fields in groups of QB, every load of a group issued before its first store
-  constexpr int QB = 4;
+  constexpr int QB = V > 1 ? 2 : 4;
   for (int q0 = 0; q0 < nf; q0 += QB) {
-    T dv[QB][3], prev[QB];
+    Vec dv[QB][3], prev[QB];
 #pragma unroll
     for (int u = 0; u < QB; ++u) {
-      prev[u] = T(0);
       if (q0 + u < nf) {
-        const T *tq = tp + (long long)(q0 + u) * 6 * n3;
+        const T *tq = tp + (long long)(q0 + u) * S * n3;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) dv[u][c] = __ldg(tq + (long long)slot[c] * n3);
-        if (accum_all) prev[u] = o[(long long)(q0 + u) * out_nops * n3];
+        for (int c = 0; c < 3; ++c) {
+          if constexpr (BOTH) {
+#pragma unroll
+            for (int k = 0; k < V; ++k) dv[u][c].v[k] = __ldg(tq + (long long)slot[c][k] * n3 + k);
+          } else {
+            dv[u][c] = *reinterpret_cast<const Vec *>(tq + (long long)c * n3);
+          }
+        }
+        if (accum_all) prev[u] = *reinterpret_cast<const Vec *>(o + (long long)(q0 + u) * out_nops * n3);
       }
     }
     // x, y, z as one FMA chain (three FP64-pipe operations per point and field for FP64 fields)
 #pragma unroll
     for (int u = 0; u < QB; ++u) {
       if (q0 + u >= nf) break;
-      T acc = accum_all ? fma(bv[0], dv[u][0], prev[u]) : bv[0] * dv[u][0];
-      acc = fma(bv[1], dv[u][1], acc);
-      acc = fma(bv[2], dv[u][2], acc);
-      o[(long long)(q0 + u) * out_nops * n3] = acc;
+      Vec acc;
+#pragma unroll
+      for (int k = 0; k < V; ++k) {
+        T a = accum_all ? fma(bv[0].v[k], dv[u][0].v[k], prev[u].v[k]) : bv[0].v[k] * dv[u][0].v[k];
+        a = fma(bv[1].v[k], dv[u][1].v[k], a);
+        acc.v[k] = fma(bv[2].v[k], dv[u][2].v[k], a);
+      }
+      *reinterpret_cast<Vec *>(o + (long long)(q0 + u) * out_nops * n3) = acc;
     }
+  }
+}
+
+// Signs of the shift as bits, per block (from word 3 intpre / 16) [axis x, y, z][pencil]: bit k of a word is set where point k of the
+// pencil takes the right-biased derivative (beta > 0).  One warp per 32 pencils of a block and axis; along
+// y and z a lane walks its pencil (consecutive x positions), along x the lanes take consecutive points.
+template <typename T>
+__global__ void __launch_bounds__(256) k_upwind_signs(const T *__restrict__ beta, const int *__restrict__ blocks,
+                                                      const long long *__restrict__ extpre,
+                                                      const long long *__restrict__ intpre, int N, int g,
+                                                      uint32_t *__restrict__ words) {
+  const int b = blocks[blockIdx.y], c = blockIdx.z, E = N + 2 * g;
+  const int lane = threadIdx.x & 31, p0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+  if (p0 >= N * N) return;
+  const T *bt = beta + 3 * extpre[b] + (long long)c * E * E * E;
+  uint32_t *w = words + 3 * (intpre[b] >> 4) + c * N * N;
+  if (c == 0) {  // x: rows; 32 / N rows per load
+    const int per = 32 / N;
+    for (int r0 = 0; r0 < 32; r0 += 8 * per) {
+      T v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int p = p0 + min(r0 + u * per, 31) + lane / N, k = lane % N;
+        v[u] = r0 + u * per < 32 ? __ldg(bt + ((long long)(p / N + g) * E + (p % N + g)) * E + k + g) : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t m = __ballot_sync(0xffffffffu, sign_bits(v[u]) == 1);
+        const int r = r0 + u * per;
+        if (r < 32 && lane % N == 0) w[p0 + r + lane / N] = N == 32 ? m : (m >> (lane / N * N)) & ((1u << N) - 1u);
+      }
+    }
+  } else {       // y: pencils (z, x); z: pencils (y, x)
+    const int p = p0 + lane, t = p / N, x = p % N;
+    const T *s = bt + (c == 1 ? (long long)(t + g) * E * E + (long long)g * E : (long long)g * E * E + (long long)(t + g) * E) + x + g;
+    const long long st = c == 1 ? E : (long long)E * E;
+    uint32_t m = 0;
+    for (int k0 = 0; k0 < N; k0 += 16) {
+      T v[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = __ldg(s + (k0 + k) * st);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) m |= (sign_bits(v[k]) == 1 ? 1u : 0u) << (k0 + k);
+    }
+    w[p] = m;
   }
 }
 
 }  // namespace
 
-cfd_status advect_combine(cfd_blocks_s *B, const void *tmp6, const void *beta, int nf, void *out, int out_nops,
-                          int out_opidx, bool accum_all, cudaStream_t st) {
+cfd_status advect_combine(cfd_blocks_s *B, const void *tmp, bool both, const void *beta, int nf, void *out,
+                          int out_nops, int out_opidx, bool accum_all, cudaStream_t st) {
   for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
     const int N = B->sizes[gi];
     const int n3 = N * N * N;
-    dim3 grid((unsigned)((n3 + 255) / 256), (unsigned)B->groups[gi].size());
     launch_begin(KF_BIASED, st);
-    auto go = [&](auto tag, auto nc) {
+    auto go = [&](auto tag, auto nc, auto vc, auto bc) {
       using T = decltype(tag);
-      k_advect_combine<T, decltype(nc)::value><<<grid, 256, 0, st>>>(
-          static_cast<const T *>(tmp6), static_cast<const T *>(beta), static_cast<T *>(out), B->d_groups[gi],
+      constexpr int V = decltype(vc)::value;
+      dim3 grid((unsigned)((n3 / V + 255) / 256), (unsigned)B->groups[gi].size());
+      k_advect_combine<T, decltype(nc)::value, V, decltype(bc)::value><<<grid, 256, 0, st>>>(
+          static_cast<const T *>(tmp), static_cast<const T *>(beta), static_cast<T *>(out), B->d_groups[gi],
           B->d_extpre, B->d_intpre, N, B->ng, nf, out_nops, out_opidx, accum_all);
     };
+    // 16-byte vectors: N is a multiple of 8, so is every block's offset in a multiple of N^3; the shift needs
+    // an even (FP32: fourfold) ghost width, and every buffer its alignment
+    const int vw = B->dtype == CFD_F32 ? 4 : 2;
+    bool vec = !both && B->ng % vw == 0;
+    for (const void *p : {tmp, beta, (const void *)out})
+      if ((uintptr_t)p & 15) vec = false;
+    using std::integral_constant;
     auto by_n = [&](auto tag) {
-      if (N == 32) go(tag, std::integral_constant<int, 32>());
-      else if (N == 16) go(tag, std::integral_constant<int, 16>());
-      else go(tag, std::integral_constant<int, 0>());
+      using T = decltype(tag);
+      constexpr int VW = 16 / sizeof(T);
+      auto by_v = [&](auto nc) {
+        if (both) go(tag, nc, integral_constant<int, 1>(), integral_constant<bool, true>());
+        else if (vec) go(tag, nc, integral_constant<int, VW>(), integral_constant<bool, false>());
+        else go(tag, nc, integral_constant<int, 1>(), integral_constant<bool, false>());
+      };
+      if (N == 32) by_v(integral_constant<int, 32>());
+      else if (N == 16) by_v(integral_constant<int, 16>());
+      else by_v(integral_constant<int, 0>());
     };
     if (B->dtype == CFD_F32) by_n(float());
     else by_n(double());
     launch_end(KF_BIASED, st);
     cfd_status s = cuda_fail(cudaGetLastError(), "k_advect_combine launch");
+    if (s != CFD_OK) return s;
+  }
+  return CFD_OK;
+}
+
+cfd_status upwind_signs(cfd_blocks_s *B, const void *beta, uint32_t *words, cudaStream_t st) {
+  for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
+    const int N = B->sizes[gi];
+    if (N < 16) { set_error("upwind signs: blocks of 16^3 or 32^3"); return CFD_ERR_UNSUPPORTED; }
+    const dim3 grid((unsigned)(N * N / 256), (unsigned)B->groups[gi].size(), 3);
+    launch_begin(KF_BIASED, st);
+    if (B->dtype == CFD_F32)
+      k_upwind_signs<float><<<grid, 256, 0, st>>>(static_cast<const float *>(beta), B->d_groups[gi], B->d_extpre,
+                                                  B->d_intpre, N, B->ng, words);
+    else
+      k_upwind_signs<double><<<grid, 256, 0, st>>>(static_cast<const double *>(beta), B->d_groups[gi], B->d_extpre,
+                                                   B->d_intpre, N, B->ng, words);
+    launch_end(KF_BIASED, st);
+    cfd_status s = cuda_fail(cudaGetLastError(), "k_upwind_signs launch");
     if (s != CFD_OK) return s;
   }
   return CFD_OK;

@@ -130,10 +130,13 @@ void launch_end(int family, cudaStream_t st);
 cfd_status advect_accumulate(cfd_blocks_s *B, const void *fields, int nf, const void *beta, void *out, int out_nops,
                              int out_opidx, cfd_precision prec, int n_iter, void *work, size_t work_bytes,
                              cudaStream_t st);
-// biased.cu: out slot = (accum_all ? out : 0) + sum_{i=x,y,z} beta^i (beta^i > 0 ? T[2i+1] : T[2i]),
-// T = [block][field][6][N^3] (both biased derivatives of every axis)
-cfd_status advect_combine(cfd_blocks_s *B, const void *tmp6, const void *beta, int nf, void *out, int out_nops,
-                          int out_opidx, bool accum_all, cudaStream_t st);
+// biased.cu: out slot = (accum_all ? out : 0) + sum_{i=x,y,z} beta^i d_i, d_i the biased derivative the sign
+// of beta^i selects: tmp = [block][field][3][N^3] (the selected ones), or with `both`
+// [block][field][6][N^3] (S+ and S- of every axis)
+cfd_status advect_combine(cfd_blocks_s *B, const void *tmp, bool both, const void *beta, int nf, void *out,
+                          int out_nops, int out_opidx, bool accum_all, cudaStream_t st);
+// biased.cu: the signs of the shift for DenseParams::upwind (blocks of 16^3 and more: 3 / 16 words per point)
+cfd_status upwind_signs(cfd_blocks_s *B, const void *beta, uint32_t *words, cudaStream_t st);
 // dense_tc.cu: the biased operators on the tensor cores
 size_t dense_biased_workspace(const cfd_blocks_s *B, int nf, int n_iter, bool advect);
 cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void *beta, const int *axes, int naxes,

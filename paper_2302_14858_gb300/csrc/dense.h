@@ -41,6 +41,10 @@ struct DenseParams {
   // exact form: halo_in / halo_out are [block][field][side: row 1, row N-2][pencil][halo_nd], halo_nd
   // the degrees kept (2, or 1: the one of halo_deg_mask)
   int halo_nd;
+  // exact form: not null in an upwinded stage (segments S+ and S-, one output): per block, axis x, y, z
+  // and interior pencil a word whose bit k says that point k takes the right-biased derivative (block b
+  // starts at word 3 intpre[b] / 16)
+  const uint32_t *upwind;
   int xrow;                  // x-axis stage with 16-byte aligned pencil rows: chunked row copies
   int xvec;                  // x-axis stage with a 16-byte aligned output: vector stores
   // Consecutive block ids (blocks[lb] = b0 + lb): offsets follow from the job index
@@ -51,6 +55,7 @@ struct DenseParams {
   // bytes along x), 2 y columns (box [t1][y][x]), 3 z columns (box [z][t1][x])
   int tma_kind, tma_boxes, tma_bytes, tma_zstep;  // zstep: z planes per job in the tensor map
   int nstg, stg_bytes;       // exact form: staging buffers (1 or 2) and bytes of one
+  int halo_stg;              // exact form, TMA: offset of a tile's halo values in its staging buffer
   // exact form, x stages: bytes of an epilogue warp's output box ([32 pencils][8 values]; 0: stores
   // straight to memory) and the output as a tensor of N-value rows
   int out_box_bytes;
@@ -84,6 +89,7 @@ void halo_rows_from(const std::vector<long double> &M, int cols, HaloRows &R);
 // P.halo_in, to the neighbours' previous iterate), written to P.halo_out.
 cfd_status halo_rows_launch(const DenseParams &P, const HaloRows &R, bool f32_in, cudaStream_t st);
 
+cfd_status dense_exact_upwind(const DenseParams &P, bool f32, unsigned grid, cudaStream_t st);
 cfd_status dense_exact_halo(const DenseParams &P, bool f32_in, unsigned grid, cudaStream_t st);
 // One launch of the exact form (dense_exact.cuh) for blocks of 16^3 / 32^3.
 cfd_status dense_exact_launch16(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);

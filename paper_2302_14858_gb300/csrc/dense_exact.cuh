@@ -47,6 +47,7 @@ constexpr int kXThreads = kXProd + kXEpiWarps * 32 + 128;
 constexpr int kXUnit = 8;                // operator rows of an epilogue unit
 constexpr int kXRowBytes = 64;           // inner bytes of a staged box of x rows
 constexpr int kXEtau = 8;                // pencil-scale ring (tiles)
+constexpr int16_t kBadTau16 = 32767;     // kBadTau in the ring (scales are -1022 .. 1024)
 
 // ---------------------------------------------------------------- digits
 
@@ -147,14 +148,16 @@ __device__ __forceinline__ void release_levels(uint32_t t_empty) {
 // The levels of one output as a 64-bit integer in units of 2^-43 sigma tau: t1 = x0 2^10 + x1 exact
 // (|x0| < 2^21 - 2^14, see the row scale in exact_image), the two low levels joined in FP32 (their
 // sum rounds at 2^-24 of a level that is itself 2^-20 of the result's scale).
-__device__ __forceinline__ long long exact_y(const uint32_t (&acc)[kSl][8], int c) {
+template <int C>
+__device__ __forceinline__ long long exact_y(const uint32_t (&acc)[kSl][C], int c) {
   const int t1 = __float2int_rn(__uint_as_float(acc[0][c])) * 1024 + __float2int_rn(__uint_as_float(acc[1][c]));
   const int t2 = __float2int_rn(fmaf(__uint_as_float(acc[2][c]), 32.0f, __uint_as_float(acc[3][c]) * 0.03125f));
   return ((long long)t1 << 15) + (long long)t2;
 }
 constexpr int kYUnit = 43, kFUnit = 48;  // result exponents: 2^(rowexp + etau - unit)
 // FP32 outputs: the levels in FP32 by Horner's rule, units of 2^-48 sigma tau
-__device__ __forceinline__ float exact_f(const uint32_t (&acc)[kSl][8], int c) {
+template <int C>
+__device__ __forceinline__ float exact_f(const uint32_t (&acc)[kSl][C], int c) {
   float y = __uint_as_float(acc[0][c]);
 #pragma unroll
   for (int k = 1; k < kSl; ++k) y = fmaf(y, 1024.0f, __uint_as_float(acc[k][c]));
@@ -237,6 +240,68 @@ __device__ __noinline__ void rows_any(uint32_t taddr, uint32_t lev, int etau, co
   }
 }
 
+// 8 rows of an upwinded stage: of the two biased derivatives of a point only the one the shift selects
+// (bit of `word`: the right-biased one, the second segment, `seg1` TMEM columns on) is rebuilt and stored.
+// The choice is made on the accumulators, before the conversion to FP64: half the conversions and half
+// the stores of writing both (256^3, 4 fields, three stages: UPWIND_NOTE).  SAFE: as rows_fast.
+template <typename TO, bool ROW, bool SAFE>
+__device__ __forceinline__ void rows_upwind(uint32_t taddr, uint32_t lev, uint32_t seg1, int etau, const int *rowexp,
+                                            int rstep, TO *fin, long long fin_stride, bool wf, uint32_t word,
+                                            uint32_t t_empty, unsigned char *box) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int c0 = 0; c0 < 8; c0 += 4) {
+    uint32_t a[kSl][4], b[kSl][4];
+#pragma unroll
+    for (int k = 0; k < kSl; ++k) {
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(a[k][0]), "=r"(a[k][1]), "=r"(a[k][2]), "=r"(a[k][3])
+                   : "r"(taddr + (uint32_t)k * lev + (uint32_t)c0));
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                   : "=r"(b[k][0]), "=r"(b[k][1]), "=r"(b[k][2]), "=r"(b[k][3])
+                   : "r"(taddr + (uint32_t)k * lev + seg1 + (uint32_t)c0));
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    if (c0 == 4) release_levels(t_empty);
+    const int4 r0 = *reinterpret_cast<const int4 *>(rowexp + c0), r1 = *reinterpret_cast<const int4 *>(rowexp + rstep + c0);
+    const int x0[4] = {r0.x, r0.y, r0.z, r0.w}, x1[4] = {r1.x, r1.y, r1.z, r1.w};
+    TO o[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool right = (word >> (c0 + u)) & 1u;
+#pragma unroll
+      for (int k = 0; k < kSl; ++k) a[k][u] = right ? b[k][u] : a[k][u];
+      const int ex = (right ? x1[u] : x0[u]) + etau;
+      if constexpr (SAFE) {
+        if constexpr (sizeof(TO) == 8) {
+          const double d = __ll2double_rn(exact_y(a, u));
+          const int hi = __double2hiint(d), lo = __double2loint(d);
+          o[u] = __hiloint2double(hi ? hi + ((ex - kYUnit) << 20) : 0, lo);
+        } else {
+          o[u] = exact_f(a, u) * __int_as_float((ex - kFUnit + 127) << 23);
+        }
+      } else {
+        const bool bad = etau == kBadTau;
+        if constexpr (sizeof(TO) == 8) o[u] = scaled_double<true>(__ll2double_rn(exact_y(a, u)), ex - kYUnit, bad);
+        else o[u] = bad ? __int_as_float(0x7FC00000) : scale_pow2(exact_f(a, u), ex - kFUnit);
+      }
+      if constexpr (!ROW) {
+        if (wf) fin[(c0 + u) * fin_stride] = o[u];
+      }
+    }
+    if constexpr (ROW) {
+      if constexpr (sizeof(TO) == 8) {
+        const int sw = (lane >> 1) & 3;
+        *reinterpret_cast<double2 *>(box + lane * 64 + (((c0 / 2) ^ sw) << 4)) = make_double2(o[0], o[1]);
+        *reinterpret_cast<double2 *>(box + lane * 64 + (((c0 / 2 + 1) ^ sw) << 4)) = make_double2(o[2], o[3]);
+      } else {
+        *reinterpret_cast<float4 *>(box + lane * 32 + (((c0 / 4) ^ ((lane >> 2) & 1)) << 4)) =
+            make_float4(o[0], o[1], o[2], o[3]);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------- the kernel
 
 // N: block size (16, 32).  AXIS 0, 1, 2: pencils along z, y, x with ghost width 4 (every stride and
@@ -246,10 +311,13 @@ __device__ __noinline__ void rows_any(uint32_t taddr, uint32_t lev, int etau, co
 // zero padding), whose outputs are the values the neighbours read at their k^c nodes.  It costs the
 // producers' share of a stage, against ~11 FP32 operations per coefficient and row in compensated
 // FP32 on the CUDA cores (256^3, 4 fields: see halo_pass in dense_tc.cu).
-template <typename TI, typename TO, int N, int AXIS, bool ITER, bool HALO>
+// UPWIND: the two biased operators of an axis, one output (rows_upwind).  (An instantiation of its own:
+// as a branch of the plain epilogue it cost that one 4 %.)
+enum ExactMode { kPlain = 0, kHaloRows = 1, kUpwind = 2 };
+template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE>
 __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_constant__ DenseParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  constexpr bool GEN = AXIS == 3;
+  constexpr bool GEN = AXIS == 3, HALO = MODE == kHaloRows, UPWIND = MODE == kUpwind;
   constexpr int KP = N == 32 ? 48 : 32, NCH = KP / 8;
   constexpr int ES = sizeof(TI);
   constexpr int SLICE = kTile * KP * 2, A_BYTES = kSl * SLICE;
@@ -267,7 +335,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   unsigned char *stg0 = smem + stg_off;
   unsigned char *s_out = stg0 + nstg * stg_bytes;  // x stages: one output box per epilogue warp
   int *s_rowexp = reinterpret_cast<int *>(s_out + P.out_box_bytes * kXEpiWarps);
-  int *s_etau = s_rowexp + 64;
+  int16_t *s_etau = reinterpret_cast<int16_t *>(s_rowexp + 64);
   uint64_t *bars = reinterpret_cast<uint64_t *>(s_etau + kXEtau * kTile);
   uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + 28);
   const uint32_t bar0 = smem_u32(bars);
@@ -294,9 +362,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       mbar_init(s_full(i), kind ? 1 : kXProd);
       mbar_init(s_empty(i), kXProdWarps);
     }
-    // warps that read a TMEM buffer: all, with 16 rows (N = 16, one operator) half of them in turn, in
-    // a halo pass one per lane quadrant in turn
-    const int readers = HALO ? kXEpiWarps / 4 : (R < 32 ? kXEpiWarps / 2 : kXEpiWarps);
+    // warps that read a TMEM buffer: all, where a tile has two units of 8 rows (N = 16 with one operator
+    // or upwinded) half of them in turn, in a halo pass one per lane quadrant in turn
+    const int readers = HALO ? kXEpiWarps / 4 : kXEpiWarps / 4 * min(4, (UPWIND ? 1 : P.nseg[0]) * (N / kXUnit));
     for (int i = 0; i < 4; ++i) { mbar_init(t_full(i), 1); mbar_init(t_empty(i), readers); }
     for (int i = 0; i < kXEtau; ++i) mbar_init(meta_full(i), kXProdWarps);
     mbar_init(drain, 1);
@@ -404,48 +472,26 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     // The neighbours' previous iterate at k^c, as columns E + m of the pencil: m = 2d from the lower
     // neighbour's row N-2 (side 1), m = 2d + 1 from the upper neighbour's row 1 (side 0), degree slot d.
     // Layout [block][field][side][pencil][halo_nd]: a stage of one degree holds (and moves) only its own.
-    // The neighbour of tile t + 2 is looked up, and the values of tile t + 1 are loaded, while tile t is
-    // split: neither load is waited for (T stages at 256^3 with the lookup in the chain: 0.34 ms).
-    auto halo_block = [&](int tile, int up) -> int {
-      if (tile >= tr.end) return -1;
-      const TileCoord c = tile_coord(P, tile, pl);
-      const int sg = up ? 1 : -1;
-      return !c.valid ? -1 : P.nbr[c.b * 26 + dir_index_dev(axis == 0 ? sg : 0, axis == 1 ? sg : 0, axis == 2 ? sg : 0)];
-    };
+    // With TMA the copies of a tile bring its two runs of 128 pencils behind the staged pencils; loaded by
+    // the producers themselves, a tile ahead, they cost the T stages at 256^3 a quarter (0.31 against
+    // HALO_T ms: the index arithmetic sat on the producers' critical path).
     const int np = P.n1 * P.n2;
-    auto halo = [&](int tile, int nb, int m) -> TI {
-      const int d = m >> 1, up = m & 1;
-      if (nb < 0 || !((P.halo_deg_mask >> d) & 1)) return TI(0);
-      const int job = fdiv(tile, P.inv_tpj), q = job - fdiv(job, P.inv_nf) * P.nf;
-      const long long hp = (((long long)nb * P.nf + q) * 2 + (up ? 0 : 1)) * np + tile_pencil(P, tile, pl);
-      return TI(P.halo_in[hp * P.halo_nd + (P.halo_nd == 2 ? d : 0)]);
+    auto halo = [&](const unsigned char *st, int tile, int m) -> TI {
+      const int d = m >> 1, up = m & 1, dd = P.halo_nd == 2 ? d : 0;
+      if (!((P.halo_deg_mask >> d) & 1)) return TI(0);
+      if (kind) return TI(reinterpret_cast<const double *>(st + P.halo_stg)[(up * kTile + pl) * P.halo_nd + dd]);
+      const TileCoord c = tile_coord(P, tile, pl);
+      if (!c.valid) return TI(0);
+      const int sg = up ? 1 : -1;
+      const int nb = P.nbr[c.b * 26 + dir_index_dev(axis == 0 ? sg : 0, axis == 1 ? sg : 0, axis == 2 ? sg : 0)];
+      const long long hp = (((long long)nb * P.nf + c.q) * 2 + (up ? 0 : 1)) * np + tile_pencil(P, tile, pl);
+      return TI(P.halo_in[hp * P.halo_nd + dd]);
     };
     constexpr int NFULL = GEN ? (NCH + 1) / 2 : N / 16;          // whole chunks of this lane
     constexpr int NV = NFULL * 8 + (GEN ? 0 : 4 + (ITER ? 2 : 0));  // values of this lane
     if (!kind)
       for (int k = 0, t = tr.first; k < nstg && t < tr.end; ++k, t += tr.step) prefetch(t, k);
-    TI hq[4] = {TI(0), TI(0), TI(0), TI(0)};
-    int nb[2] = {-1, -1};  // lower and upper neighbour of the next tile to load
-    auto load_halo = [&](int tile) {
-      if constexpr (ITER) {
-        const int lo = nb[0], hi = nb[1];
-        nb[0] = halo_block(tile + tr.step, 0);
-        nb[1] = halo_block(tile + tr.step, 1);
-        if constexpr (GEN) {
-#pragma unroll
-          for (int m = 0; m < 4; ++m) hq[m] = halo(tile, m & 1 ? hi : lo, m);
-        } else {  // the two lanes of a pencil take one degree slot each
-          hq[0] = halo(tile, lo, 2 * half);
-          hq[1] = halo(tile, hi, 2 * half + 1);
-        }
-      }
-    };
-    if (ITER) {
-      nb[0] = halo_block(tr.first, 0);
-      nb[1] = halo_block(tr.first, 1);
-    }
     int it = 0;
-    if (tr.first < tr.end) load_halo(tr.first);
     for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
       const int buf = it & 1, sb = nstg == 2 ? it & 1 : 0, su = nstg == 2 ? it >> 1 : it;
       if (!wait(s_full(sb), (uint32_t)(su & 1))) { failed = true; break; }
@@ -460,14 +506,17 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
             const int j = (half + 2 * h) * 8 + k;
             TI x = TI(0);
             if (valid && j < E) x = *reinterpret_cast<const TI *>(st + stg_byte(pl, j));
-            else if (ITER && valid) x = j == E ? hq[0] : (j == E + 1 ? hq[1] : (j == E + 2 ? hq[2] : (j == E + 3 ? hq[3] : TI(0))));
+            else if (ITER && valid && j < E + 4) x = halo(st, tile, j - E);
             v[h * 8 + k] = x;
           }
       } else {
 #pragma unroll
         for (int h = 0; h < NFULL; ++h) load(st, (half + 2 * h) * 8, 8, v + h * 8);
         load(st, N + 4 * half, 4, v + NFULL * 8);
-        if constexpr (ITER) { v[NFULL * 8 + 4] = hq[0]; v[NFULL * 8 + 5] = hq[1]; }
+        if constexpr (ITER) {  // the two lanes of a pencil take one degree slot each
+          v[NFULL * 8 + 4] = halo(st, tile, 2 * half);
+          v[NFULL * 8 + 5] = halo(st, tile, 2 * half + 1);
+        }
         if (!kind && !tile_coord(P, tile, pl).valid) {
 #pragma unroll
           for (int k = 0; k < NV; ++k) v[k] = TI(0);
@@ -478,7 +527,6 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       for (int k = 0; k < NV; ++k) am = max(am, abs_word(v[k]));
       am = max(am, __shfl_xor_sync(0xffffffffu, am, 16));  // also: every lane has read its staged values
       if (lane == 0) mbar_arrive(s_empty(sb));
-      if (ITER && tile + tr.step < tr.end) load_halo(tile + tr.step);
       if (!kind && tile + nstg * tr.step < tr.end) {
         if (!wait(s_empty(sb), (uint32_t)(su & 1))) { failed = true; break; }
         prefetch(tile + nstg * tr.step, sb);
@@ -487,7 +535,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       // a NaN or an infinity anywhere in the pencil: every output of the pencil is NaN (the epilogue
       // sees kBadTau); its digits are written as zeros
       const bool bad = emax >= nonfinite_exp(TI(0));
-      const int etau = bad ? kBadTau : tau_exp(emax, TI(0));
+      const int etau = bad ? kBadTau16 : tau_exp(emax, TI(0));
       if (emax < 64) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) v[k] = lift64(v[k]);
@@ -497,7 +545,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       const int C = split_base(emax, TI(0));
       // A[buf] must be free: the MMAs of its previous use have completed
       if (it >= 2 && !wait(a_empty(buf), (uint32_t)(((it >> 1) - 1) & 1))) { failed = true; break; }
-      if (half == 0) s_etau[(it & (kXEtau - 1)) * kTile + pl] = etau;
+      if (half == 0) s_etau[(it & (kXEtau - 1)) * kTile + pl] = (int16_t)etau;
       // canonical K-major rows, no swizzle: [row / 8][chunk][row % 8][8]
       unsigned char *row = sA + buf * A_BYTES + (pl >> 3) * (NCH * 128) + (pl & 7) * 16;
 #pragma unroll
@@ -550,7 +598,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
         if ((it & 3) != ew) continue;
         const TileCoord c = tile_coord(P, tile, pl);
         if (!wait(meta_full(it & (kXEtau - 1)), (uint32_t)((it / kXEtau) & 1))) { failed = true; break; }
-        const int etau = s_etau[(it & (kXEtau - 1)) * kTile + pl];
+        const int etau16 = s_etau[(it & (kXEtau - 1)) * kTile + pl], etau = etau16 == kBadTau16 ? kBadTau : etau16;
         if (!wait(t_full(ew), (uint32_t)((it >> 2) & 1))) { failed = true; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         uint32_t acc[kSl][8];
@@ -573,7 +621,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
         }
       }
     } else {
-    const int units = P.nseg[0] * UPS;
+    const int units = (UPWIND ? 1 : P.nseg[0]) * UPS;
     const bool rows_out = axis == 2 && P.out_box_bytes != 0;
     unsigned char *box = s_out + (warp - kXProdWarps) * P.out_box_bytes;
     int it = 0;
@@ -608,13 +656,55 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
         }
       }
       if (!wait(meta_full(it & (kXEtau - 1)), (uint32_t)((it / kXEtau) & 1))) { failed = true; break; }
-      const int etau = s_etau[(it & (kXEtau - 1)) * kTile + pl];
+      const int etau16 = s_etau[(it & (kXEtau - 1)) * kTile + pl], etau = etau16 == kBadTau16 ? kBadTau : etau16;
       const bool bad = etau == kBadTau;
       const bool safe = !bad && etau + rlo >= kLo && etau + rhi <= kHi;
       const int tb = it & (nbuf - 1), tu = nbuf == 2 ? it >> 1 : it >> 2;
       if (!wait(t_full(tb), (uint32_t)(tu & 1))) { failed = true; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t tbase = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(tb * buf_cols);
+      // one TMA store of this warp's output box (its previous store has read it, see box_free)
+      auto box_free = [&]() {
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        __syncwarp();
+      };
+      auto box_store = [&](int op, int o) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          const int job = c.lb * P.nf + c.q;
+          const int row = (job * P.nops + op) * N * N + tile_pencil(P, tile, quad * 32);
+          asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                           reinterpret_cast<uint64_t>(&P.tmap_out)),
+                       "r"(o), "r"(row), "r"(smem_u32(box))
+                       : "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+      };
+      if constexpr (UPWIND) {
+        // the shift's signs along this pencil, one bit per point
+        const uint32_t signs =
+            interior ? __ldg(P.upwind + 3 * ((P.contig ? P.int0 + (long long)c.lb * n3 : P.intpre[c.b]) >> 4) +
+                             (2 - axis) * N * N + tile_pencil(P, tile, pl))
+                     : 0u;
+#pragma unroll 1
+        for (int u = u0; u < units; u += 4) {
+          const int o = u * kXUnit;
+          TO *f0 = fb + (long long)P.seg_op[0][0] * n3 + o * f_ax;
+          const uint32_t ta = tbase + (uint32_t)o, rel = u + 4 >= units ? t_empty(tb) : 0u;
+          const uint32_t w = signs >> o;
+          const bool all = __all_sync(0xffffffffu, safe && interior);
+          if (all && axis == 2 && rows_out) {
+            box_free();
+            rows_upwind<TO, true, true>(ta, R, N, etau, s_rowexp + o, N, f0, 1, true, w, rel, box);
+            box_store(P.seg_op[0][0], o);
+          } else if (all) {
+            rows_upwind<TO, false, true>(ta, R, N, etau, s_rowexp + o, N, f0, f_ax, true, w, rel, nullptr);
+          } else {
+            rows_upwind<TO, false, false>(ta, R, N, etau, s_rowexp + o, N, f0, f_ax, interior, w, rel, nullptr);
+          }
+        }
+      } else {
 #pragma unroll 1
       for (int u = u0; u < units; u += 4) {
         const int sg = u >= UPS ? 1 : 0, o = (u - sg * UPS) * kXUnit;
@@ -628,21 +718,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
         // warp-uniform choices: tcgen05.ld is a warp-wide instruction
         const bool all_f = __all_sync(0xffffffffu, safe && wf), any_s = __any_sync(0xffffffffu, ws);
         if (axis == 2 && rows_out && all_f) {
-          // the box's previous store must have read it
-          if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-          __syncwarp();
+          box_free();
           rows_fast<TO, true, true, false>(ta, R, etau, rexp, f0, 1, nullptr, 0, 0, 0, rel, box);
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) {
-            const int job = c.lb * P.nf + c.q;
-            const int row = (job * P.nops + P.seg_op[0][sg]) * N * N + tile_pencil(P, tile, quad * 32);
-            asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
-                             reinterpret_cast<uint64_t>(&P.tmap_out)),
-                         "r"(o), "r"(row), "r"(smem_u32(box))
-                         : "memory");
-            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-          }
+          box_store(P.seg_op[0][sg], o);
         } else if (all_f && !any_s) {
           rows_fast<TO, false, true, false>(ta, R, etau, rexp, f0, f_ax, nullptr, 0, 0, 0, rel, nullptr);
         } else {
@@ -655,6 +733,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
             rows_any<TO>(ta, R, etau, rexp, f0, f_ax, s0, c_ax, gx, gy, wf, ws, rel);
         }
       }
+    }
     }
     // the output boxes must have been read before the CTA leaves
     if (rows_out && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -703,10 +782,29 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       int it = 0;
       for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
         const int sb = nstg == 2 ? it & 1 : 0, su = nstg == 2 ? it >> 1 : it;
+        const int job = fdiv(tile, P.inv_tpj), tj = tile - job * P.tiles_per_job, t1_0 = tj * (kTile / N);
+        int nb[2] = {0, 0}, q = 0;
+        if constexpr (ITER) {  // (looked up before the wait for the staging buffer)
+          const int lb = fdiv(job, P.inv_nf), b = P.contig ? P.b0 + lb : P.blocks[lb];
+          q = job - lb * P.nf;
+          nb[0] = __ldg(P.nbr + b * 26 + dir_index_dev(axis == 0 ? -1 : 0, axis == 1 ? -1 : 0, axis == 2 ? -1 : 0));
+          nb[1] = __ldg(P.nbr + b * 26 + dir_index_dev(axis == 0 ? 1 : 0, axis == 1 ? 1 : 0, axis == 2 ? 1 : 0));
+        }
         if (su > 0 && !mbar_wait_bounded(s_empty(sb), (uint32_t)((su - 1) & 1), WL)) { failed = true; break; }
-        const int job = fdiv(tile, P.inv_tpj), t1_0 = (tile - job * P.tiles_per_job) * (kTile / N);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(s_full(sb)), "r"(P.tma_bytes)
                      : "memory");
+        if constexpr (ITER) {
+          const int np = P.n1 * P.n2, bytes = kTile * P.halo_nd * 8;
+#pragma unroll
+          for (int up = 0; up < 2; ++up) {
+            const double *src = P.halo_in + ((((long long)nb[up] * P.nf + q) * 2 + (up ? 0 : 1)) * np + tj * kTile) * P.halo_nd;
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    smem_u32(stg0) + (uint32_t)(sb * stg_bytes + P.halo_stg + up * bytes)),
+                "l"(src), "r"(bytes), "r"(s_full(sb))
+                : "memory");
+          }
+        }
         const int cz = P.in_start[0] + job * P.tma_zstep + (axis == 0 ? 0 : t1_0);
         const int cy = P.in_start[1] + (axis == 0 ? t1_0 : 0);
         for (int bx = 0; bx < P.tma_boxes; ++bx) {

@@ -18,16 +18,21 @@ size_t plan_smem(DenseParams &P) {
   constexpr int KP = N == 32 ? 48 : 32;
   const int E = N + 2 * P.g;
   const size_t fixed = ((2 * (size_t)kSl * kTile * KP * 2 + (size_t)kSl * P.rows * KP * 2 + 1023) & ~(size_t)1023) +
-                       (64 + kXEtau * kTile) * 4 + 28 * 8 + 16;
+                       64 * 4 + kXEtau * kTile * 2 + 28 * 8 + 16;
   const size_t rows = P.axis == 2 ? (size_t)((E * (int)sizeof(TI) + kXRowBytes - 1) / kXRowBytes) * kTile * kXRowBytes
                                   : (size_t)E * kTile * sizeof(TI);
   P.stg_bytes = (int)((rows + 1023) & ~(size_t)1023);
+  if (P.halo_in && P.tma_kind) {  // both sides' halo values of a tile, by bulk copies into the same buffer
+    P.halo_stg = P.stg_bytes;
+    P.stg_bytes += 2 * kTile * P.halo_nd * 8;
+    P.tma_bytes += 2 * kTile * P.halo_nd * 8;
+  }
   const size_t out = (size_t)P.out_box_bytes * kXEpiWarps;
   P.nstg = fixed + out + 2 * (size_t)P.stg_bytes <= kSmemMax ? 2 : 1;
   return std::max(fixed + out + (size_t)P.nstg * P.stg_bytes, (size_t)116 * 1024);
 }
 
-template <typename TI, typename TO, int N, int AXIS, bool ITER, bool HALO = false>
+template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE = kPlain>
 cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   const size_t smem = plan_smem<TI, N>(P);
   // The shared-memory opt-in is made once per device and instantiation, for the most any launch may
@@ -36,7 +41,7 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   int dev = 0;
   cfd_status s = cuda_fail(cudaGetDevice(&dev), "cudaGetDevice");
   if (s != CFD_OK) return s;
-  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER, HALO>;
+  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER, MODE>;
   if (dev < 0 || dev >= 64 || !opted[dev].load()) {
     s = cuda_fail(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax),
                   "cudaFuncSetAttribute");
@@ -44,33 +49,33 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
     if (dev >= 0 && dev < 64) opted[dev].store(true);
   }
   if (smem > kSmemMax) { set_error("dense: shared memory plan too large"); return CFD_ERR_UNSUPPORTED; }
-  launch_begin(HALO ? KF_HALO : KF_DENSE, st);
+  launch_begin(MODE == kHaloRows ? KF_HALO : KF_DENSE, st);
   fn<<<grid, kXThreads, smem, st>>>(P);
-  launch_end(HALO ? KF_HALO : KF_DENSE, st);
+  launch_end(MODE == kHaloRows ? KF_HALO : KF_DENSE, st);
   return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
 }
 
 // Ghost width 4 has the axis compiled in; other widths share one instantiation per type.
-template <typename TI, typename TO, int N>
+template <typename TI, typename TO, int N, int MODE = kPlain>
 cfd_status launch_exact_types(const DenseParams &P, unsigned grid, cudaStream_t st) {
   const bool it = P.halo_in != nullptr;
   if (P.g == 4) {
-    if (P.axis == 2) return it ? launch_one<TI, TO, N, 2, true>(P, grid, st) : launch_one<TI, TO, N, 2, false>(P, grid, st);
-    if (P.axis == 1) return it ? launch_one<TI, TO, N, 1, true>(P, grid, st) : launch_one<TI, TO, N, 1, false>(P, grid, st);
-    return it ? launch_one<TI, TO, N, 0, true>(P, grid, st) : launch_one<TI, TO, N, 0, false>(P, grid, st);
+    if (P.axis == 2) return it ? launch_one<TI, TO, N, 2, true, MODE>(P, grid, st) : launch_one<TI, TO, N, 2, false, MODE>(P, grid, st);
+    if (P.axis == 1) return it ? launch_one<TI, TO, N, 1, true, MODE>(P, grid, st) : launch_one<TI, TO, N, 1, false, MODE>(P, grid, st);
+    return it ? launch_one<TI, TO, N, 0, true, MODE>(P, grid, st) : launch_one<TI, TO, N, 0, false, MODE>(P, grid, st);
   }
-  return it ? launch_one<TI, TO, N, 3, true>(P, grid, st) : launch_one<TI, TO, N, 3, false>(P, grid, st);
+  return it ? launch_one<TI, TO, N, 3, true, MODE>(P, grid, st) : launch_one<TI, TO, N, 3, false, MODE>(P, grid, st);
 }
 
 // Halo passes: the first one (closed operator rows) has the axis compiled in for ghost width 4; the
 // further iterates, which only n_iter > 1 needs, take the general form.
 template <typename TI, int N>
 cfd_status launch_exact_halo(const DenseParams &P, unsigned grid, cudaStream_t st) {
-  if (P.halo_in) return launch_one<TI, double, N, 3, true, true>(P, grid, st);
-  if (P.g != 4) return launch_one<TI, double, N, 3, false, true>(P, grid, st);
-  if (P.axis == 2) return launch_one<TI, double, N, 2, false, true>(P, grid, st);
-  if (P.axis == 1) return launch_one<TI, double, N, 1, false, true>(P, grid, st);
-  return launch_one<TI, double, N, 0, false, true>(P, grid, st);
+  if (P.halo_in) return launch_one<TI, double, N, 3, true, kHaloRows>(P, grid, st);
+  if (P.g != 4) return launch_one<TI, double, N, 3, false, kHaloRows>(P, grid, st);
+  if (P.axis == 2) return launch_one<TI, double, N, 2, false, kHaloRows>(P, grid, st);
+  if (P.axis == 1) return launch_one<TI, double, N, 1, false, kHaloRows>(P, grid, st);
+  return launch_one<TI, double, N, 0, false, kHaloRows>(P, grid, st);
 }
 
 template <int N>

@@ -1539,6 +1539,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
   auto launch = [&](DenseParams Q) -> cfd_status {
     if (exact) {
       set_launch_constants(Q);
+      if (Q.upwind) return dense_exact_upwind(Q, f32, grid, st);
       return Q.N == 32 ? dense_exact_launch32(Q, Q.in_field && f32, f32, grid, st)
                        : dense_exact_launch16(Q, Q.in_field && f32, f32, grid, st);
     }
@@ -1923,8 +1924,9 @@ size_t dense_biased_workspace(const cfd_blocks_s *B, int nf, int n_iter, bool ad
 }
 
 // Biased first derivatives on the tensor cores: mode 0 (S+) or 1 (S-) of the axes in `axes`
-// into `out` (one op per axis); mode 2: both sides of every axis (one stage per axis) into the
-// workspace, then the upwind blend (advect_combine) into slot out_opidx of out_nops in `out`.
+// into `out` (one op per axis); mode 2: the derivatives of every axis (one stage per axis) into the
+// workspace, then the upwind blend (advect_combine) into slot out_opidx of out_nops in `out`.  The exact
+// form stores the side that the shift selects (upwind_signs, rows_upwind), the others both sides.
 // (Blending in the k_dense epilogue instead reads the shift twice per axis and adds a
 // read-modify-write of the output to the epilogue; measured slower, 9.5 vs 5.7 ms at 256^3.)
 // The operators are
@@ -1949,20 +1951,27 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
   const int S = slices_of(prec), L = levels_of(prec);
   const DensePlanSizes z = dense_sizes(B, nf, 0, n_iter);
   char *base_w = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
-  void *tmp6 = nullptr;
+  void *tmp = nullptr;
+  const bool upwind = mode == 2 && prec == CFD_TC_BF16_EXACT;
+  uint32_t *signs = nullptr;
   if (mode == 2) {
-    tmp6 = base_w;
-    base_w += (interior_points(B) * nf * 6 * (B->dtype == CFD_F32 ? 4 : 8) + 255) & ~(size_t)255;
+    const size_t elem = B->dtype == CFD_F32 ? 4 : 8;
+    tmp = base_w;
+    // (the exact form fills half of the six slots; the signs follow: 3 N^2 words against 3 N^3 values)
+    signs = (uint32_t *)(base_w + ((interior_points(B) * nf * 3 * elem + 255) & ~(size_t)255));
+    base_w += (interior_points(B) * nf * 6 * elem + 255) & ~(size_t)255;
   }
   double *halo[2] = {(double *)base_w, (double *)(base_w + bytes256(z.halo))};
   const int sms = B->num_sms > 0 ? B->num_sms : 148;
   cfd_status s;
-  for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
-    const DenseGroup &G = ds->groups[gi];
-    if (!G.ok || !G.biased) {
+  for (size_t gi = 0; gi < B->sizes.size(); ++gi)
+    if (!ds->groups[gi].ok || !ds->groups[gi].biased) {
       set_error("dense biased: block group unsupported (N must be 16 or 32, uniform spacing, kc <= N)");
       return CFD_ERR_UNSUPPORTED;
     }
+  if (upwind && (s = upwind_signs(B, beta, signs, st)) != CFD_OK) return s;
+  for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
+    const DenseGroup &G = ds->groups[gi];
     const int N = G.N, g = B->ng, E = N + 2 * g;
     if (n_iter > 0 && !G.iter_ok) {
       set_error("dense: hybrid iteration needs N + 2 ng + 4 <= the padded K of the block size");
@@ -1975,11 +1984,12 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
     base.intpre = B->d_intpre;
     base.nblk = (int)B->groups[gi].size();
     base.nf = nf;
-    base.nops = mode == 2 ? 6 : naxes;
+    base.nops = mode == 2 ? (upwind ? 3 : 6) : naxes;
     base.N = N;
     base.g = g;
     base.status = B->d_status;
-    base.out = mode == 2 ? tmp6 : out;
+    base.out = mode == 2 ? tmp : out;
+    base.upwind = upwind ? signs : nullptr;
     base.seg_rows = N;
     base.kext = E;
     {
@@ -2022,9 +2032,9 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       P.n1 = N;
       P.n2 = N;
       P.int_lo1 = 0; P.int_hi1 = N; P.int_lo2 = 0; P.int_hi2 = N;
-      // segments: (side, op); both sides of axis i go to ops 2i, 2i+1 of the workspace
+      // segments: (side, op); both sides of axis i go to ops 2i, 2i+1 of the workspace (upwinded: op i)
       int side[2], op[2], n = 0;
-      if (mode == 2) { side[0] = 0; op[0] = 2 * i; side[1] = 1; op[1] = 2 * i + 1; n = 2; }
+      if (mode == 2) { side[0] = 0; side[1] = 1; op[0] = upwind ? i : 2 * i; op[1] = upwind ? i : 2 * i + 1; n = 2; }
       else { side[0] = mode; op[0] = i; n = 1; }
       const int per_pass = (n * N <= pass_rows(prec)) ? n : 1;
       P.passes = n / per_pass;
@@ -2057,7 +2067,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       if ((s = run(P)) != CFD_OK) return s;
     }
   }
-  if (mode == 2) return advect_combine(B, tmp6, beta, nf, out, out_nops, out_opidx, accum_all, st);
+  if (mode == 2) return advect_combine(B, tmp, !upwind, beta, nf, out, out_nops, out_opidx, accum_all, st);
   return CFD_OK;
 }
 
