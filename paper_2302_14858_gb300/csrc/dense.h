@@ -41,6 +41,9 @@ struct DenseParams {
   // exact form: halo_in / halo_out are [block][field][side: row 1, row N-2][pencil][halo_nd], halo_nd
   // the degrees kept (2, or 1: the one of halo_deg_mask)
   int halo_nd;
+  // exact form: direct = 1: the stage reads output slot direct_op (consecutive blocks, face neighbours on
+  // both sides along the axis) instead of an intermediate
+  int direct, direct_op;
   // exact form: not null in an upwinded stage (segments S+ and S-, one output): per block, axis x, y, z
   // and interior pencil a word whose bit k says that point k takes the right-biased derivative (block b
   // starts at word 3 intpre[b] / 16)
@@ -69,6 +72,7 @@ struct DenseParams {
   const int *sc_local;
   CUtensorMap tmap;          // (the type carries its own 128-byte alignment)
   CUtensorMap tmap_out;
+  CUtensorMap tmap_ghost;    // exact form, direct: the ghost boxes
   int *status;
   long long wait_limit;      // clock cycles a main-loop wait may take before it latches CFD_ERR_TIMEOUT
   float inv_tpj, inv_nf, inv_n2;  // 1 / tiles_per_job, 1 / nf, 1 / n2 (set at launch)
@@ -90,6 +94,7 @@ void halo_rows_from(const std::vector<long double> &M, int cols, HaloRows &R);
 cfd_status halo_rows_launch(const DenseParams &P, const HaloRows &R, bool f32_in, cudaStream_t st);
 
 cfd_status dense_exact_upwind(const DenseParams &P, bool f32, unsigned grid, cudaStream_t st);
+cfd_status dense_exact_direct(const DenseParams &P, bool halo, unsigned grid, cudaStream_t st);
 cfd_status dense_exact_halo(const DenseParams &P, bool f32_in, unsigned grid, cudaStream_t st);
 // One launch of the exact form (dense_exact.cuh) for blocks of 16^3 / 32^3.
 cfd_status dense_exact_launch16(const DenseParams &P, bool f32_in, bool f32_out, unsigned grid, cudaStream_t st);

@@ -243,7 +243,7 @@ __device__ __noinline__ void rows_any(uint32_t taddr, uint32_t lev, int etau, co
 // 8 rows of an upwinded stage: of the two biased derivatives of a point only the one the shift selects
 // (bit of `word`: the right-biased one, the second segment, `seg1` TMEM columns on) is rebuilt and stored.
 // The choice is made on the accumulators, before the conversion to FP64: half the conversions and half
-// the stores of writing both (256^3, 4 fields, three stages: UPWIND_NOTE).  SAFE: as rows_fast.
+// the stores of writing both (256^3, 4 fields: a stage 0.36 -> 0.27 to 0.30 ms).  SAFE: as rows_fast.
 template <typename TO, bool ROW, bool SAFE>
 __device__ __forceinline__ void rows_upwind(uint32_t taddr, uint32_t lev, uint32_t seg1, int etau, const int *rowexp,
                                             int rstep, TO *fin, long long fin_stride, bool wf, uint32_t word,
@@ -313,11 +313,17 @@ __device__ __forceinline__ void rows_upwind(uint32_t taddr, uint32_t lev, uint32
 // FP32 on the CUDA cores (256^3, 4 fields: see halo_pass in dense_tc.cu).
 // UPWIND: the two biased operators of an axis, one output (rows_upwind).  (An instantiation of its own:
 // as a branch of the plain epilogue it cost that one 4 %.)
-enum ExactMode { kPlain = 0, kHaloRows = 1, kUpwind = 2 };
+// DIRECT: an outer stage of a mixed derivative that takes the inner one from its output slot, own points
+// from the block's, ghost columns from the face neighbours' (g = 4, FP64; the columns are in the order
+// [own | lower | upper], and so are the operator's).  No intermediate is written or read: at 256^3, 4
+// fields, the y and z stages drop from 0.45 and 0.49 to 0.38 ms.
+enum ExactMode { kPlain = 0, kHaloRows = 1, kUpwind = 2, kDirect = 3, kHaloDirect = 4 };
 template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE>
 __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_constant__ DenseParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  constexpr bool GEN = AXIS == 3, HALO = MODE == kHaloRows, UPWIND = MODE == kUpwind;
+  constexpr bool GEN = AXIS == 3, HALO = MODE == kHaloRows || MODE == kHaloDirect, UPWIND = MODE == kUpwind,
+                 DIRECT = MODE == kDirect || MODE == kHaloDirect;
+  static_assert(!DIRECT || (AXIS == 1 || AXIS == 2), "outer stages run along y and x");
   constexpr int KP = N == 32 ? 48 : 32, NCH = KP / 8;
   constexpr int ES = sizeof(TI);
   constexpr int SLICE = kTile * KP * 2, A_BYTES = kSl * SLICE;
@@ -406,7 +412,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     // staged element j of this lane's pencil: x rows in boxes of 64 bytes, 16-byte chunks swizzled by
     // the row (chunk ^ (row / 2) % 4: eight rows' chunks cover all banks); columns [t1][j][N] along y,
     // [j][128] along z
-    const int col_base = axis == 1 ? (pl / N) * E * N + pl % N : pl, col_step = axis == 1 ? N : kTile;
+    const int col_base = axis == 1 ? (pl / N) * (DIRECT ? N : E) * N + pl % N : pl, col_step = axis == 1 ? N : kTile;
     auto stg_byte = [&](int pp, int j) -> int {  // for the cp.async path and single elements
       if (axis == 2) {
         const int c = j * ES / 16;
@@ -474,7 +480,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     // Layout [block][field][side][pencil][halo_nd]: a stage of one degree holds (and moves) only its own.
     // With TMA the copies of a tile bring its two runs of 128 pencils behind the staged pencils; loaded by
     // the producers themselves, a tile ahead, they cost the T stages at 256^3 a quarter (0.31 against
-    // HALO_T ms: the index arithmetic sat on the producers' critical path).
+    // 0.28 ms: the index arithmetic sat on the producers' critical path).
     const int np = P.n1 * P.n2;
     auto halo = [&](const unsigned char *st, int tile, int m) -> TI {
       const int d = m >> 1, up = m & 1, dd = P.halo_nd == 2 ? d : 0;
@@ -512,7 +518,25 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       } else {
 #pragma unroll
         for (int h = 0; h < NFULL; ++h) load(st, (half + 2 * h) * 8, 8, v + h * 8);
-        load(st, N + 4 * half, 4, v + NFULL * 8);
+        if constexpr (DIRECT) {
+          // the lower (upper) neighbour's four columns: [128 rows][4] in 32-byte rows, chunk ^ (row / 4) % 2,
+          // or [t1][4][N]
+          const unsigned char *gs = st + kTile * N * ES + half * (kTile * 4 * ES);
+          if (axis == 2) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              const double2 u = *reinterpret_cast<const double2 *>(gs + pl * 32 + ((k ^ ((pl >> 2) & 1)) << 4));
+              v[NFULL * 8 + 2 * k] = u.x;
+              v[NFULL * 8 + 2 * k + 1] = u.y;
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              v[NFULL * 8 + k] = reinterpret_cast<const TI *>(gs)[(pl / N) * 4 * N + pl % N + k * N];
+          }
+        } else {
+          load(st, N + 4 * half, 4, v + NFULL * 8);
+        }
         if constexpr (ITER) {  // the two lanes of a pencil take one degree slot each
           v[NFULL * 8 + 4] = halo(st, tile, 2 * half);
           v[NFULL * 8 + 5] = halo(st, tile, 2 * half + 1);
@@ -784,7 +808,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
         const int sb = nstg == 2 ? it & 1 : 0, su = nstg == 2 ? it >> 1 : it;
         const int job = fdiv(tile, P.inv_tpj), tj = tile - job * P.tiles_per_job, t1_0 = tj * (kTile / N);
         int nb[2] = {0, 0}, q = 0;
-        if constexpr (ITER) {  // (looked up before the wait for the staging buffer)
+        if constexpr (ITER || DIRECT) {  // (looked up before the wait for the staging buffer)
           const int lb = fdiv(job, P.inv_nf), b = P.contig ? P.b0 + lb : P.blocks[lb];
           q = job - lb * P.nf;
           nb[0] = __ldg(P.nbr + b * 26 + dir_index_dev(axis == 0 ? -1 : 0, axis == 1 ? -1 : 0, axis == 2 ? -1 : 0));
@@ -804,6 +828,27 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
                 "l"(src), "r"(bytes), "r"(s_full(sb))
                 : "memory");
           }
+        }
+        if constexpr (DIRECT) {
+          // own points and the two ghost boxes from the output slot [job][op][z][y][x]
+          auto box = [&](const CUtensorMap &m, uint32_t off, int cx, int cy, int j) {
+            const int cz = (j * P.nops + P.direct_op) * N + t1_0;
+            asm volatile(
+                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                "%4}], [%5];" ::"r"(smem_u32(stg0) + (uint32_t)(sb * stg_bytes) + off),
+                "l"(reinterpret_cast<uint64_t>(&m)), "r"(cx), "r"(cy), "r"(cz), "r"(s_full(sb))
+                : "memory");
+          };
+          if (axis == 2) {
+            for (int bx = 0; bx < N / 8; ++bx) box(P.tmap, bx * kTile * kXRowBytes, bx * 8, 0, job);
+          } else {
+            box(P.tmap, 0, 0, 0, job);
+          }
+#pragma unroll
+          for (int up = 0; up < 2; ++up)
+            box(P.tmap_ghost, kTile * N * ES + up * (kTile * 4 * ES), axis == 2 && !up ? N - 4 : 0,
+                axis == 1 && !up ? N - 4 : 0, (nb[up] - P.b0) * P.nf + q);
+          continue;
         }
         const int cz = P.in_start[0] + job * P.tma_zstep + (axis == 0 ? 0 : t1_0);
         const int cy = P.in_start[1] + (axis == 0 ? t1_0 : 0);

@@ -49,9 +49,10 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
     if (dev >= 0 && dev < 64) opted[dev].store(true);
   }
   if (smem > kSmemMax) { set_error("dense: shared memory plan too large"); return CFD_ERR_UNSUPPORTED; }
-  launch_begin(MODE == kHaloRows ? KF_HALO : KF_DENSE, st);
+  constexpr int family = MODE == kHaloRows || MODE == kHaloDirect ? KF_HALO : KF_DENSE;
+  launch_begin(family, st);
   fn<<<grid, kXThreads, smem, st>>>(P);
-  launch_end(MODE == kHaloRows ? KF_HALO : KF_DENSE, st);
+  launch_end(family, st);
   return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
 }
 

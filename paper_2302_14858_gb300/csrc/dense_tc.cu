@@ -1174,6 +1174,10 @@ struct DenseGroup {
   // the same rows (16 with zero padding) as digit images, for the exact form's halo passes:
   // [box][0 closed, 1 iterated], centred and biased
   DenseOp hop[3][2], bhop[3][2];
+  // degree 1 along y and x with the columns in the order of the direct stages [own | lower | upper | halo]:
+  // closed, iterated, and their halo rows (FP64 fields, four ghost layers)
+  DenseOp dop[3], dopI[3], dhop[3][2];
+  bool direct[3] = {false, false, false};  // every block has reciprocal face neighbours along the axis
 };
 
 // Launch choices of the autotuner: per request (fields, ops, precision, iterations, entry
@@ -1195,6 +1199,15 @@ struct DenseState {
 DenseState *state_of(cfd_blocks_s *B) { return reinterpret_cast<DenseState *>(B->dense_state); }
 
 }  // namespace
+
+// columns of the direct stages: own points, lower ghosts, upper ghosts, then whatever follows E
+static std::vector<ld> direct_columns(const std::vector<ld> &D, int rows, int cols, int N, int g) {
+  std::vector<ld> P((size_t)rows * cols);
+  for (int i = 0; i < rows; ++i)
+    for (int j = 0; j < cols; ++j)
+      P[(size_t)i * cols + j] = D[(size_t)i * cols + (j < N ? g + j : (j < N + g ? j - N : j))];
+  return P;
+}
 
 // Device images of one operator; halo rows (all = false) only ever run in the exact form.
 static cfd_status upload_op(cfd_blocks_s *B, const std::vector<ld> &D, int rows, int cols, int Kp, DenseOp &o,
@@ -1272,6 +1285,10 @@ cfd_status dense_bind(cfd_blocks_s *B) {
           G.bopI[box][d] = G.bopI[same][d];
           G.bhop[box][d] = G.bhop[same][d];
         }
+        G.dop[box] = G.dop[same];
+        G.dopI[box] = G.dopI[same];
+        G.dhop[box][0] = G.dhop[same][0];
+        G.dhop[box][1] = G.dhop[same][1];
         G.hr0[box] = G.hr0[same];
         G.hrI[box] = G.hrI[same];
         G.bhr0[box] = G.bhr0[same];
@@ -1288,6 +1305,8 @@ cfd_status dense_bind(cfd_blocks_s *B) {
         else closed_operator(B->s[d - 1], N, g, scale, D);
         cfd_status s = upload_op(B, D, N, E, G.Kp, G.op[box][d - 1]);
         if (s != CFD_OK) return s;
+        const bool dir = d == 1 && g == 4 && B->dtype == CFD_F64;
+        if (dir && (s = upload_op(B, direct_columns(D, N, E, N, g), N, E, G.Kp, G.dop[box], false)) != CFD_OK) return s;
         if (cyc || !G.iter_ok) continue;
         // closed operator without dx scaling: rows 1 and N-2 feed the first halo pass
         std::vector<ld> D0;
@@ -1306,6 +1325,8 @@ cfd_status dense_bind(cfd_blocks_s *B) {
           F[i * G.Kp + hc + 1] = cp[i] * scale;
         }
         if ((s = upload_op(B, F, N, G.Kp, G.Kp, G.opI[box][d - 1])) != CFD_OK) return s;
+        if (dir && (s = upload_op(B, direct_columns(F, N, G.Kp, N, g), N, G.Kp, G.Kp, G.dopI[box], false)) != CFD_OK)
+          return s;
         const int rows[2] = {1, N - 2};
         for (int w = 0; w < 2; ++w) {
           const int r = 2 * (d - 1) + w, i = rows[w];
@@ -1319,6 +1340,10 @@ cfd_status dense_bind(cfd_blocks_s *B) {
         halo_rows_from(HI, G.Kp, G.hrI[box]);
         cfd_status s = upload_op(B, H0, 16, E, G.Kp, G.hop[box][0], false);
         if (s == CFD_OK) s = upload_op(B, HI, 16, G.Kp, G.Kp, G.hop[box][1], false);
+        if (s == CFD_OK && g == 4 && B->dtype == CFD_F64) {
+          s = upload_op(B, direct_columns(H0, 16, E, N, g), 16, E, G.Kp, G.dhop[box][0], false);
+          if (s == CFD_OK) s = upload_op(B, direct_columns(HI, 16, G.Kp, N, g), 16, G.Kp, G.Kp, G.dhop[box][1], false);
+        }
         if (s != CFD_OK) return s;
       }
       if (B->biased.present && B->biased.kc <= N) {
@@ -1386,6 +1411,8 @@ cfd_status dense_bind(cfd_blocks_s *B) {
         }
       }
     }
+    G.direct[2] = mb[0].empty() && mb[1].empty();
+    G.direct[1] = mb[2].empty() && mb[3].empty();
     cfd_status s = cuda_fail(cudaMalloc((void **)&G.d_nl, nl.size() * 4), "cudaMalloc");
     if (G.d_nl) B->d_dense_ptrs.push_back(G.d_nl);
     if (s == CFD_OK) s = cuda_fail(cudaMemcpy(G.d_nl, nl.data(), nl.size() * 4, cudaMemcpyHostToDevice), "cudaMemcpy");
@@ -1522,6 +1549,34 @@ void plan_out_tma(DenseParams &P, size_t elem) {
   P.out_box_bytes = (int)(8 * 32 * elem);
 }
 
+// Tensor maps of a direct stage (DenseParams::direct): the output as [job][op][z][y][x], own points in boxes
+// as plan_tma stages them, four ghost columns (rows) per side.  False where a rule does not hold.
+bool plan_direct(DenseParams &P) {
+  const int N = P.N;
+  const unsigned long long nz = (unsigned long long)P.nblk * P.nf * P.nops * N;
+  if (nz >= (1ull << 31)) return false;
+  char *base = static_cast<char *>(P.out) + (size_t)P.nf * P.nops * P.int0 * 8;
+  if ((uintptr_t)base & 15) return false;
+  EncodeTiledFn enc = tensor_map_encoder();
+  if (!enc) return false;
+  const cuuint64_t gdim[3] = {(cuuint64_t)N, (cuuint64_t)N, (cuuint64_t)nz};
+  const cuuint64_t gstr[2] = {(cuuint64_t)N * 8, (cuuint64_t)N * N * 8};
+  const cuuint32_t estr[3] = {1, 1, 1}, n = (cuuint32_t)N, t = (cuuint32_t)(kTile / N);
+  const cuuint32_t own_x[3] = {8, n, t}, ghost_x[3] = {4, n, t}, own_y[3] = {n, n, t}, ghost_y[3] = {n, 4, t};
+  const bool x = P.axis == 2;
+  auto make = [&](CUtensorMap *m, const cuuint32_t *box, CUtensorMapSwizzle sw) {
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, base, gdim, gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  };
+  if (!make(&P.tmap, x ? own_x : own_y, x ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE) ||
+      !make(&P.tmap_ghost, x ? ghost_x : ghost_y, x ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_NONE))
+    return false;
+  P.tma_kind = x ? 1 : 2;
+  P.tma_boxes = 0;
+  P.tma_bytes = (N + 8) * kTile * 8;
+  return true;
+}
+
 void set_launch_constants(DenseParams &P) {
   P.wait_limit = dense_wait_limit();
   P.inv_tpj = 1.0f / (float)P.tiles_per_job;
@@ -1540,6 +1595,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
     if (exact) {
       set_launch_constants(Q);
       if (Q.upwind) return dense_exact_upwind(Q, f32, grid, st);
+      if (Q.direct) return dense_exact_direct(Q, false, grid, st);
       return Q.N == 32 ? dense_exact_launch32(Q, Q.in_field && f32, f32, grid, st)
                        : dense_exact_launch16(Q, Q.in_field && f32, f32, grid, st);
     }
@@ -1554,7 +1610,8 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
     DenseParams Q = P;
     Q.tile_order = order;
     Q.tiles_per_cta = (Q.ntiles + (int)grid - 1) / (int)grid;
-    if (staging == 0) plan_tma(Q, ein, exact);
+    if (Q.direct) plan_direct(Q);  // (checked before the stage was made)
+    else if (staging == 0) plan_tma(Q, ein, exact);
     else { Q.tma_kind = 0; Q.tma_boxes = 0; }
     if (exact) plan_out_tma(Q, f32 ? 4 : 8);
     return Q;
@@ -1569,7 +1626,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
   TuneRec &r = recs[idx];
   const char axis = "zyx"[P.axis];
   r.stage = std::string(P.in_field ? "S_" : "T_") + axis;
-  const int nstaging = configure(0, 0).tma_kind ? 2 : 1;
+  const int nstaging = configure(0, 0).tma_kind && !P.direct ? 2 : 1;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cfd_status s = cuda_fail(cudaEventCreate(&e0), "cudaEventCreate");
   if (s == CFD_OK) s = cuda_fail(cudaEventCreate(&e1), "cudaEventCreate");
@@ -1618,8 +1675,12 @@ static cfd_status halo_pass(DenseParams H, const DenseOp &op, const HaloRows &ro
   H.ntiles = H.tiles_per_job * H.nblk * H.nf;
   H.tile_order = 0;
   H.out_box_bytes = 0;
-  plan_tma(H, ein, true);
   set_launch_constants(H);
+  if (H.direct) {
+    if (!plan_direct(H)) { set_error("dense: tensor maps of a direct stage"); return CFD_ERR_UNSUPPORTED; }
+    return dense_exact_direct(H, true, (unsigned)std::min(H.ntiles, sms), st);
+  }
+  plan_tma(H, ein, true);
   return dense_exact_halo(H, f32_in, (unsigned)std::min(H.ntiles, sms), st);
 }
 
@@ -1748,7 +1809,8 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
         P.nseg[ps] = per_pass;
         for (int k = 0; k < per_pass; ++k) {
           const int sgi = ps * per_pass + k;
-          const DenseOp &o = iterating(box) ? G.opI[box][deg[sgi] - 1] : G.op[box][deg[sgi] - 1];
+          const DenseOp &o = P.direct ? (iterating(box) ? G.dopI[box] : G.dop[box])
+                                      : (iterating(box) ? G.opI[box][deg[sgi] - 1] : G.op[box][deg[sgi] - 1]);
           P.seg_img[ps][k] = o.image(prec);
           P.seg_exp[ps][k] = o.exps(prec);
           P.seg_mode[ps][k] = mode[sgi];
@@ -1774,7 +1836,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
         H.halo_in = it == 0 ? nullptr : halo[(it - 1) & 1];
         H.halo_out = halo[it & 1];
         H.kext = it == 0 ? E : E + 4;
-        cfd_status r = halo_pass(H, G.hop[box][it > 0], it == 0 ? G.hr0[box] : G.hrI[box], prec == CFD_TC_BF16_EXACT,
+        cfd_status r = halo_pass(H, H.direct ? G.dhop[box][it > 0] : G.hop[box][it > 0], it == 0 ? G.hr0[box] : G.hrI[box], prec == CFD_TC_BF16_EXACT,
                                  B->dtype == CFD_F32, sms, st);
         if (r != CFD_OK) return r;
       }
@@ -1834,9 +1896,37 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
       set_segments(P, P.axis, 2, 0, -1, -1);  // the degree-1 operator, intermediate only
       return run(P);
     };
+    // Direct outer stages: FP64 outputs of d_y (d_z) are the intermediate, ghost columns are the face
+    // neighbours' own points (the values the strips and ghost copies below would hold).
+    auto direct_stage = [&](int inner_op, int box, int op) {
+      DenseParams P = base;
+      P.direct = 1;
+      P.direct_op = inner_op;
+      P.in = out;
+      P.in_box = 0;
+      P.axis = box;
+      P.t1 = 0;
+      P.t2 = box == 2 ? 1 : 2;
+      for (int t = 0; t < 3; ++t) P.in_dims[t] = N;
+      P.n1 = N;
+      P.n2 = N;
+      P.int_hi1 = N;
+      P.int_hi2 = N;
+      set_segments(P, box, 0, op, -1, -1);
+      return P;
+    };
+    auto can = [&](int inner_op, int box) {
+      if (prec != CFD_TC_BF16_EXACT || B->dtype != CFD_F64 || g != 4 || inner_op < 0 || !base.contig || !G.direct[box])
+        return false;
+      DenseParams P = direct_stage(inner_op, box, 0);
+      return plan_direct(P);
+    };
+    const bool dir_xy = odxy >= 0 && can(ody, 2);
+    // (both users of the z intermediate, or none: a lone one would still need it written)
+    const bool dir_z = (odxz >= 0 || odyz >= 0) && (odxz < 0 || can(odz, 2)) && (odyz < 0 || can(odz, 1));
     // S_y: D_y on (z interior, x interior) -> d_y, d_yy, and G_y for d_xy
     if (ody >= 0 || odyy >= 0 || odxy >= 0) {
-      const bool ext = odxy >= 0;
+      const bool ext = odxy >= 0 && !dir_xy;
       const bool copy = ext && N >= 2 * g;  // interior pencils + ghost columns from the epilogue
       DenseParams P = field_stage(1, 0, 2, g, N, (ext && !copy) ? 0 : g, (ext && !copy) ? E : N);
       const int m1 = (ody >= 0 && ext) ? 3 : (ody >= 0 ? 0 : (ext ? 2 : -1));
@@ -1857,7 +1947,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
     }
     // S_z: D_z on (y, x) interior -> d_z, d_zz, and G_z for d_xz / d_yz
     if (odz >= 0 || odzz >= 0 || odxz >= 0 || odyz >= 0) {
-      const bool ext = odxz >= 0 || odyz >= 0;
+      const bool ext = (odxz >= 0 || odyz >= 0) && !dir_z;
       const bool copy = ext && N >= 2 * g;
       const bool wide = ext && !copy;
       DenseParams P = field_stage(0, 1, 2, wide ? 0 : g, wide ? E : N, wide ? 0 : g, wide ? E : N);
@@ -1901,9 +1991,15 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
       P.halo_deg_mask = 1;  // the mixed products apply the degree-1 operator only
       return run_stage(P, box);
     };
-    if (odxy >= 0 && (s = scratch_stage(gy, N, N, E, 2, 0, 1, 0, 0, odxy)) != CFD_OK) return s;
-    if (odxz >= 0 && (s = scratch_stage(gz, N, E, E, 2, 0, 1, 0, g, odxz)) != CFD_OK) return s;
-    if (odyz >= 0 && (s = scratch_stage(gz, N, E, E, 1, 0, 2, 0, g, odyz)) != CFD_OK) return s;
+    if (odxy >= 0 && (s = dir_xy ? run_stage(direct_stage(ody, 2, odxy), 2)
+                                 : scratch_stage(gy, N, N, E, 2, 0, 1, 0, 0, odxy)) != CFD_OK)
+      return s;
+    if (odxz >= 0 && (s = dir_z ? run_stage(direct_stage(odz, 2, odxz), 2)
+                                : scratch_stage(gz, N, E, E, 2, 0, 1, 0, g, odxz)) != CFD_OK)
+      return s;
+    if (odyz >= 0 && (s = dir_z ? run_stage(direct_stage(odz, 1, odyz), 1)
+                                : scratch_stage(gz, N, E, E, 1, 0, 2, 0, g, odyz)) != CFD_OK)
+      return s;
   }
   return CFD_OK;
 }
