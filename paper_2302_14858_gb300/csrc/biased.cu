@@ -579,19 +579,18 @@ __global__ void __launch_bounds__(256) k_advect_combine(const T *__restrict__ tm
   }
 }
 
-// Signs of the shift as bits, per block (from word 3 intpre / 16) [axis x, y, z][pencil]: bit k of a word is set where point k of the
+// Signs of the shift as bits, [block of the size][axis x, y, z][pencil]: bit k of a word is set where point k of the
 // pencil takes the right-biased derivative (beta > 0).  One warp per 32 pencils of a block and axis; along
 // y and z a lane walks its pencil (consecutive x positions), along x the lanes take consecutive points.
 template <typename T>
 __global__ void __launch_bounds__(256) k_upwind_signs(const T *__restrict__ beta, const int *__restrict__ blocks,
-                                                      const long long *__restrict__ extpre,
-                                                      const long long *__restrict__ intpre, int N, int g,
+                                                      const long long *__restrict__ extpre, int N, int g,
                                                       uint32_t *__restrict__ words) {
   const int b = blocks[blockIdx.y], c = blockIdx.z, E = N + 2 * g;
   const int lane = threadIdx.x & 31, p0 = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
   if (p0 >= N * N) return;
   const T *bt = beta + 3 * extpre[b] + (long long)c * E * E * E;
-  uint32_t *w = words + 3 * (intpre[b] >> 4) + c * N * N;
+  uint32_t *w = words + ((long long)blockIdx.y * 3 + c) * N * N;
   if (c == 0) {  // x: rows; 32 / N rows per load
     const int per = 32 / N;
     for (int r0 = 0; r0 < 32; r0 += 8 * per) {
@@ -668,6 +667,12 @@ cfd_status advect_combine(cfd_blocks_s *B, const void *tmp, bool both, const voi
   return CFD_OK;
 }
 
+size_t upwind_words(const cfd_blocks_s *B) {
+  size_t n = 0;
+  for (size_t gi = 0; gi < B->sizes.size(); ++gi) n += B->groups[gi].size() * 3 * B->sizes[gi] * B->sizes[gi];
+  return n;
+}
+
 cfd_status upwind_signs(cfd_blocks_s *B, const void *beta, uint32_t *words, cudaStream_t st) {
   for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
     const int N = B->sizes[gi];
@@ -676,15 +681,22 @@ cfd_status upwind_signs(cfd_blocks_s *B, const void *beta, uint32_t *words, cuda
     launch_begin(KF_BIASED, st);
     if (B->dtype == CFD_F32)
       k_upwind_signs<float><<<grid, 256, 0, st>>>(static_cast<const float *>(beta), B->d_groups[gi], B->d_extpre,
-                                                  B->d_intpre, N, B->ng, words);
+                                                  N, B->ng, words);
     else
       k_upwind_signs<double><<<grid, 256, 0, st>>>(static_cast<const double *>(beta), B->d_groups[gi], B->d_extpre,
-                                                   B->d_intpre, N, B->ng, words);
+                                                   N, B->ng, words);
     launch_end(KF_BIASED, st);
     cfd_status s = cuda_fail(cudaGetLastError(), "k_upwind_signs launch");
     if (s != CFD_OK) return s;
+    words += B->groups[gi].size() * 3 * N * N;
   }
   return CFD_OK;
+}
+
+cfd_status advect_check(cfd_blocks_s *B, int nf, cfd_precision prec, int n_iter, void *work, size_t work_bytes) {
+  int win;
+  cfd_status s = check_request(B, nf, prec, n_iter, &win);
+  return s != CFD_OK ? s : check_work(B, nf, prec, n_iter, work, work_bytes);
 }
 
 cfd_status advect_accumulate(cfd_blocks_s *B, const void *fields, int nf, const void *beta, void *out, int out_nops,

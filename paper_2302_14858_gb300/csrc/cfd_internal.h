@@ -130,18 +130,27 @@ void launch_end(int family, cudaStream_t st);
 cfd_status advect_accumulate(cfd_blocks_s *B, const void *fields, int nf, const void *beta, void *out, int out_nops,
                              int out_opidx, cfd_precision prec, int n_iter, void *work, size_t work_bytes,
                              cudaStream_t st);
+// biased.cu: the checks of advect_accumulate alone (stencil window, iteration, workspace)
+cfd_status advect_check(cfd_blocks_s *B, int nf, cfd_precision prec, int n_iter, void *work, size_t work_bytes);
 // biased.cu: out slot = (accum_all ? out : 0) + sum_{i=x,y,z} beta^i d_i, d_i the biased derivative the sign
 // of beta^i selects: tmp = [block][field][3][N^3] (the selected ones), or with `both`
 // [block][field][6][N^3] (S+ and S- of every axis)
 cfd_status advect_combine(cfd_blocks_s *B, const void *tmp, bool both, const void *beta, int nf, void *out,
                           int out_nops, int out_opidx, bool accum_all, cudaStream_t st);
-// biased.cu: the signs of the shift for DenseParams::upwind (blocks of 16^3 and more: 3 / 16 words per point)
+// biased.cu: the signs of the shift for DenseParams::upwind: sizes in order, 3 N^2 words per block
+size_t upwind_words(const cfd_blocks_s *B);
 cfd_status upwind_signs(cfd_blocks_s *B, const void *beta, uint32_t *words, cudaStream_t st);
 // dense_tc.cu: the biased operators on the tensor cores
 size_t dense_biased_workspace(const cfd_blocks_s *B, int nf, int n_iter, bool advect);
+// (signs, tmp: the upwinded derivatives of every axis into tmp [block][field][3][N^3] with the signs given,
+// without the blend; exact form only)
 cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void *beta, const int *axes, int naxes,
                         int mode, cfd_precision prec, int n_iter, void *out, int out_nops, int out_opidx,
-                        bool accum_all, void *work, size_t work_bytes, cudaStream_t st);
+                        bool accum_all, void *work, size_t work_bytes, cudaStream_t st,
+                        const uint32_t *signs = nullptr, void *tmp = nullptr);
+// Where a step may keep the shift's signs in a one-field workspace of dense_biased whose six slots it fills
+// itself (behind the used part of a halo buffer); null without iteration or where they do not fit.
+uint32_t *dense_sign_space(const cfd_blocks_s *B, void *work, int n_iter);
 
 // exchange.cu
 cfd_status launch_exchange(cfd_blocks_s *B, void *fields, int nfields, cudaStream_t st);

@@ -44,9 +44,8 @@ struct DenseParams {
   // exact form: direct = 1: the stage reads output slot direct_op (consecutive blocks, face neighbours on
   // both sides along the axis) instead of an intermediate
   int direct, direct_op;
-  // exact form: not null in an upwinded stage (segments S+ and S-, one output): per block, axis x, y, z
-  // and interior pencil a word whose bit k says that point k takes the right-biased derivative (block b
-  // starts at word 3 intpre[b] / 16)
+  // exact form: not null in an upwinded stage (segments S+ and S-, one output): per block of the launch,
+  // axis x, y, z and interior pencil a word whose bit k says that point k takes the right-biased derivative
   const uint32_t *upwind;
   int xrow;                  // x-axis stage with 16-byte aligned pencil rows: chunked row copies
   int xvec;                  // x-axis stage with a 16-byte aligned output: vector stores

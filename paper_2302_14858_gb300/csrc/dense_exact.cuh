@@ -708,9 +708,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       if constexpr (UPWIND) {
         // the shift's signs along this pencil, one bit per point
         const uint32_t signs =
-            interior ? __ldg(P.upwind + 3 * ((P.contig ? P.int0 + (long long)c.lb * n3 : P.intpre[c.b]) >> 4) +
-                             (2 - axis) * N * N + tile_pencil(P, tile, pl))
-                     : 0u;
+            interior ? __ldg(P.upwind + (c.lb * 3 + 2 - axis) * N * N + tile_pencil(P, tile, pl)) : 0u;
 #pragma unroll 1
         for (int u = u0; u < units; u += 4) {
           const int o = u * kXUnit;

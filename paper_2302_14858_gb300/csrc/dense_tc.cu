@@ -2019,6 +2019,16 @@ size_t dense_biased_workspace(const cfd_blocks_s *B, int nf, int n_iter, bool ad
   return (advect ? ((interior_points(B) * nf * 6 * elem + 255) & ~(size_t)255) : 0) + 2 * bytes256(z.halo) + 256;
 }
 
+uint32_t *dense_sign_space(const cfd_blocks_s *B, void *work, int n_iter) {
+  if (n_iter <= 0 || B->sizes.size() != 1) return nullptr;
+  const size_t N = B->sizes[0], E = N + 2 * B->ng, nb = B->nblocks;
+  // a halo buffer has 4 E^2 doubles per block, the exact form fills 4 N^2
+  if (upwind_words(B) * 4 > nb * 4 * (E * E - N * N) * 8) return nullptr;
+  char *base = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
+  base += (interior_points(B) * 6 * (B->dtype == CFD_F32 ? 4 : 8) + 255) & ~(size_t)255;
+  return (uint32_t *)(base + nb * 4 * N * N * 8);
+}
+
 // Biased first derivatives on the tensor cores: mode 0 (S+) or 1 (S-) of the axes in `axes`
 // into `out` (one op per axis); mode 2: the derivatives of every axis (one stage per axis) into the
 // workspace, then the upwind blend (advect_combine) into slot out_opidx of out_nops in `out`.  The exact
@@ -2032,7 +2042,8 @@ size_t dense_biased_workspace(const cfd_blocks_s *B, int nf, int n_iter, bool ad
 // lower one).
 cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void *beta, const int *axes, int naxes,
                         int mode, cfd_precision prec, int n_iter, void *out, int out_nops, int out_opidx,
-                        bool accum_all, void *work, size_t work_bytes, cudaStream_t st) {
+                        bool accum_all, void *work, size_t work_bytes, cudaStream_t st, const uint32_t *signs_in,
+                        void *tmp_in) {
   if (!tc_precision(prec)) {
     set_error("unknown precision");
     return CFD_ERR_ARG;
@@ -2065,7 +2076,13 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       set_error("dense biased: block group unsupported (N must be 16 or 32, uniform spacing, kc <= N)");
       return CFD_ERR_UNSUPPORTED;
     }
-  if (upwind && (s = upwind_signs(B, beta, signs, st)) != CFD_OK) return s;
+  const uint32_t *group_signs = signs;
+  if (tmp_in) {
+    tmp = tmp_in;
+    group_signs = signs_in;
+  } else if (upwind && (s = upwind_signs(B, beta, signs, st)) != CFD_OK) {
+    return s;
+  }
   for (size_t gi = 0; gi < B->sizes.size(); ++gi) {
     const DenseGroup &G = ds->groups[gi];
     const int N = G.N, g = B->ng, E = N + 2 * g;
@@ -2085,7 +2102,8 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
     base.g = g;
     base.status = B->d_status;
     base.out = mode == 2 ? tmp : out;
-    base.upwind = upwind ? signs : nullptr;
+    base.upwind = upwind ? group_signs : nullptr;
+    if (upwind) group_signs += (size_t)base.nblk * 3 * N * N;
     base.seg_rows = N;
     base.kext = E;
     {
@@ -2163,7 +2181,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       if ((s = run(P)) != CFD_OK) return s;
     }
   }
-  if (mode == 2) return advect_combine(B, tmp, !upwind, beta, nf, out, out_nops, out_opidx, accum_all, st);
+  if (mode == 2 && !tmp_in) return advect_combine(B, tmp, !upwind, beta, nf, out, out_nops, out_opidx, accum_all, st);
   return CFD_OK;
 }
 
