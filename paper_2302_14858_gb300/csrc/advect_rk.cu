@@ -19,16 +19,23 @@ struct KoArgs {
   const double *scale;     // [b][degree][axis x, y, z] = 1/dx^d
   int N, g, nf, r, ko_on;
   double ko;               // -((-1)^r / 2^{2r}) sigma
-  int c[13];               // (D_+)^r (D_-)^r stencil, m = -r..r
+  double c[13];            // (D_+)^r (D_-)^r stencil, m = -r..r
 };
 
 // F = sum_i Q_i[u] (0 without dissipation), axes x, y, z, taps m = -r..r in FP64.  RC: the
-// stencil order r as a compile-time constant (0: taken from A.r).
+// stencil order r as a compile-time constant (0: taken from A.r).  Bound by the FP64 pipe (30 FMAs per
+// point at r = 4): the coefficients come through shared memory as register operands (64 cycles an FMA, 76
+// from the constant bank; converted per thread from integers they were another 9 operations).
 template <int NC, int RC>
 __global__ void k_ko_fields(const KoArgs A) {
   const int N = NC ? NC : A.N, g = A.g, E = N + 2 * g;
   const int r = RC ? RC : A.r;
   const int n3 = N * N * N;
+  __shared__ double sc[17];
+  if (threadIdx.x < 14) sc[threadIdx.x] = threadIdx.x < 13 ? A.c[threadIdx.x] : 0.0;
+  else if (threadIdx.x < 17)
+    sc[threadIdx.x] = A.ko * A.scale[(A.blocks[blockIdx.y / A.nf] * 2 + 0) * 3 + threadIdx.x - 14];  // x, y, z
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n3) return;
   const int job = blockIdx.y;
@@ -37,15 +44,16 @@ __global__ void k_ko_fields(const KoArgs A) {
   const int x = i % N, y = (i / N) % N, z = i / (N * N);
   const long long E3 = (long long)E * E * E;
   const long long e = (long long)A.nf * A.extpre[b] + q * E3 + ((long long)(z + g) * E + (y + g)) * E + (x + g);
-  double f = 0.0;
+  const double nil = sc[13];
+  double f = nil;
   if (A.ko_on) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const long long st = a == 0 ? 1ll : (a == 1 ? (long long)E : (long long)E * E);   // x, y, z
-      const double w = A.ko * A.scale[(b * 2 + 0) * 3 + a];
-      double s = 0.0;
+      const double w = sc[14 + a];
+      double s = nil;
 #pragma unroll
-      for (int m = -r; m <= r; ++m) s = fma((double)A.c[m + r], __ldg(A.u + e + m * st), s);
+      for (int m = -r; m <= r; ++m) s = fma(sc[m + r], __ldg(A.u + e + m * st), s);
       f = fma(w, s, f);
     }
   }
@@ -59,7 +67,7 @@ struct UpdFArgs {
   const long long *extpre, *intpre;
   const int *blocks;
   int N, g, nf, first;
-  double gamma1, gamma2, bdt, delta;
+  double c[4];             // gamma1, gamma2, beta dt, delta
 };
 
 // S2 <- S2 + delta S1;  S1 <- (gamma1 S1 + gamma2 S2) + (beta dt) F.
@@ -67,6 +75,9 @@ template <int NC>
 __global__ void k_lsrk_fields(const UpdFArgs A) {
   const int N = NC ? NC : A.N, g = A.g, E = N + 2 * g;
   const int n3 = N * N * N;
+  __shared__ double sc[4];  // (register operands: see k_ko_fields)
+  if (threadIdx.x < 4) sc[threadIdx.x] = A.c[threadIdx.x];
+  __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n3) return;
   const int job = blockIdx.y;
@@ -77,9 +88,9 @@ __global__ void k_lsrk_fields(const UpdFArgs A) {
   const long long e = (long long)A.nf * A.extpre[b] + q * E3 + ((long long)(z + g) * E + (y + g)) * E + (x + g);
   const long long in = (long long)A.nf * A.intpre[b] + (long long)q * n3 + i;
   const double u = A.u[e];
-  const double s = A.first ? __dmul_rn(A.delta, u) : __dadd_rn(A.s2[in], __dmul_rn(A.delta, u));
+  const double s = A.first ? __dmul_rn(sc[3], u) : __dadd_rn(A.s2[in], __dmul_rn(sc[3], u));
   A.s2[in] = s;
-  A.u[e] = __dadd_rn(__dadd_rn(__dmul_rn(A.gamma1, u), __dmul_rn(A.gamma2, s)), __dmul_rn(A.bdt, A.F[in]));
+  A.u[e] = __dadd_rn(__dadd_rn(__dmul_rn(sc[0], u), __dmul_rn(sc[1], s)), __dmul_rn(sc[2], A.F[in]));
 }
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -155,7 +166,7 @@ extern "C" cfd_status cfd_advect_lsrk_step(cfd_blocks_t B, void *u, int nfields,
     K.r = r;
     long long binom = 1;
     for (int j = 0; j <= 2 * r; ++j) {
-      K.c[j] = (int)((j % 2 == 0 ? 1 : -1) * binom);  // (-1)^j C(2r, j) at m = j - r
+      K.c[j] = (double)((j % 2 == 0 ? 1 : -1) * binom);  // (-1)^j C(2r, j) at m = j - r
       binom = binom * (2 * r - j) / (j + 1);
     }
     K.ko = -((r % 2 == 0) ? 1.0 : -1.0) / (double)(1ll << (2 * r)) * sigma;
@@ -191,10 +202,8 @@ extern "C" cfd_status cfd_advect_lsrk_step(cfd_blocks_t B, void *u, int nfields,
       U.g = B->ng;
       U.nf = nfields;
       U.first = stage == 0;
-      U.gamma1 = rk->gamma1[stage];
-      U.gamma2 = rk->gamma2[stage];
-      U.bdt = rk->beta[stage] * dt;
-      U.delta = rk->delta[stage];
+      const double cs[4] = {rk->gamma1[stage], rk->gamma2[stage], rk->beta[stage] * dt, rk->delta[stage]};
+      memcpy(U.c, cs, sizeof(U.c));
       launch_begin(KF_RK, st);
       if (N == 32) k_lsrk_fields<32><<<grid, 256, 0, st>>>(U);
       else if (N == 16) k_lsrk_fields<16><<<grid, 256, 0, st>>>(U);

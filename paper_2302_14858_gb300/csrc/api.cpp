@@ -307,6 +307,7 @@ cfd_status apply_banded(cfd_blocks_s *B, const void *fields, int nf, unsigned ma
           ts[k].only = 2;
           ts.push_back(ts[k]);
           ts.back().only = 1;
+          ts.back().cyclic = 1;
         }
       for (size_t i = 0; i < ts.size();) {
         size_t used = 0, j = i;
@@ -346,6 +347,14 @@ cfd_status apply_banded(cfd_blocks_s *B, const void *fields, int nf, unsigned ma
       PencilTask t;
       memset(&t, 0, sizeof(t));
       t.tab = tabs + ptab_index(deg, axis, half);
+      const PencilTab &T = B->h_ptab[gi][ptab_index(deg, axis, half)];
+      t.N = T.N;
+      t.W = T.W;
+      t.h = T.h;
+      t.deg = T.deg;
+      t.anti = T.anti;
+      t.unscaled = T.unscaled;
+      t.cyclic = cyc[axis];
       t.axis = axis;
       t.t1 = axis == 0 ? 1 : 0;
       t.t2 = axis == 2 ? 1 : 2;
@@ -594,6 +603,7 @@ cfd_status cfd_blocks_bind(cfd_scheme_t scheme, int nblocks, const int *block_n,
     PencilTab *p = nullptr;
     if ((s = upload(&p, tabs.data(), tabs.size())) != CFD_OK) return fail(s, nullptr);
     B->d_ptab.push_back(p);
+    B->h_ptab.push_back(std::move(tabs));
   }
   if ((s = upload(&B->d_lidx, lidx.data(), lidx.size())) != CFD_OK) return fail(s, nullptr);
   {

@@ -11,6 +11,13 @@
 // one as it is produced, so one pass over the pencil yields the upwinded right-hand-side term
 // beta d f = beta_+ D[S-] f + beta_- D[S+] f for that axis (transport velocity -beta: the
 // right-biased scheme where beta > 0, the left-biased one where beta < 0).
+//
+// What bounds it: GB300's FP64 pipe.  The tables are read through shared memory, so that every operation
+// is an FMA of three registers (64 cycles per warp and SM sub-partition, 76 with a constant-bank operand
+// or as an add or multiply), and the shift and the running sum are one FMA: 12 operations of 64 cycles per
+// point and axis (X_2), 13 of 76 before.  Pencils on
+// which the shift is zero are left alone, axes on which every block is cyclic take one launch, and for one
+// iteration the halo rows of two axes share a launch.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -138,13 +145,34 @@ template <int NT, int G, int ILO, int IHI, int CLO, int CHI, typename T>
 __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const BiasedTables Tb) {
   constexpr int E = NT + 2 * G;
   constexpr int np = NT * NT;
+  // rhs, closure, (-a)^j, the halo rows of this pass's operator; a, csup, 1/dx-free factors, 0
+  __shared__ double s_rhs[kBTaps], s_clo[kBTaps], s_pw[NT + 1], s_row[2][E], s_c[4];
+  const int axis_slot = blockIdx.z;
+  {
+    const int it = P.pass > 0 ? 1 : 0;
+    for (int i = threadIdx.x; i < kBTaps; i += blockDim.x) {
+      s_rhs[i] = Tb.rhs[i];
+      s_clo[i] = Tb.clo[i];
+    }
+    for (int i = threadIdx.x; i <= NT; i += blockDim.x) s_pw[i] = Tb.pw[i];
+    if (!P.last)
+      for (int i = threadIdx.x; i < 2 * E; i += blockDim.x) s_row[i / E][i % E] = Tb.hrow[i / E][it][i % E];
+    if (threadIdx.x == 0) {
+      s_c[0] = Tb.a;
+      s_c[1] = Tb.csup;
+      s_c[2] = 0.0;
+    }
+  }
+  __syncthreads();
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
   const int job = blockIdx.y;
   const int lb = job / P.nf, q = job - lb * P.nf;
   const int b = P.blocks[lb];
   const int t1 = p / NT, t2 = p - t1 * NT;
-  const int ax = P.axis;
+  // (a halo launch of two axes: the second one's parameters)
+  const int ax = axis_slot ? P.axis2 : P.axis, xt1 = ax == 0 ? 1 : 0, xt2 = ax == 2 ? 1 : 2;
+  double *const halo_out = axis_slot ? P.halo_out2 : P.halo_out;
   const int ez = ax == 0, ey = ax == 1, ex = ax == 2;
   const int nlo = P.nbr[b * 26 + dir_index(-ez, -ey, -ex)];
   const int nhi = P.nbr[b * 26 + dir_index(ez, ey, ex)];
@@ -156,7 +184,7 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
   auto estr = [](int i) { return i == 0 ? (long long)E * E : (i == 1 ? (long long)E : 1ll); };
   constexpr long long box = (long long)E * E * E;
   const long long sa = estr(ax);
-  const long long tr = (long long)(t1 + G) * estr(P.t1) + (long long)(t2 + G) * estr(P.t2);
+  const long long tr = (long long)(t1 + G) * estr(xt1) + (long long)(t2 + G) * estr(xt2);
   const T *fin = static_cast<const T *>(P.in) + (long long)P.nf * P.extpre[b] + (long long)q * box + tr;
 
   double fv[E];
@@ -164,46 +192,69 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
   for (int j = 0; j < E; ++j) fv[j] = static_cast<double>(__ldg(fin + j * sa));
 
   const double scale = P.scale[(b * 2 + 0) * 3 + (2 - ax)];
-  const double a = Tb.a;
+  const double a = s_c[0], csup = s_c[1], nil = s_c[2];
+  double co[IHI - ILO + 1];   // interior coefficients in registers
+#pragma unroll
+  for (int m = ILO; m <= IHI; ++m) co[m - ILO] = s_rhs[m + kBOff];
 
-  // unscaled sums; k is a compile-time constant after unrolling
+  // interior sums with 1/dx, closure sums without; k is a compile-time constant after unrolling.  (1/dx
+  // stays out of the coefficients: their rounded sum, the operator's value on a constant, must not grow.)
   auto left_int = [&](int k) {
-    double acc = 0.0;
+    double acc = nil;
 #pragma unroll
     for (int m = ILO; m <= IHI; ++m) {
       const int j = k + m + G;
-      if (j >= 0 && j < E) acc = fma(Tb.rhs[m + kBOff], fv[j], acc);
+      if (j >= 0 && j < E) acc = fma(co[m - ILO], fv[j], acc);
     }
-    return acc;
+    return fma(acc, scale, nil);
   };
   auto left_clo = [&](int k) {
-    double acc = 0.0;
+    double acc = nil;
 #pragma unroll
     for (int m = CLO; m <= CHI; ++m) {
       const int j = k + m + G;
-      if (j >= 0 && j < E) acc = fma(Tb.clo[m + kBOff], fv[j], acc);
+      if (j >= 0 && j < E) acc = fma(s_clo[m + kBOff], fv[j], acc);
     }
     return acc;
   };
   // mirror: alpha^{(0)}_m -> -alpha^{(0)}_{-m}; the sign is applied by the caller
   auto right_int = [&](int k) {
-    double acc = 0.0;
+    double acc = nil;
 #pragma unroll
     for (int m = ILO; m <= IHI; ++m) {
       const int j = k - m + G;
-      if (j >= 0 && j < E) acc = fma(Tb.rhs[m + kBOff], fv[j], acc);
+      if (j >= 0 && j < E) acc = fma(co[m - ILO], fv[j], acc);
     }
-    return acc;
+    return fma(acc, scale, nil);
   };
   auto right_clo = [&](int k) {
-    double acc = 0.0;
+    double acc = nil;
 #pragma unroll
     for (int m = CLO; m <= CHI; ++m) {
       const int j = k - m + G;
-      if (j >= 0 && j < E) acc = fma(Tb.clo[m + kBOff], fv[j], acc);
+      if (j >= 0 && j < E) acc = fma(s_clo[m + kBOff], fv[j], acc);
     }
     return acc;
   };
+
+  // R consecutive interior rows (k, k + dir, ..) at a time: R independent chains keep the FP64 pipe fed
+  // where only two warps share a sub-partition (one chain at a time it was busy 57 % of the time)
+  auto rows = [&](auto left_c, auto r_c, int k, double *r) {
+    constexpr bool LEFT = decltype(left_c)::value;
+    constexpr int R = decltype(r_c)::value;
+#pragma unroll
+    for (int u = 0; u < R; ++u) r[u] = nil;
+#pragma unroll
+    for (int m = ILO; m <= IHI; ++m)
+#pragma unroll
+      for (int u = 0; u < R; ++u) {
+        const int j = (LEFT ? k + u + m : k - u - m) + G;
+        if (j >= 0 && j < E) r[u] = fma(co[m - ILO], fv[j], r[u]);
+      }
+#pragma unroll
+    for (int u = 0; u < R; ++u) r[u] = fma(r[u], scale, nil);
+  };
+  using std::integral_constant;
 
   const bool do_p = P.mode != 1, do_m = P.mode != 0;
   const long long hp = (long long)np * 2;
@@ -212,20 +263,22 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
     // halo-only pass: the two values the neighbours read next pass (d+ at N-kc, d- at kc-1),
     // each one row of the dense block operator (closed for pass 0, iterated after that)
     const int it = P.pass > 0 ? 1 : 0;
-    double *h = P.halo_out + ((long long)b * P.nf + q) * hp + 2 * p;
-    if (do_p) {
-      double acc = 0.0;
+    double *h = halo_out + ((long long)b * P.nf + q) * hp + 2 * p;
+    double s0[2] = {nil, nil}, s1[2] = {nil, nil};   // both rows, even and odd columns
 #pragma unroll
-      for (int j = 0; j < E; ++j) acc = fma(Tb.hrow[0][it][j], fv[j], acc);
-      double v = acc * scale;
+    for (int j = 0; j < E; j += 2)
+#pragma unroll
+      for (int w = 0; w < 2; ++w) {
+        s0[w] = fma(s_row[w][j], fv[j], s0[w]);
+        s1[w] = fma(s_row[w][j + 1], fv[j + 1], s1[w]);
+      }
+    if (do_p) {
+      double v = (s0[0] + s1[0]) * scale;
       if (it) v = fma(Tb.hc[0], P.halo_in[((long long)nlo * P.nf + q) * hp + 2 * p + 0], v);
       h[0] = v;
     }
     if (do_m) {
-      double acc = 0.0;
-#pragma unroll
-      for (int j = 0; j < E; ++j) acc = fma(Tb.hrow[1][it][j], fv[j], acc);
-      double v = acc * scale;
+      double v = (s0[1] + s1[1]) * scale;
       if (it) v = fma(Tb.hc[1], P.halo_in[((long long)nhi * P.nf + q) * hp + 2 * p + 1], v);
       h[1] = v;
     }
@@ -243,40 +296,46 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
     for (int k = 0; k < NT; ++k) any |= sign_bits(__ldg(bet + k * sa));
     need_p = (any & 2) != 0;   // beta < 0 somewhere: left-biased
     need_m = (any & 1) != 0;   // beta > 0 somewhere: right-biased
+    if (any == 0 && P.accum) return;  // nothing to add
   }
 
   // ---- right-biased derivative (S-), rows k = N-1 .. 0, kept in registers
   double dm[NT];
   if (need_m) {
-    const double ms = -scale;
     if (cyclic) {
       // y_{N-1} = r_{N-1}, y_k = r_k - a y_{k+1};  d_k = y_k + (-a)^{N-k} d_0, d_0 = y_0 / (1 - (-a)^N)
 #pragma unroll
       for (int k = NT - 1; k >= 0; --k) {
-        const double r = right_int(k) * ms;
-        dm[k] = (k == NT - 1) ? r : fma(-a, dm[k + 1], r);
+        const double r = right_int(k);
+        dm[k] = (k == NT - 1) ? -r : fma(-a, dm[k + 1], -r);
       }
       const double d0 = dm[0] * Tb.cyc_inv;
 #pragma unroll
-      for (int k = 1; k < NT; ++k) dm[k] = fma(Tb.pw[NT - k], d0, dm[k]);
+      for (int k = 1; k < NT; ++k) dm[k] = fma(s_pw[NT - k], d0, dm[k]);
       dm[0] = d0;
-    } else if (P.pass == 0) {
-      // closure row N-1 (csup d_{N-2} + d_{N-1}) coupled with interior row N-2
-      const double rc = right_clo(NT - 1) * ms;
-      const double r2 = right_int(NT - 2) * ms;
-      dm[NT - 1] = fma(-Tb.csup, r2, rc) * Tb.inv01;
-      dm[NT - 2] = fma(-a, dm[NT - 1], r2);
-#pragma unroll
-      for (int k = NT - 3; k >= 0; --k) dm[k] = fma(-a, dm[k + 1], right_int(k) * ms);
     } else {
-      // iterated: d at k^c_+ = N-1+kc is the right neighbour's previous iterate
-      double h = P.halo_in[((long long)nhi * P.nf + q) * hp + 2 * p + 1];
-      if (Tb.kc >= 3) h = fma(-a, h, right_int(NT + 1) * ms);
-      if (Tb.kc >= 2) h = fma(-a, h, right_int(NT) * ms);
+      if (P.pass == 0) {
+        // closure row N-1 (csup d_{N-2} + d_{N-1}) coupled with interior row N-2
+        const double rc = right_clo(NT - 1) * -scale;
+        const double r2 = -right_int(NT - 2);
+        dm[NT - 1] = fma(-csup, r2, rc) * Tb.inv01;
+        dm[NT - 2] = fma(-a, dm[NT - 1], r2);
+      } else {
+        // iterated: d at k^c_+ = N-1+kc is the right neighbour's previous iterate
+        double h = P.halo_in[((long long)nhi * P.nf + q) * hp + 2 * p + 1];
+        if (Tb.kc >= 3) h = fma(-a, h, -right_int(NT + 1));
+        if (Tb.kc >= 2) h = fma(-a, h, -right_int(NT));
+        dm[NT - 1] = fma(-a, h, -right_int(NT - 1));
+        dm[NT - 2] = fma(-a, dm[NT - 1], -right_int(NT - 2));
+      }
 #pragma unroll
-      for (int k = NT - 1; k >= 0; --k) {
-        h = fma(-a, h, right_int(k) * ms);
-        dm[k] = h;
+      for (int k = NT - 3; k >= 1; k -= 4) {
+        double r[4];
+        if (k >= 3) rows(integral_constant<bool, false>(), integral_constant<int, 4>(), k, r);
+        else rows(integral_constant<bool, false>(), integral_constant<int, 2>(), k, r);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k - u >= 0) dm[k - u] = fma(-a, dm[k - u + 1], -r[u]);
       }
     }
   }
@@ -286,22 +345,20 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
   auto ostr = [](int i) { return i == 0 ? (long long)NT * NT : (i == 1 ? (long long)NT : 1ll); };
   const long long oa = ostr(ax);
   T *o = static_cast<T *>(P.out) + (long long)P.nf * P.nops * P.intpre[b] + ((long long)q * P.nops + P.opidx) * n3 +
-         (long long)t1 * ostr(P.t1) + (long long)t2 * ostr(P.t2);
+         (long long)t1 * ostr(xt1) + (long long)t2 * ostr(xt2);
   auto emit = [&](int k, double dp) {
-    double v;
     if (P.mode == 0) {
-      v = dp;
+      o[k * oa] = static_cast<T>(P.accum ? static_cast<double>(o[k * oa]) + dp : dp);
     } else if (P.mode == 1) {
-      v = dm[k];
+      o[k * oa] = static_cast<T>(P.accum ? static_cast<double>(o[k * oa]) + dm[k] : dm[k]);
     } else {
-      // beta_+ dm + beta_- dp: beta dm where beta > 0, beta dp where beta < 0, 0 where beta = 0
+      // beta_+ dm + beta_- dp: beta dm where beta > 0, beta dp where beta < 0, nothing where beta = 0
       const T braw = __ldg(bet + k * sa);
       const int sg = sign_bits(braw);
-      const double bb = static_cast<double>(braw);
-      v = sg == 1 ? bb * dm[k] : (sg == 2 ? bb * dp : 0.0);
+      const double old = P.accum ? static_cast<double>(o[k * oa]) : nil;
+      const double v = fma(static_cast<double>(braw), sg == 1 ? dm[k] : dp, old);
+      o[k * oa] = static_cast<T>(sg == 0 ? old : v);
     }
-    if (P.accum) v = static_cast<double>(o[k * oa]) + v;
-    o[k * oa] = static_cast<T>(v);
   };
 
   // ---- left-biased derivative (S+), rows k = 0 .. N-1, emitted as produced
@@ -311,40 +368,47 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
       double y = 0.0;
 #pragma unroll
       for (int k = 0; k < NT; ++k) {
-        const double r = left_int(k) * scale;
+        const double r = left_int(k);
         y = (k == 0) ? r : fma(-a, y, r);
       }
       const double dl = y * Tb.cyc_inv;
 #pragma unroll
       for (int k = 0; k < NT; ++k) {
-        const double r = left_int(k) * scale;
+        const double r = left_int(k);
         y = (k == 0) ? r : fma(-a, y, r);
-        emit(k, fma(Tb.pw[k + 1], dl, y));
+        emit(k, fma(s_pw[k + 1], dl, y));
       }
     } else {
       double d;
-      int k0;
       if (P.pass == 0) {
         // closure row 0 (d_0 + csup d_1) coupled with interior row 1
         const double r0 = left_clo(0) * scale;
-        const double r1 = left_int(1) * scale;
-        d = fma(-Tb.csup, r1, r0) * Tb.inv01;
+        const double r1 = left_int(1);
+        d = fma(-csup, r1, r0) * Tb.inv01;
         emit(0, d);
         d = fma(-a, d, r1);
         emit(1, d);
-        k0 = 2;
       } else {
         // iterated: d at k^c_- = -kc is the left neighbour's previous iterate
         d = P.halo_in[((long long)nlo * P.nf + q) * hp + 2 * p + 0];
-        if (Tb.kc >= 3) d = fma(-a, d, left_int(-2) * scale);
-        if (Tb.kc >= 2) d = fma(-a, d, left_int(-1) * scale);
-        k0 = 0;
+        if (Tb.kc >= 3) d = fma(-a, d, left_int(-2));
+        if (Tb.kc >= 2) d = fma(-a, d, left_int(-1));
+        d = fma(-a, d, left_int(0));
+        emit(0, d);
+        d = fma(-a, d, left_int(1));
+        emit(1, d);
       }
 #pragma unroll
-      for (int k = 0; k < NT; ++k) {
-        if (k < k0) continue;
-        d = fma(-a, d, left_int(k) * scale);
-        emit(k, d);
+      for (int k = 2; k < NT; k += 4) {
+        double r[4];
+        if (k + 4 <= NT) rows(integral_constant<bool, true>(), integral_constant<int, 4>(), k, r);
+        else rows(integral_constant<bool, true>(), integral_constant<int, 2>(), k, r);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u < NT) {
+            d = fma(-a, d, r[u]);
+            emit(k + u, d);
+          }
       }
     }
   } else {
@@ -356,7 +420,7 @@ __global__ void __launch_bounds__(128) k_biased(const BiasedParams P, const Bias
 template <int G, int ILO, int IHI, int CLO, int CHI>
 cfd_status launch_window(const BiasedParams &P, const BiasedTables &T, cudaStream_t st, cfd_dtype dt) {
   const int np = T.N * T.N;
-  dim3 grid((np + 127) / 128, P.nblk * P.nf);
+  dim3 grid((np + 127) / 128, P.nblk * P.nf, P.axes);
   auto go = [&](auto nt) {
     constexpr int NT = decltype(nt)::value;
     if (dt == CFD_F32) k_biased<NT, G, ILO, IHI, CLO, CHI, float><<<grid, 128, 0, st>>>(P, T);
@@ -402,6 +466,11 @@ size_t halo_elems(const cfd_blocks_s *B, int nf, int n_iter) {
   int nmax = 0;
   for (int N : B->sizes) nmax = std::max(nmax, N);
   return (size_t)B->nblocks * nf * nmax * nmax * 2;
+}
+
+int dir_index_host(int dz, int dy, int dx) {
+  const int r = 9 * (dz + 1) + 3 * (dy + 1) + (dx + 1);
+  return r > 13 ? r - 1 : r;
 }
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -475,21 +544,40 @@ cfd_status run_biased(cfd_blocks_s *B, const void *fields, int nf, const void *b
     P.nf = nf;
     P.nops = out_nops > 0 ? out_nops : (mode == 2 ? 1 : naxes);
     P.mode = mode;
+    // blocks that are their own neighbour along an axis: on all of them one pass is enough
+    auto cyclic_blocks = [&](int a) {
+      size_t n = 0;
+      for (int b : B->groups[gi])
+        if (B->nbr[b * 26 + dir_index_host(-(a == 0), -(a == 1), -(a == 2))] == b &&
+            B->nbr[b * 26 + dir_index_host(a == 0, a == 1, a == 2)] == b)
+          ++n;
+      return n;
+    };
+    int ahead = -1;  // axis whose (only) halo pass has run with the previous axis's, into halo[1]
     for (int i = 0; i < naxes; ++i) {
       const int a = axes[i];
       P.axis = a;
-      P.t1 = a == 0 ? 1 : 0;
-      P.t2 = a == 2 ? 1 : 2;
       P.opidx = mode == 2 ? out_opidx : i;
       P.accum = (mode == 2 && (i > 0 || accum_all)) ? 1 : 0;
-      for (int pass = 0; pass <= n_iter; ++pass) {
+      const int last = cyclic_blocks(a) == B->groups[gi].size() ? 0 : n_iter;
+      for (int pass = a == ahead ? 1 : 0; pass <= last; ++pass) {
         P.pass = pass;
-        P.last = pass == n_iter;
-        P.halo_in = pass > 0 ? halo[(pass - 1) & 1] : nullptr;
+        P.last = pass == last;
+        P.axes = 1;
+        P.halo_in = pass > 0 ? halo[a == ahead ? 1 : (pass - 1) & 1] : nullptr;
         P.halo_out = halo[pass & 1];
+        // (a cyclic block writes its outputs in pass 0: such axes keep their launches to themselves)
+        if (n_iter == 1 && pass == 0 && ahead < 0 && i + 1 < naxes && cyclic_blocks(a) == 0 &&
+            cyclic_blocks(axes[i + 1]) == 0) {
+          ahead = axes[i + 1];
+          P.axes = 2;
+          P.axis2 = ahead;
+          P.halo_out2 = halo[1];
+        }
         cfd_status s = launch_biased(win, P, T, st, B->dtype);
         if (s != CFD_OK) return s;
       }
+      if (a == ahead) ahead = -1;
     }
   }
   return CFD_OK;

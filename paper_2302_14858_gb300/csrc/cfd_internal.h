@@ -62,7 +62,9 @@ struct BiasedParams {
   const double *halo_in;   // [nblocks][nf][N^2][2]: (d+ at N-kc, d- at kc-1) of the previous iterate
   double *halo_out;
   int nblk, nf, nops, opidx;
-  int axis, t1, t2;        // box axes (0 z, 1 y, 2 x)
+  int axis;                // box axis of the pencils (0 z, 1 y, 2 x)
+  int axes, axis2;         // axes = 2: a halo pass of `axis2` too, into halo_out2
+  double *halo_out2;
   int mode;                // 0 d[S+], 1 d[S-], 2 advect (beta_+ d[S+] + beta_- d[S-])
   int accum;               // 1: add into out
   int pass, last;
@@ -73,6 +75,35 @@ void build_biased_tables(const BiasedCoef &c, int N, int g, BiasedTables &T);
 void biased_operator(const BiasedCoef &c, int N, int g, int side, int kind, std::vector<long double> &W,
                      std::vector<long double> &coup);
 
+}  // namespace cfd
+
+namespace cfd {
+// What the solves along one axis need, for one block size, degree and scale (device copy), prepared in
+// long double.  Antisymmetric stencils act on differences, which vanish for a constant whatever the
+// coefficients round to: the scale 1/dx^d and the reciprocal pivot of a row are folded into them, and a
+// row costs its right-hand side and one FMA forward, one back.  Other stencils keep the coefficients as
+// given (their rounded sum, the operator's value on a constant, must not grow): pivot and scale come in
+// on the way back, one more operation per row.
+struct PencilTab {
+  int N, M, h, deg;      // block size, interior and closure half-widths, degree
+  int W;                 // points needed beyond the block on each side: max(h, M + 1)
+  int anti;              // degree 1 with exactly antisymmetric coefficients: differences of pairs
+  int unscaled;          // spacing differs between blocks: results are multiplied per block
+  double neg, nil;       // -1 and 0 (see stencil() in line.cu)
+  double factor;         // folded into the results (1, or 1/2 for one half of an averaged pair)
+  double clo[2 * kMaxH + 1];
+  double sc, isc;        // scale of rows that keep their coefficients (1: folded), and its reciprocal
+  // closed system (rows 1..N-2; rows 0 and N-1 are the closures): row k
+  //   z_k = sum_m rc[k][m + M] f_{k+m} - lo[k] z_{k-1},   x_k = pv[k] z_k - up[k] x_{k+1}
+  double rc[kMaxN][2 * kMaxM + 1], lo[kMaxN], up[kMaxN], pv[kMaxN];
+  // iterated system, rows k = -1..N at k + 1; the fixed values enter the first and last row
+  double irc[kMaxN + 2][2 * kMaxM + 1], ilo[kMaxN + 2], iup[kMaxN + 2], ipv[kMaxN + 2], hhi;
+  // cyclic system: Thomas rows of the corner-modified matrix, its Sherman-Morrison vector
+  double yrc[kMaxN][2 * kMaxM + 1], ylo[kMaxN], yup[kMaxN], ypv[kMaxN], z[kMaxN], a, vfac;
+  // rows 1 and N-2 of the closed and of the iterated operator over the window (index j + W for point
+  // j), and the coefficients of the fixed values: what the neighbours read (factor 1 always)
+  double hrow[2][2][kMaxN + 2 * kMaxH + 2], hc[2][2];
+};
 }  // namespace cfd
 
 struct cfd_scheme_s {
@@ -93,6 +124,7 @@ struct cfd_blocks_s {
   std::vector<std::vector<int>> groups;  // block ids per distinct N
   // FP64 banded tables per distinct N (line.h), device: [degree 1: axis, full / half][degree 2: axis]
   std::vector<void *> d_ptab;
+  std::vector<std::vector<cfd::PencilTab>> h_ptab;
   cfd::BiasedCoef biased;
   std::vector<cfd::BiasedTables> btab; // per distinct N (when biased.present)
   bool iter_ok = true;                 // same-size face neighbours everywhere

@@ -48,13 +48,13 @@ constexpr int kTabDoubles = (kMaxN + 2) * (2 * 3 + 1) + 4 * (kMaxN + 2) + 2 * kM
 // measured); a symmetric one the plain chain, whose partial sums stay small (pair sums f_{k+m} + f_{k-m}
 // cost as much and rounded 30 % worse).  R rows at a time are R independent chains: a row by row loop
 // took 1.5 times as long where few warps share an SM.
-template <int M, int R>
-__device__ __forceinline__ void stencils(double (&r)[R], const double *c, int cw, const double *p, bool anti, double neg,
+template <int M, int R, bool anti>
+__device__ __forceinline__ void stencils(double (&r)[R], const double *c, int cw, const double *p, double neg,
                                          double nil) {
   double f[R + 2 * M];
 #pragma unroll
   for (int i = 0; i < R + 2 * M; ++i) f[i] = p[(i - M) * kPitch];
-  if (anti) {
+  if constexpr (anti) {
 #pragma unroll
     for (int m = M; m >= 1; --m)
 #pragma unroll
@@ -80,15 +80,15 @@ __device__ __forceinline__ double closure_row(const double *c, const double *p, 
 
 // Forward sweep over rows k0 .. k0 + n - 1 (n even): z_k = r_k - lo_k z_{k-1}, stored where point k - M
 // was (the rows after k no longer read it).  c, lo: the first row's.
-template <int M>
+template <int M, bool anti>
 __device__ __forceinline__ double forward(const double *c, const double *lo, double *f0, int k0, int n, double z,
-                                          bool anti, double neg, double nil) {
+                                          double neg, double nil) {
   constexpr int CW = 2 * M + 1;
   int i = 0;
   auto rows = [&](auto rc) {
     constexpr int R = decltype(rc)::value;
     double r[R];
-    stencils<M, R>(r, c + i * CW, CW, f0 + (k0 + i) * kPitch, anti, neg, nil);
+    stencils<M, R, anti>(r, c + i * CW, CW, f0 + (k0 + i) * kPitch, neg, nil);
 #pragma unroll
     for (int u = 0; u < R; ++u) {
       z = fma(-lo[i + u], z, r[u]);
@@ -136,7 +136,8 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
   extern __shared__ double line_smem[];
   const PencilTask &K = A.task[blockIdx.y];
   const PencilTab &tab = *K.tab;
-  const int N = tab.N, W = tab.W, L = N + 2 * W, g = A.g;
+  const int N = K.N, W = K.W, L = N + 2 * W, g = A.g;
+  const bool cyc = K.cyclic != 0, unscaled = K.unscaled != 0;
   const int lane = threadIdx.x & 31;
   constexpr bool HALO = M == 0;
   constexpr int CW = 2 * M + 1;
@@ -159,32 +160,31 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
   const long long n3 = (long long)N * N * N;
   auto stride = [](int axis, int n) { return axis == 0 ? n * n : (axis == 1 ? n : 1); };
 
-  // a block that is its own neighbour on both faces is a whole periodic line
-  const int blo = A.nbr[b * 26 + dir_index(-(ax == 0), -(ax == 1), -(ax == 2))];
-  const int bhi = A.nbr[b * 26 + dir_index(ax == 0, ax == 1, ax == 2)];
-  const bool cyc = blo == b && bhi == b;
-  if (K.only) valid = valid && cyc == (K.only == 1);
-  const bool any_cyc = __syncthreads_or(valid && cyc);  // (all or none: see PencilTask::only)
+  // the face neighbours (a block that is its own on both sides is a whole periodic line)
+  const bool look = K.only || (!cyc && A.pass > 0);
+  const int blo = look ? A.nbr[b * 26 + dir_index(-(ax == 0), -(ax == 1), -(ax == 2))] : 0;
+  const int bhi = look ? A.nbr[b * 26 + dir_index(ax == 0, ax == 1, ax == 2)] : 0;
+  if (K.only) valid = valid && (blo == b && bhi == b) == (K.only == 1);
+  // (copied while the pencils are fetched; one barrier for both)
   if (HALO) {
     const double *h = &tab.hrow[A.pass > 0][0][0];
     constexpr int HW = sizeof(tab.hrow[0][0]) / sizeof(double);
     for (int i = threadIdx.x; i < 2 * HW; i += blockDim.x) s_rc[i] = __ldg(h + i);
   } else {
-    const double(*rc)[2 * kMaxM + 1] = any_cyc ? tab.yrc : (A.pass > 0 ? tab.irc : tab.rc);
-    const double *lo = any_cyc ? tab.ylo : (A.pass > 0 ? tab.ilo : tab.lo);
-    const double *up = any_cyc ? tab.yup : (A.pass > 0 ? tab.iup : tab.up);
-    const double *pv = any_cyc ? tab.ypv : (A.pass > 0 ? tab.ipv : tab.pv);
-    const int rows = !any_cyc && A.pass > 0 ? N + 2 : N;
+    const double(*rc)[2 * kMaxM + 1] = cyc ? tab.yrc : (A.pass > 0 ? tab.irc : tab.rc);
+    const double *lo = cyc ? tab.ylo : (A.pass > 0 ? tab.ilo : tab.lo);
+    const double *up = cyc ? tab.yup : (A.pass > 0 ? tab.iup : tab.up);
+    const double *pv = cyc ? tab.ypv : (A.pass > 0 ? tab.ipv : tab.pv);
+    const int rows = !cyc && A.pass > 0 ? N + 2 : N;
     for (int i = threadIdx.x; i < rows * CW; i += blockDim.x) s_rc[i] = __ldg(&rc[i / CW][i % CW]);
     for (int i = threadIdx.x; i < rows; i += blockDim.x) {
       s_lo[i] = __ldg(lo + i);
       s_up[i] = __ldg(up + i);
       s_pv[i] = __ldg(pv + i);
-      if (any_cyc) s_z[i] = __ldg(&tab.z[i]);
+      if (cyc) s_z[i] = __ldg(&tab.z[i]);
     }
     if (threadIdx.x <= 2 * kMaxH) s_clo[threadIdx.x] = __ldg(&tab.clo[threadIdx.x]);
   }
-  __syncthreads();
 
   // ---- the pencil: points -W .. N+W-1 at tile entries 0 .. L-1
   if (!K.gather) {
@@ -222,9 +222,9 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       }
     }
   }
-  __syncwarp();
+  __syncthreads();
   double *f0 = tile + W * kPitch + lane;  // point 0 of this lane's pencil
-  const double scale = tab.unscaled ? A.scale[(b * 2 + (tab.deg - 1)) * 3 + (2 - ax)] : 1.0;
+  const double scale = unscaled ? A.scale[(b * 2 + (K.deg - 1)) * 3 + (2 - ax)] : 1.0;
   // the neighbours' previous iterate at k^c = -2 and N+1 (their rows N-2 and 1)
   double dlo = 0.0, dhi = 0.0;
   if (valid && !cyc && A.pass > 0) {
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
     const double *h = A.halo + K.halo_in;
     dlo = h[(((long long)nlo * A.nf + q) * np + p) * 2 + 1];
     dhi = h[(((long long)nhi * A.nf + q) * np + p) * 2 + 0];
-    if (tab.unscaled) {
+    if (unscaled) {
       dlo /= scale;
       dhi /= scale;
     }
@@ -256,13 +256,16 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       }
       for (; j < L; ++j) s0 = fma(c[j], f[j * kPitch], s0);
       s0 = (s0 + s1) + (s2 + s3);
-      h[w] = tab.unscaled ? s0 * scale : s0;
+      h[w] = unscaled ? s0 * scale : s0;
     }
     return;
   } else {
+    // (the stencil's kind and the output's are compile-time inside: left to run time, the compiler executes
+    // both sides of a choice between operations and selects, two more per output)
+    auto solve = [&](auto anti_c, auto add_c, auto unscaled_c) {
+    constexpr bool anti = decltype(anti_c)::value, ADD = decltype(add_c)::value, UNSCALED = decltype(unscaled_c)::value;
     // ---- solve
-    const bool anti = tab.anti;
-    const double neg = __ldg(&tab.neg), nil = __ldg(&tab.nil);
+    const double neg = __ldg(&tab.neg), nil = __ldg(&tab.nil), one = -neg;
     double *zrow = f0 - M * kPitch;
     const bool closed = !cyc && A.pass == 0;
     double x = 0.0, z = 0.0, x0 = 0.0;
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
     const double *up, *pv;   // x_k = pv[k] z_k - up[k] x_{k+1} (pv: rows that keep their coefficients)
     auto scaled = [&](double v, double p) { return anti ? v : fma(v, p, nil); };
     if (cyc) {
-      z = forward<M>(s_rc, s_lo, f0, 0, N, 0.0, anti, neg, nil);
+      z = forward<M, anti>(s_rc, s_lo, f0, 0, N, 0.0, neg, nil);
       x = scaled(z, s_pv[N - 1]);
       zrow[(N - 1) * kPitch] = x;
       const double xn = x;
@@ -283,17 +286,17 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       top = -1;
       up = pv = nullptr;
     } else if (closed) {
-      x0 = closure_row(s_clo, f0, tab.h, anti, neg, nil);
-      x = closure_row(s_clo, f0 + (N - 1) * kPitch, tab.h, anti, neg, nil);
+      x0 = closure_row(s_clo, f0, K.h, anti, neg, nil);
+      x = closure_row(s_clo, f0 + (N - 1) * kPitch, K.h, anti, neg, nil);
       // (the closure rows take a zero times their neighbour, so a NaN or an infinity reaches the whole pencil)
-      x = fma(nil, forward<M>(s_rc + CW, s_lo + 1, f0, 1, N - 2, x0, anti, neg, nil), scaled(x, tab.sc));
+      x = fma(nil, forward<M, anti>(s_rc + CW, s_lo + 1, f0, 1, N - 2, x0, neg, nil), scaled(x, tab.sc));
       x0 = scaled(x0, tab.sc);
       top = N - 2;
       up = s_up;
       pv = s_pv;
     } else {
       // row -1 starts from the fixed value: z_{-2} enters as hlo / lo times it
-      z = forward<M>(s_rc, s_lo, f0, -1, N + 2, scaled(tab.factor * dlo, tab.isc), anti, neg, nil);
+      z = forward<M, anti>(s_rc, s_lo, f0, -1, N + 2, scaled(tab.factor * dlo, tab.isc), neg, nil);
       x = fma(-tab.hhi, dhi, scaled(z, s_pv[N + 1]));  // row N
       top = N - 1;
       up = s_up + 1;
@@ -320,19 +323,18 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
     }
     const long long ostr = stride(ax, N);
     const bool rows = ax == 2 && !K.strip;  // x pencils leave through the tile, row by row
-    const bool add = K.accum && out && !rows;
     auto emit = [&](int k, double v, double old) {
-      if (tab.unscaled) v *= scale;
+      if constexpr (UNSCALED) v = fma(v, scale, nil);
       if (rows) {
         zrow[k * kPitch] = v;
         return;
       }
       if (sc) sc[k * sstr] = v;
-      if (out) out[k * ostr] = (T)(add ? v + old : v);
+      if (out) out[k * ostr] = (T)(ADD ? fma(old, one, v) : v);
     };
-    auto before = [&](int k) { return add ? (double)out[k * ostr] : 0.0; };
+    auto before = [&](int k) { return ADD && out && !rows ? (double)out[k * ostr] : 0.0; };
     if (top < 0) {
-      if (!rows || tab.unscaled)
+      if (!rows || UNSCALED)
         for (int k = 0; k < N; ++k) emit(k, zrow[k * kPitch], before(k));
     } else {
       if (closed) {
@@ -366,11 +368,25 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
         for_rows(sc, N, [&](double *, int r, int k) { return row0[k * kPitch + r]; },
                  [](double *row, int, int k, double v) { row[k] = v; });
       if (K.out_op >= 0) {
-        const bool acc = K.accum != 0;
         for_rows(out, N,
-                 [&](T *row, int r, int k) { return acc ? row0[k * kPitch + r] + (double)row[k] : row0[k * kPitch + r]; },
+                 [&](T *row, int r, int k) { 
+                   double v = row0[k * kPitch + r];
+                   if constexpr (ADD) v = fma((double)row[k], one, v);
+                   return v;
+                 },
                  [](T *row, int, int k, double v) { row[k] = (T)v; });
       }
+    }
+    };
+    using std::false_type;
+    using std::true_type;
+    if (unscaled) {
+      if (K.anti) K.accum ? solve(true_type(), true_type(), true_type()) : solve(true_type(), false_type(), true_type());
+      else K.accum ? solve(false_type(), true_type(), true_type()) : solve(false_type(), false_type(), true_type());
+    } else if (K.anti) {
+      K.accum ? solve(true_type(), true_type(), false_type()) : solve(true_type(), false_type(), false_type());
+    } else {
+      K.accum ? solve(false_type(), true_type(), false_type()) : solve(false_type(), false_type(), false_type());
     }
   }
 }
