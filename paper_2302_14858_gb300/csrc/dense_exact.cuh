@@ -352,11 +352,11 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   auto t_full = [&](int i) { return bar0 + 8u * (uint32_t)(8 + i); };
   auto t_empty = [&](int i) { return bar0 + 8u * (uint32_t)(12 + i); };
   auto meta_full = [&](int i) { return bar0 + 8u * (uint32_t)(16 + i); };
-  const uint32_t drain = bar0 + 8u * 24u;
+  const uint32_t drain = bar0 + 8u * 24u, b_full = bar0 + 8u * 25u;
   const long long WL = P.wait_limit;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  if (warp == 0) {
+  if (warp == kXProdWarps + kXEpiWarps) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
                  "r"(kTmemCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -374,27 +374,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     for (int i = 0; i < 4; ++i) { mbar_init(t_full(i), 1); mbar_init(t_empty(i), readers); }
     for (int i = 0; i < kXEtau; ++i) mbar_init(meta_full(i), kXProdWarps);
     mbar_init(drain, 1);
+    mbar_init(b_full, kXEpiWarps);
     asm volatile("fence.mbarrier_init.release.cluster;");
   }
-  // operator digits: slices stacked along the MMA's N rows, [t][segment][N]
-  for (int sg = 0; sg < P.nseg[0]; ++sg) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(P.seg_img[0][sg]);
-    constexpr int U = SR * KP * 2 / 16;
-    for (int i = tid; i < kSl * U; i += kXThreads) {
-      const int t = i / U, r = i - t * U;
-      reinterpret_cast<uint4 *>(sB + (t * R + sg * SR) * KP * 2)[r] = __ldg(src + i);
-    }
-    for (int i = tid; i < SR; i += kXThreads) s_rowexp[sg * SR + i] = P.seg_exp[0][sg][i];
-  }
-  if constexpr (!GEN) {
-    // the columns behind the pencil (K padding; the halo columns are rewritten per tile) stay zero
-    constexpr int PADC = NCH - (N + 8) / 8;
-    for (int i = tid; i < 2 * kSl * (kTile / 8) * PADC * 8; i += kXThreads) {
-      const int w = i & 7, r = i >> 3, ch = (N + 8) / 8 + r % PADC, rg = r / PADC;  // rg: [buf][slice][row group]
-      reinterpret_cast<uint4 *>(sA)[(rg * NCH + ch) * 8 + w] = make_uint4(0u, 0u, 0u, 0u);
-    }
-  }
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
@@ -408,6 +390,18 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   if (warp < kXProdWarps) {
     // ================================================================ producers
     asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
+    if constexpr (!GEN) {
+      // the columns behind the pencil (K padding; halo columns are rewritten per tile) stay zero: each lane
+      // clears its pencil's rows of one buffer
+      const int zp = warp * 16 + (lane & 15);
+      unsigned char *z = sA + (lane >> 4) * A_BYTES + (zp >> 3) * (NCH * 128) + (zp & 7) * 16;
+#pragma unroll
+      for (int sl = 0; sl < kSl; ++sl)
+#pragma unroll
+        for (int ch = (N + 8) / 8; ch < NCH; ++ch)
+          *reinterpret_cast<uint4 *>(z + sl * SLICE + ch * 128) = make_uint4(0u, 0u, 0u, 0u);
+      __syncwarp();
+    }
     const int pl = warp * 16 + (lane & 15), half = lane >> 4;
     // staged element j of this lane's pencil: x rows in boxes of 64 bytes, 16-byte chunks swizzled by
     // the row (chunk ^ (row / 2) % 4: eight rows' chunks cover all banks); columns [t1][j][N] along y,
@@ -591,6 +585,25 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else if (warp < kXProdWarps + kXEpiWarps) {
     // ================================================================ epilogue
+    // First the operator digits, while the first tiles are copied and split: slices stacked along the MMA's
+    // N rows, [t][segment][N].  (With the whole CTA loading them before it starts, a launch of one tile per
+    // CTA took 0.3 us longer, 256^3 with nine ops 20 us.)
+    {
+      const int et = tid - kXProd;
+      constexpr int ET = kXEpiWarps * 32, U = SR * KP * 2 / 16;
+      for (int sg = 0; sg < P.nseg[0]; ++sg) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(P.seg_img[0][sg]);
+        for (int i = et; i < kSl * U; i += ET) {
+          const int t = i / U, r = i - t * U;
+          reinterpret_cast<uint4 *>(sB + (t * R + sg * SR) * KP * 2)[r] = __ldg(src + i);
+        }
+        for (int i = et; i < SR; i += ET) s_rowexp[sg * SR + i] = P.seg_exp[0][sg][i];
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_full);
+      asm volatile("bar.sync 1, %0;" ::"n"(ET) : "memory");  // the row exponents
+    }
     const int quad = warp & 3, ew = (warp - kXProdWarps) >> 2;
     const int pl = quad * 32 + lane;
     constexpr int UPS = N / kXUnit;  // units per segment
@@ -766,9 +779,10 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     if (lane == 0) {
       bool issued = false;
       int it = 0;
+      if (!mbar_wait_bounded(b_full, 0u, WL)) failed = true;
       for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
         const int buf = it & 1, tb = it & (nbuf - 1), tu = nbuf == 2 ? it >> 1 : it >> 2;
-        if (!mbar_wait_bounded(a_full(buf), (uint32_t)((it >> 1) & 1), WL) ||
+        if (failed || !mbar_wait_bounded(a_full(buf), (uint32_t)((it >> 1) & 1), WL) ||
             (tu > 0 && !mbar_wait_bounded(t_empty(tb), (uint32_t)((tu - 1) & 1), WL))) {
           failed = true;
           break;
@@ -872,7 +886,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   __syncwarp();
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+  if (warp == kXProdWarps + kXEpiWarps) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 
 }  // namespace
