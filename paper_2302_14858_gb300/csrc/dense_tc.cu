@@ -24,6 +24,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <array>
 #include <map>
 #include <new>
 #include <string>
@@ -1190,9 +1191,11 @@ struct TuneRec {
 };
 struct DenseState {
   std::vector<DenseGroup> groups;
-  std::map<std::string, std::vector<TuneRec>> tuned;
+  // a request: entry point (0 apply, 1 biased), fields, ops (biased: mode), precision, iterations, axes
+  typedef std::array<int, 6> Key;
+  std::map<Key, std::vector<TuneRec>> tuned;
   bool tuning = false;             // cfd_autotune in progress: every launch tries its candidates
-  std::string key;                 // the request of the current call
+  Key key = {};                    // the request of the current call
   int launch = 0;                  // launches of the current call so far
 };
 
@@ -1617,11 +1620,12 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
     return Q;
   };
   const int idx = ds->launch++;
-  std::vector<TuneRec> &recs = ds->tuned[ds->key];
   if (!ds->tuning) {
-    const bool have = idx < (int)recs.size();
-    return launch(configure(have ? recs[idx].staging : 0, have ? recs[idx].order : 0));
+    const auto found = ds->tuned.find(ds->key);
+    const bool have = found != ds->tuned.end() && idx < (int)found->second.size();
+    return launch(configure(have ? found->second[idx].staging : 0, have ? found->second[idx].order : 0));
   }
+  std::vector<TuneRec> &recs = ds->tuned[ds->key];
   if ((int)recs.size() <= idx) recs.resize(idx + 1);
   TuneRec &r = recs[idx];
   const char axis = "zyx"[P.axis];
@@ -1724,8 +1728,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
   }
   DenseState *ds = state_of(B);
   if (!ds) { set_error("dense: operators were not built at bind"); return CFD_ERR_UNSUPPORTED; }
-  ds->key = "apply nf=" + std::to_string(nf) + " ops=" + std::to_string(mask) + " prec=" + std::to_string((int)prec) +
-            " n_iter=" + std::to_string(n_iter);
+  ds->key = {0, nf, (int)mask, (int)prec, n_iter, 0};
   ds->launch = 0;
   const int S = slices_of(prec), L = levels_of(prec);
   const DensePlanSizes z = dense_sizes(B, nf, mask, n_iter);
@@ -2050,8 +2053,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
   }
   DenseState *ds = state_of(B);
   if (!ds) { set_error("dense: operators were not built at bind"); return CFD_ERR_UNSUPPORTED; }
-  ds->key = "biased nf=" + std::to_string(nf) + " mode=" + std::to_string(mode) + " naxes=" + std::to_string(naxes) +
-            " prec=" + std::to_string((int)prec) + " n_iter=" + std::to_string(n_iter);
+  ds->key = {1, nf, mode, (int)prec, n_iter, naxes};
   ds->launch = 0;
   const size_t need = dense_biased_workspace(B, nf, n_iter, mode == 2);
   if (!work || work_bytes < need) { set_error("biased path: workspace too small (see cfd_biased_workspace)"); return CFD_ERR_ARG; }
@@ -2212,7 +2214,13 @@ std::string dense_tuning_report(cfd_blocks_s *B) {
   if (ds) {
     bool first = true;
     for (const auto &kv : ds->tuned) {
-      o += std::string(first ? "" : ", ") + "\"" + kv.first + "\": [";
+      const DenseState::Key &k = kv.first;
+      auto num = [](int v) { return std::to_string(v); };
+      const std::string name = k[0] ? "biased nf=" + num(k[1]) + " mode=" + num(k[2]) + " naxes=" + num(k[5]) + " prec=" +
+                                          num(k[3]) + " n_iter=" + num(k[4])
+                                    : "apply nf=" + num(k[1]) + " ops=" + num(k[2]) + " prec=" + num(k[3]) +
+                                          " n_iter=" + num(k[4]);
+      o += std::string(first ? "" : ", ") + "\"" + name + "\": [";
       first = false;
       for (size_t i = 0; i < kv.second.size(); ++i) {
         const TuneRec &r = kv.second[i];
