@@ -246,14 +246,17 @@ __device__ __forceinline__ double to_double(float f) {
 
 // The right-hand side with FP32 stencil sums for N in {16, 32} and r = 4, the tensor-core steps' form.  A
 // CTA of N x 16 threads marches along z through the planes of its 16 rows.  Each plane (with its 4-wide
-// halo) is converted to FP32 once, when it enters a ring of five planes four steps ahead; the z taps come
-// from a register queue fed by the ring.  What bounds it: the FP64 pipe had 13 operations per point (seven
-// of them conversions), 0.52 ms a stage at 256^3; now four, and 0.43 ms.
+// halo) is converted to FP32 once, when it enters a ring of planes four steps ahead; the z taps come from a
+// register queue fed by the ring.  What bounds it: the FP64 pipe had 13 operations per point (seven of them
+// conversions), 0.52 ms a stage at 256^3; with four it is memory latency: 0.43 ms with five planes in the
+// ring, two barriers per plane and the Laplacian's loads behind the first; 0.37 with a sixth plane, so that
+// the slot written is none of those that warps behind the single barrier still read, and those loads ahead
+// of it.  (Two points per thread, 24 warps per SM instead of 32: 0.52.)
 template <int N>
 __global__ void __launch_bounds__(N * 16) k_wave_rhs_ring(const RhsArgs A) {
-  constexpr int RR = 4, TY = 16, NT = N * TY, W = N + 2 * RR, H = TY + 2 * RR, Q = 2 * RR + 1, HW = H * W;
+  constexpr int RR = 4, TY = 16, NT = N * TY, W = N + 2 * RR, H = TY + 2 * RR, Q = 2 * RR + 1, HW = H * W, SLOTS = RR + 2;
   constexpr int PER = (HW + NT - 1) / NT;  // values of a plane and field per thread
-  __shared__ float ring[5][2][HW];
+  __shared__ float ring[SLOTS][2][HW];
   __shared__ double s_one;
   const int g = A.g, E = N + 2 * g;
   const long long E2 = (long long)E * E;
@@ -309,11 +312,11 @@ __global__ void __launch_bounds__(N * 16) k_wave_rhs_ring(const RhsArgs A) {
   fetch(RR);
   int cur = 0, in = RR;      // ring slots of plane z and of plane z + 4
   for (int z = 0; z < N; ++z) {
+    const int i = (z * N + (y0 + ty)) * N + tx;
+    const double l0 = L[i], l1 = L[n3 + i], l2 = L[2 * n3 + i], kk = __ldg(f[1] + (long long)(g + z) * E2 + col);
     put(in);
     __syncthreads();
     if (z + 1 < N) fetch(z + 1 + RR);
-    const int i = (z * N + (y0 + ty)) * N + tx;
-    const double l0 = L[i], l1 = L[n3 + i], l2 = L[2 * n3 + i], kk = __ldg(f[1] + (long long)(g + z) * E2 + col);
     float sum[2];
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -332,9 +335,8 @@ __global__ void __launch_bounds__(N * 16) k_wave_rhs_ring(const RhsArgs A) {
     }
     L[i] = fma(fma(fma(l0, one, l1), one, l2), one, to_double(sum[1]));
     L[n3 + i] = fma(kk, one, to_double(sum[0]));
-    cur = cur == 4 ? 0 : cur + 1;
-    in = in == 4 ? 0 : in + 1;
-    __syncthreads();         // plane z is read: its slot takes plane z + 5
+    cur = cur == SLOTS - 1 ? 0 : cur + 1;
+    in = in == SLOTS - 1 ? 0 : in + 1;
   }
 }
 

@@ -116,3 +116,93 @@ def test_rows_with_a_flat_operator_keep_their_accuracy(lib, nblk):
     want = np.einsum("ij,bzyj->bzyi", D, f[:, 0, I, I, :])
     bound = 2.0 ** -36 * np.abs(D).sum(1)      # |f| < 1 = tau; 2^-37 sum |D f| is the design bound
     assert np.all(np.abs(got - want) <= bound[None, None, None, :])
+
+
+@pytest.mark.parametrize("N,g,dtype,nf,n_iter,offset", [
+    (32, 4, "f64", 4, 0, 0),      # a quarter of a million points, four fields: the side is chosen in the stages
+    (32, 4, "f64", 4, 1, 1),      # element copies in, per-thread x outputs
+    (32, 4, "f32", 6, 2, 0),      # two groups of four fields, the second partial
+    (16, 6, "f64", 5, 1, 0),      # another ghost width: run-time addressing
+    (16, 4, "f32", 4, 0, 1),
+])
+def test_upwinded_stages_match_the_banded_solve(lib, N, g, dtype, nf, n_iter, offset):
+    """The shift term where the stages store only the side that the shift selects, with shift components
+    of both signs, of one sign and of zeros (of either sign, which select the same finite side)."""
+    import torch
+    from tests.helpers import SCHEMES
+    nb = 64 // N
+    mesh = W.periodic_box_mesh(nb, nb, nb, N, g)
+    np_t, t_t = (np.float32, torch.float32) if dtype == "f32" else (np.float64, torch.float64)
+    r = W.rng(300 + N + g + n_iter)
+    fs = []
+    for _ in range(nf + 1):
+        s = W.sine_sum(r, 6, 1, 4)
+        s.k = 2 * np.pi * s.k / (64 * mesh.dx[0, 0])
+        fs.append(s)
+    E = N + 2 * g
+    flat = W.pack(W.sample(mesh, fs, np_t)).reshape(nb ** 3, nf + 1, E ** 3)
+    fields = np.ascontiguousarray(flat[:, :nf]).reshape(-1)
+    shift = np.zeros((nb ** 3, 3, E ** 3), np_t)
+    shift[:, 0] = flat[:, nf]                                   # both signs inside a block
+    shift[:, 1] = 0.25                                          # one side everywhere
+    shift[:, 2] = np.where(np.arange(E ** 3) % 3 == 0, np_t(-0.0), np_t(0.0))
+    shift[nb ** 3 // 2:, 2] = -0.5
+    dev = torch.device("cuda", 0)
+
+    def put(a):
+        hold = torch.zeros(a.size + 8, dtype=t_t, device=dev)
+        v = hold[offset:offset + a.size]
+        v.copy_(torch.from_numpy(a.reshape(-1)))
+        return v
+
+    f, b = put(fields), put(shift)
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), None)
+    lib.cfd_scheme_set_biased(s, SCHEMES["X2_d1"])
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F32 if dtype == "f32" else lib.CFD_F64)
+    outs = []
+    for prec in (lib.CFD_TC_BF16_EXACT, lib.CFD_FP64_BANDED):
+        buf = torch.full((64 ** 3 * nf + 8,), float("nan"), dtype=t_t, device=dev)
+        out = buf[offset:offset + 64 ** 3 * nf]
+        work = torch.empty(max(lib.cfd_biased_workspace(B, nf, prec, n_iter), 256), dtype=torch.uint8, device=dev)
+        lib.cfd_advect(B, f, nf, b, prec, n_iter, out, work)
+        lib.cfd_sync_status(B)
+        outs.append(out.double().cpu().numpy().reshape(nb ** 3, nf, -1))
+    tol = 2e-6 if dtype == "f32" else 1e-7
+    for q in range(nf):
+        assert rel_max(outs[0][:, q], outs[1][:, q]) < tol, q
+
+
+@pytest.mark.parametrize("N,g,offset", [(16, 4, 0), (16, 4, 1), (32, 4, 0), (32, 4, 1), (32, 5, 0)])
+def test_wave_step_with_dissipation_matches_the_banded_one(lib, N, g, offset):
+    """One 2S step with r = 4 dissipation (the FP32 ring of planes) on aligned and unaligned fields, for an
+    odd ghost width and with an axis of a single block."""
+    import torch
+    from oracle import timestep as T
+    mesh = W.periodic_box_mesh(2, 1, 2, N, g)
+    L = [m * N * mesh.dx[0, a] for a, m in enumerate((2, 1, 2))]
+    r = W.rng(900 + N + g)
+    fs = []
+    for _ in range(2):
+        s = W.sine_sum(r, 6, 1, 4)
+        s.k = 2 * np.pi * s.k / np.asarray(L)
+        fs.append(s)
+    E = N + 2 * g
+    flat = W.pack(W.sample(mesh, fs, np.float64)).reshape(4, 2, E ** 3)
+    dev = torch.device("cuda", 0)
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), desc("Q13_1_d2"))
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F64)
+    outs = []
+    for prec in (lib.CFD_TC_BF16_EXACT, lib.CFD_FP64_BANDED):
+        u = []
+        for q in range(2):
+            hold = torch.zeros(4 * E ** 3 + 2, dtype=torch.float64, device=dev)
+            v = hold[offset:offset + 4 * E ** 3]
+            v.copy_(torch.from_numpy(flat[:, q].reshape(-1).copy()))
+            u.append(v)
+        work = torch.empty(lib.cfd_wave_lsrk_workspace(B, prec, 1), dtype=torch.uint8, device=dev)
+        lib.cfd_wave_lsrk_step(B, u[0], u[1], 0.2 * mesh.dx.min(), T.lsrk2s_rk4_float(), 0.04, 4, prec, 1, work)
+        lib.cfd_sync_status(B)
+        I = slice(g, g + N)
+        outs.append([v.cpu().numpy().reshape(4, E, E, E)[:, I, I, I] for v in u])
+    for q in range(2):
+        assert rel_max(outs[0][q], outs[1][q]) < 1e-7, q
