@@ -898,9 +898,9 @@ def main():
             a1 = algorithmic_bytes(nint, nf, nops, elem) * n1 / ((tl1 + th1) * 1e-3) / 1e9
             iter1["roofline"] = {"achieved": round(a1, 1), "unit": "GB/s", "frac": round(a1 / hbm, 4),
                                  "how": "algorithmic bytes per step / time per step of the final passes (k_dense) "
-                                        "and the halo passes (k_halo_rows)",
+                                        "and the halo passes",
                                  "k_dense_ms_per_step": round(tl1 / n1, 4),
-                                 "k_halo_rows": {"launches_per_step": round(nh1 / n1, 2),
+                                 "halo_passes": {"launches_per_step": round(nh1 / n1, 2),
                                                  "ms_per_step": round(th1 / n1, 4)}}
         del work1
 
@@ -1103,7 +1103,7 @@ def run_advect(args, spec):
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     if prec != cfd.CFD_FP64_BANDED:
         # k_dense: per axis the field is read once and both biased derivatives written once; each
-        # halo pass of the iteration (k_halo_rows) reads the field again.  The blend kernel reads the
+        # halo pass of the iteration reads the field again.  The blend kernel reads the
         # upwind derivative of each axis per field, the three shift components once per point,
         # and writes the term.
         elem = fields.element_size()
@@ -1119,7 +1119,8 @@ def run_advect(args, spec):
                 "algorithmic_bytes_per_launch": round(per_pf * units / max(ndl / prof_steps, 1)),
                 "launches_per_step": ndl / prof_steps, "avg_launch_ms": round(tdl / max(ndl, 1), 5),
                 "share_of_step": round(tdl / (ms_prof * prof_steps), 4),
-                "halo_passes": {"kernel": "k_halo_rows (compensated FP32 on the CUDA cores)",
+                "halo_passes": {"kernel": "k_dense_exact, 16-row operators" if prec == cfd.CFD_TC_BF16_EXACT
+                                else "k_halo_rows (compensated FP32 on the CUDA cores)",
                                 "launches_per_step": nhl / prof_steps, "ms_per_step": round(thl / prof_steps, 4),
                                 "hbm_gbs": round(3 * n_iter * elem * units * prof_steps / (thl * 1e-3) / 1e9, 1)
                                 if thl > 0 else None},

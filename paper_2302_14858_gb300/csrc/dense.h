@@ -35,7 +35,7 @@ struct DenseParams {
   int seg_rows;              // operator rows per segment (N, or 16 for a halo pass)
   int kext;                  // K values loaded per pencil: N + 2g, or N + 2g + 4 with halo columns
   const double *halo_in;     // [nblocks][nf][n1 n2][4]: previous iterate at rows 1, N-2 per degree (x dx^d)
-  double *halo_out;          // same layout, written by a halo pass (k_halo_rows)
+  double *halo_out;          // same layout, written by a halo pass
   const int *nbr;            // [nblocks][26] neighbour table
   int halo_deg_mask;         // degrees whose halo columns are filled (bit d-1)
   // exact form: halo_in / halo_out are [block][field][side: row 1, row N-2][pencil][halo_nd], halo_nd

@@ -18,7 +18,7 @@
 // outputs).  In both digit forms row i of D is scaled by a power of two sigma_i, every pencil p by a
 // power of two tau_p (taken from its values in the kernel), and the epilogue writes the integer sum
 // times 2^{e(sigma_i) + e(tau_p) - const} by assembling the IEEE bits.  The halo passes of the hybrid
-// iteration run on the CUDA cores (halo_rows.cu).
+// iteration run in the exact kernel too; those of the other two forms on the CUDA cores (halo_rows.cu).
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -2040,7 +2040,7 @@ uint32_t *dense_sign_space(const cfd_blocks_s *B, void *work, int n_iter) {
 // read-modify-write of the output to the epilogue; measured slower, 9.5 vs 5.7 ms at 256^3.)
 // The operators are
 // the dense forms of the block systems of Eqs. closure_left_X / iter_left_X (bind time); the
-// iteration runs the halo passes of the centred path (k_halo_rows) with the biased halo rows
+// iteration runs the halo passes of the centred path (halo_pass) with the biased halo rows
 // (slot 1: S+ at row N-kc, read by the upper neighbour; slot 2: S- at row kc-1, read by the
 // lower one).
 cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void *beta, const int *axes, int naxes,

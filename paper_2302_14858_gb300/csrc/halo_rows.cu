@@ -1,4 +1,5 @@
-// Halo passes of the hybrid iteration on the CUDA cores, in compensated FP32.
+// Halo passes of the hybrid iteration for the BF16X3 and TF32 forms, on the CUDA cores in compensated FP32
+// (the exact form computes them on the tensor cores, in its own digits).
 //
 // The hybrid iteration (Eq. iter_center_P for the centred schemes, Eq. iter_left_X for the
 // biased ones) needs, before each final pass along a decomposed axis, the values every block's
