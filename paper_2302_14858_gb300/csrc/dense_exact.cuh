@@ -14,9 +14,11 @@
 // Measured (256^3 as 512 blocks of 32^3, 4 FP64 fields, nine ops: six launches, event times): five
 // BF16 digits with 15 pairs, 8 + 8 warps, one staging buffer 2.87 ms in all; this form with 8 epilogue
 // warps 2.69; with 16 epilogue warps and TMA stores of the x outputs 2.03 (S_x 0.37, S_y 0.45, S_z 0.48,
-// T_x 0.25, T_y 0.24 ms).  A producer's value costs ~20 instructions against ~45 before, an output ~15
-// against ~28.  What bounds it now: DRAM traffic (S_y and S_z move ~2.6 GB each, 0.40 ms at the copy
-// rate), and in S_x the FP64 pipe (64 conversions of 64 cycles per SM sub-partition and tile, 0.23 ms).
+// T_x 0.25, T_y 0.24 ms); direct outer stages, the operator's load behind the first tiles and a quarter of
+// the outputs converted by integers 1.79 (S 0.36 to 0.37, T 0.24 to 0.25).  A producer's value costs ~20
+// instructions against ~45 before, an output ~15 against ~28.  What bounds it now: T stages DRAM; S stages
+// DRAM (0.25 ms at the copy rate) and the FP64 pipe (48 conversions of 64 cycles per SM sub-partition and
+// tile, 0.17 ms) beside the integer work, no one of them alone.
 //
 // Roles (28 warps, one persistent CTA per SM):
 //   warps 0-7    producers: wait for a staged tile, split it into 4 digit rows of A[buf];
@@ -402,6 +404,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
   bool failed = false;
+  chain_next();
   const TileRange tr = tile_range(P);
   // a whole warp waits together: its lanes leave a loop on the same outcome
   auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
@@ -423,6 +426,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
           *reinterpret_cast<uint4 *>(z + sl * SLICE + ch * 128) = make_uint4(0u, 0u, 0u, 0u);
       __syncwarp();
     }
+    chain_wait();
     const int pl = warp * 16 + (lane & 15), half = lane >> 4;
     // staged element j of this lane's pencil: x rows in boxes of 64 bytes, 16-byte chunks swizzled by
     // the row (chunk ^ (row / 2) % 4: eight rows' chunks cover all banks); columns [t1][j][N] along y,
@@ -624,6 +628,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       __syncwarp();
       if (lane == 0) mbar_arrive(b_full);
       asm volatile("bar.sync 1, %0;" ::"n"(ET) : "memory");  // the row exponents
+      chain_wait();
     }
     const int quad = warp & 3, ew = (warp - kXProdWarps) >> 2;
     const int pl = quad * 32 + lane;
@@ -742,7 +747,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       if constexpr (UPWIND) {
         // the shift's signs along this pencil, one bit per point
         const uint32_t signs =
-            interior ? __ldg(P.upwind + (c.lb * 3 + 2 - axis) * N * N + tile_pencil(P, tile, pl)) : 0u;
+            interior ? P.upwind[(c.lb * 3 + 2 - axis) * N * N + tile_pencil(P, tile, pl)] : 0u;
 #pragma unroll 1
         for (int u = u0; u < units; u += 4) {
           const int o = u * kXUnit;
@@ -835,6 +840,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     // ================================================================ TMA issue
     asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
     if (lane == 0 && kind) {
+      chain_wait();
       const uint64_t tmap = reinterpret_cast<uint64_t>(&P.tmap);
       int it = 0;
       for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {

@@ -51,7 +51,7 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   if (smem > kSmemMax) { set_error("dense: shared memory plan too large"); return CFD_ERR_UNSUPPORTED; }
   constexpr int family = MODE == kHaloRows || MODE == kHaloDirect ? KF_HALO : KF_DENSE;
   launch_begin(family, st);
-  fn<<<grid, kXThreads, smem, st>>>(P);
+  launch_chained(fn, dim3(grid), kXThreads, smem, st, true, P);
   launch_end(family, st);
   return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
 }

@@ -206,3 +206,50 @@ def test_wave_step_with_dissipation_matches_the_banded_one(lib, N, g, offset):
         outs.append([v.cpu().numpy().reshape(4, E, E, E)[:, I, I, I] for v in u])
     for q in range(2):
         assert rel_max(outs[0][q], outs[1][q]) < 1e-7, q
+
+
+@pytest.mark.parametrize("nb,N,nf,graph", [((1, 1, 1), 32, 1, False), ((2, 2, 2), 16, 1, False), ((2, 2, 2), 16, 1, True),
+                                           ((4, 4, 4), 16, 3, False), ((5, 5, 5), 16, 2, False), ((4, 4, 4), 32, 2, False)])
+def test_chained_launches_keep_their_order(lib, nb, N, nf, graph):
+    """Exchanges and applies follow one another without a host synchronisation, each pass on fields that a
+    torch kernel or the apply before it has just written or read: the same bits as with a synchronisation
+    after every call.  Sizes on both sides of the line up to which an exchange is chained."""
+    import torch
+    g, dev = 4, torch.device("cuda", 0)
+    mesh = W.periodic_box_mesh(*nb, N, g)
+    E, nblk, mask = N + 2 * g, nb[0] * nb[1] * nb[2], lib.op_mask(("dx", "dyy", "dz", "dxz", "dyz", "dy"))
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), desc("Q13_1_d2"))
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F64)
+    start = torch.from_numpy(W.rng(nblk + N).uniform(-1, 1, size=nblk * nf * E ** 3)).to(dev)
+    passes, prec = 6, lib.CFD_TC_BF16_EXACT
+    work = torch.empty(max(lib.cfd_apply_workspace(B, nf, mask, prec, 1), 256), dtype=torch.uint8, device=dev)
+
+    def run(sync, fields, outs):
+        for p in range(passes):
+            lib.cfd_exchange_ghosts(B, fields, nf)
+            if sync:
+                torch.cuda.synchronize()
+            lib.cfd_apply(B, fields, nf, mask, prec, 1, outs[p], work)
+            if sync:
+                torch.cuda.synchronize()
+            if p % 2:            # every other pass follows the apply directly
+                fields.mul_(-0.5)
+
+    want = torch.zeros(passes, nblk * nf * 6 * N ** 3, dtype=torch.float64, device=dev)
+    f = start.clone()
+    run(True, f, want)
+    got = torch.zeros_like(want)
+    h = start.clone()
+    torch.cuda.synchronize()
+    if graph:
+        G = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(G):
+            run(False, h, got)
+        h.copy_(start)
+        got.zero_()
+        G.replay()
+    else:
+        run(False, h, got)
+    lib.cfd_sync_status(B)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want) and torch.equal(h, f)
