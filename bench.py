@@ -271,30 +271,24 @@ def _eval_torch(f, X, Y, Z, torch):
 # ------------------------------------------------------------------ algorithmic work
 
 
-def banded_flops_per_step(mesh, nf, mask_ops, n_iter, M=3, h=4, g=4, orders=2):
-    """FP64 flops of the banded path (RHS FMA chains + Thomas sweeps) for one apply; a mixed
-    derivative is solved in ``orders`` orders (2: both, averaged; 1: one order)."""
-    def closed(N, pencils):
-        rows_int, rows_clo = N - 2, 2
-        rhs = rows_int * (2 * (2 * M + 1) - 1) + rows_clo * (2 * (2 * h + 1) - 1)
-        return pencils * (rhs + N + 1 + 3 * (N - 1) + 2 * (N - 1))
-
-    def iterated(N, pencils):
-        rows = N + 2
-        return pencils * (rows * (2 * (2 * M + 1) - 1) + rows + 3 * (N + 3) + 2 * (N + 1))
-
-    def stage(N, pencils):
-        return closed(N, pencils) + n_iter * iterated(N, pencils)
+def banded_flops_per_step(mesh, nf, mask_ops, n_iter, M=3, g=4, orders=2):
+    """FP64 flops of the banded path for one apply, as k_line does it: per row of a solve an odd stencil is M
+    differences and M FMAs, an even one 2M + 1 FMAs and the pivot, and both have one FMA forward and one back;
+    a pass that feeds the neighbours is two rows of the dense operator per pencil.  A mixed derivative is done
+    in ``orders`` orders (2: both, averaged): the inner derivative on the ghost strips (its own points are the
+    d_j output's) and the outer one."""
+    def solve(N, pencils, deg):
+        row = 3 * M + 4 if deg == 1 else 2 * (2 * M + 1) + 5
+        return pencils * ((N + (2 if n_iter else 0)) * row + n_iter * 2 * 2 * (N + 2 * g))
 
     total = 0
     for b in range(mesh.nblocks):
         N = int(mesh.n[b])
-        E = N + 2 * g
         for op in mask_ops:
             if len(op) == 2 or op[1] == op[2]:
-                total += stage(N, N * N)
+                total += solve(N, N * N, len(op) - 1)
             else:
-                total += orders * (stage(N, E * N) + stage(N, N * N)) + (2 * N ** 3 if orders == 2 else 0)
+                total += orders * (solve(N, 2 * g * N, 1) + solve(N, N * N, 1)) + (2 * N ** 3 if orders == 2 else 0)
     return total * nf
 
 
@@ -1102,12 +1096,14 @@ def run_advect(args, spec):
         pass
     hbm = float(peaks.get("hbm_gbs", 6800.0))
     if prec != cfd.CFD_FP64_BANDED:
-        # k_dense: per axis the field is read once and both biased derivatives written once; each
+        # k_dense: per axis the field is read once and both biased derivatives written once (the exact form,
+        # on calls as large as these workloads: the one that the shift selects); each
         # halo pass of the iteration reads the field again.  The blend kernel reads the
         # upwind derivative of each axis per field, the three shift components once per point,
         # and writes the term.
         elem = fields.element_size()
-        per_pf = 3 * 3 * elem
+        sides = 1 if prec == cfd.CFD_TC_BF16_EXACT else 2
+        per_pf = 3 * (1 + sides) * elem
         ach = per_pf * units * prof_steps / (tdl * 1e-3) / 1e9
         nhl, thl = prof["dense_halo"]
         comb_b = (3 + 1 + 3 / nf) * elem * units * prof_steps
