@@ -295,9 +295,6 @@ cfd_status apply_banded(cfd_blocks_s *B, const void *fields, int nf, unsigned ma
       cyc[a] = n == blocks.size();
       some[a] = n > 0 && !cyc[a];
     }
-    int W = 0;
-    for (int d = 0; d < 2; ++d)
-      if (B->s[d].present) W = std::max(W, std::max(B->s[d].h, B->s[d].M + 1));
     auto half_width = [&](const PencilTask &t) { return B->s[t.tab - tabs >= 6 ? 1 : 0].M; };
     // tasks in as few launches as their number and the halo space allow
     auto run = [&](std::vector<PencilTask> ts, double *hbase, size_t hcap) -> cfd_status {
@@ -336,7 +333,7 @@ cfd_status apply_banded(cfd_blocks_s *B, const void *fields, int nf, unsigned ma
             t.halo_out = off[k - i] + (bufs == 2 ? (pass & 1) * len : 0);
             A.task[A.ntask++] = t;
           }
-          cfd_status s = launch_pencils(A, hp, f32, N, half_width(ts[i]), W, st);
+          cfd_status s = launch_pencils(A, hp, f32, N, half_width(ts[i]), st);
           if (s != CFD_OK) return s;
         }
         i = j;

@@ -393,12 +393,19 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
 
 }  // namespace
 
-cfd_status launch_pencils(const PencilArgs &A, bool halo, bool f32, int N, int M, int W, cudaStream_t st) {
+cfd_status launch_pencils(const PencilArgs &A, bool halo, bool f32, int N, int M, cudaStream_t st) {
+  // Windows of the launch's own tasks: W <= 5 (the widths apply_banded admits) keeps N = 32 within the 48 KB
+  // that need no opt-in; a scheme's other degree may be wider.
   long long most = 0;
-  for (int t = 0; t < A.ntask; ++t) most = std::max(most, (long long)A.task[t].n1 * A.task[t].n2 * A.nblk * A.nf);
+  int W = 0;
+  for (int t = 0; t < A.ntask; ++t) {
+    most = std::max(most, (long long)A.task[t].n1 * A.task[t].n2 * A.nblk * A.nf);
+    W = std::max(W, A.task[t].W);
+  }
   if (most == 0 || A.ntask == 0) return CFD_OK;
   const dim3 grid((unsigned)((most + kLineWarps * 32 - 1) / (kLineWarps * 32)), (unsigned)A.ntask);
   const size_t smem = ((size_t)kLineWarps * (N + 2 * W) * kPitch + kTabDoubles) * sizeof(double);
+  static_assert(((size_t)kLineWarps * (kMaxN + 2 * 5) * kPitch + kTabDoubles) * sizeof(double) <= 48 * 1024, "no opt-in");
   void (*fn)(const __grid_constant__ PencilArgs) = nullptr;
   switch (halo ? 0 : M) {
     case 0: fn = f32 ? k_line<float, 0> : k_line<double, 0>; break;

@@ -38,7 +38,7 @@ struct PencilArgs {
 };
 
 // halo: the values the neighbours read (rows 1 and N-2 of this pass's iterate); else the solve.  M: the
-// interior half-width of every task of the launch, W: the widest window.
-cfd_status launch_pencils(const PencilArgs &A, bool halo, bool f32, int N, int M, int W, cudaStream_t st);
+// interior half-width of every task of the launch.
+cfd_status launch_pencils(const PencilArgs &A, bool halo, bool f32, int N, int M, cudaStream_t st);
 
 }  // namespace cfd

@@ -105,3 +105,19 @@ def test_op_subsets_and_fp32_agree_with_fp64(lib, ops, n_iter):
         want = full[:, :, OPS.index(op)]
         assert rel_max(some[:, :, i], want) < 1e-13, op
         assert rel_max(f32[:, :, i], want) < 2e-6, op
+
+
+@pytest.mark.parametrize("N,g,wide", [(32, 6, 2), (32, 6, 1), (16, 6, 2), (32, 8, 2)])
+def test_a_wider_stencil_of_the_other_degree_changes_nothing(lib, N, g, wide):
+    """A scheme whose other degree has the widest closure there is (half-width 6): the requested degree's
+    solves are the same bits as with the ordinary scheme, and the call is accepted as such."""
+    mesh = W.periodic_box_mesh(2, 1, 1, N, g)
+    flat = field(mesh, 1, 31 + N)
+    d = [desc("Q13_1_d1"), desc("Q13_1_d2")]
+    ops = ("dx", "dy", "dz", "dxy") if wide == 2 else ("dxx", "dyy", "dzz")
+    want = run(lib, *d, mesh.n, mesh.dx, mesh.neighbors, g, flat, 1, ops, 1)
+    c = d[wide - 1]["closure"]
+    pad = [0.0] * ((13 - len(c)) // 2)
+    d[wide - 1] = dict(d[wide - 1], closure=pad + list(c) + pad)
+    got = run(lib, *d, mesh.n, mesh.dx, mesh.neighbors, g, flat, 1, ops, 1)
+    assert np.array_equal(got, want)
