@@ -807,6 +807,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       bool issued = false;
       int it = 0;
       if (!mbar_wait_bounded(b_full, 0u, WL)) failed = true;
+      // (it touches no global memory, but the limit of its first wait for a tile must not count the time that
+      // the launch before still takes: the producers are held until then)
+      chain_wait();
       for (int tile = tr.first; tile < tr.end; tile += tr.step, ++it) {
         const int buf = it & 1, tb = it & (nbuf - 1), tu = nbuf == 2 ? it >> 1 : it >> 2;
         if (failed || !mbar_wait_bounded(a_full(buf), (uint32_t)((it >> 1) & 1), WL) ||
