@@ -342,7 +342,10 @@ __device__ __forceinline__ void rows_upwind(uint32_t taddr, uint32_t lev, uint32
 // [own | lower | upper], and so are the operator's).  No intermediate is written or read: at 256^3, 4
 // fields, the y and z stages drop from 0.45 and 0.49 to 0.38 ms.
 enum ExactMode { kPlain = 0, kHaloRows = 1, kUpwind = 2, kDirect = 3, kHaloDirect = 4 };
-template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE>
+// STG: the staging of the input, 0: P.tma_kind decides, 1: TMA, 2: copies.  x stages have it compiled in: with both
+// in one kernel the copy loop cost the TMA stages up to a tenth (T_x of 16^3 blocks, 22 FP32 fields: 0.172 against
+// 0.150 ms), and without it they are 2 to 5 % faster than before it (256^3, one iteration: 3.12 -> 3.00 ms).
+template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE, int STG>
 __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_constant__ DenseParams P) {
   extern __shared__ __align__(1024) unsigned char smem[];
   constexpr bool GEN = AXIS == 3, HALO = MODE == kHaloRows || MODE == kHaloDirect, UPWIND = MODE == kUpwind,
@@ -357,7 +360,8 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
   const int R = P.rows;
   constexpr int SR = HALO ? 16 : N;  // operator rows of a segment
   const int B_BYTES = kSl * R * KP * 2;
-  const int kind = P.tma_kind, nstg = P.nstg, stg_bytes = P.stg_bytes;
+  // (direct stages have no other staging than TMA)
+  const int kind = STG == 2 ? 0 : (DIRECT || STG == 1 ? 1 : P.tma_kind), nstg = P.nstg, stg_bytes = P.stg_bytes;
   const int nbuf = R > 32 ? 2 : 4, buf_cols = kTmemCols / nbuf;
 
   unsigned char *sA = smem, *sB = smem + 2 * A_BYTES;
@@ -472,21 +476,49 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
     const int in_s1 = P.t1 == 0 ? P.in_start[0] : (P.t1 == 1 ? P.in_start[1] : P.in_start[2]);
     const int in_s2 = P.t2 == 0 ? P.in_start[0] : (P.t2 == 1 ? P.in_start[1] : P.in_start[2]);
     const long long E3 = (long long)E * E * E;
+    // 16-byte rows along x: consecutive threads on consecutive pieces.  A thread per row touches 32 rows per warp
+    // instruction (256^3, 4 fields, S_x staged this way: 0.93 -> 0.46 ms together with the row boxes on the way
+    // out, see plan_out_tma).  Rows that are not aligned stay with a thread per row, element by element: the
+    // spread-out form was up to 1.37 times slower there (16^3 blocks, FP32).
+    auto copy_rows = [&](unsigned char *st, int tile) {
+      constexpr int VE = 16 / ES;
+      const int job = fdiv(tile, P.inv_tpj), p0 = (tile - job * P.tiles_per_job) * kTile, np = P.n1 * P.n2;
+      const int lb = fdiv(job, P.inv_nf), q = job - lb * P.nf;
+      const TI *in = static_cast<const TI *>(P.in) +
+                     (!P.in_field ? (long long)job * (long long)P.in_box
+                      : P.contig  ? (long long)P.nf * P.ext0 + (long long)job * E3
+                                  : (long long)P.nf * P.extpre[P.blocks[lb]] + (long long)q * E3);
+      const int per = E / VE;            // pieces of a row
+      const int dp = kXProd / per, dr = kXProd - dp * per;
+      int pp = tid / per, r = tid - pp * per;
+      while (pp < kTile) {
+        const int p = p0 + pp;
+        if (p < np) {
+          const int t1 = fdiv(p, P.inv_n2), t2 = p - t1 * P.n2;
+          cp_async16(st + stg_byte(pp, r * VE), in + (long long)(in_s1 + t1) * s_t1 + (long long)(in_s2 + t2) * s_t2 + r * VE);
+        }
+        pp += dp;
+        r += dr;
+        if (r >= per) {
+          r -= per;
+          ++pp;
+        }
+      }
+    };
     auto prefetch = [&](int tile, int sb) {
-      const int pp = tid & (kTile - 1), jq = tid >> 7;
-      const TileCoord c = tile_coord(P, tile, pp);
       unsigned char *st = stg0 + sb * stg_bytes;
-      if (c.valid) {
-        const long long job = (long long)c.lb * P.nf + c.q;
-        const long long ib = (!P.in_field ? job * (long long)P.in_box
-                              : P.contig  ? (long long)P.nf * P.ext0 + job * E3
-                                          : (long long)P.nf * P.extpre[c.b] + (long long)c.q * E3) +
-                             (long long)(in_s1 + c.t1) * s_t1 + (long long)(in_s2 + c.t2) * s_t2;
-        const TI *src = static_cast<const TI *>(P.in) + ib;
-        if (P.xrow) {
-          constexpr int VE = 16 / ES;
-          for (int j = jq * VE; j < E; j += 2 * VE) cp_async16(st + stg_byte(pp, j), src + j);
-        } else {
+      if (axis == 2 && P.xrow) {
+        copy_rows(st, tile);
+      } else {
+        const int pp = tid & (kTile - 1), jq = tid >> 7;
+        const TileCoord c = tile_coord(P, tile, pp);
+        if (c.valid) {
+          const long long job = (long long)c.lb * P.nf + c.q;
+          const long long ib = (!P.in_field ? job * (long long)P.in_box
+                                : P.contig  ? (long long)P.nf * P.ext0 + job * E3
+                                            : (long long)P.nf * P.extpre[c.b] + (long long)c.q * E3) +
+                               (long long)(in_s1 + c.t1) * s_t1 + (long long)(in_s2 + c.t2) * s_t2;
+          const TI *src = static_cast<const TI *>(P.in) + ib;
           for (int j = jq; j < E; j += 2) {
             if constexpr (ES == 8) cp_async8(st + stg_byte(pp, j), src + (long long)j * s_ax);
             else cp_async4(st + stg_byte(pp, j), src + (long long)j * s_ax);
@@ -735,9 +767,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_dense_exact(const __grid_const
       auto box_store = [&](int op, int o) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) {
-          const int job = c.lb * P.nf + c.q;
-          const int row = (job * P.nops + op) * N * N + tile_pencil(P, tile, quad * 32);
+        if (lane == 0) {  // (fb: this pencil's row of op 0; every block starts at a multiple of 512 values)
+          const unsigned long long at = reinterpret_cast<char *>(fb) - static_cast<char *>(P.out);
+          const int row = (int)(at / (N * sizeof(TO))) + op * N * N;
           asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.tile.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
                            reinterpret_cast<uint64_t>(&P.tmap_out)),
                        "r"(o), "r"(row), "r"(smem_u32(box))

@@ -32,8 +32,8 @@ size_t plan_smem(DenseParams &P) {
   return std::max(fixed + out + (size_t)P.nstg * P.stg_bytes, (size_t)116 * 1024);
 }
 
-template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE = kPlain>
-cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
+template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE, int STG>
+cfd_status launch_staged(DenseParams P, unsigned grid, cudaStream_t st) {
   const size_t smem = plan_smem<TI, N>(P);
   // The shared-memory opt-in is made once per device and instantiation, for the most any launch may
   // need, so later calls issue nothing but the launch (a stream under capture sees kernel nodes only).
@@ -41,7 +41,7 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   int dev = 0;
   cfd_status s = cuda_fail(cudaGetDevice(&dev), "cudaGetDevice");
   if (s != CFD_OK) return s;
-  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER, MODE>;
+  auto fn = k_dense_exact<TI, TO, N, AXIS, ITER, MODE, STG>;
   if (dev < 0 || dev >= 64 || !opted[dev].load()) {
     s = cuda_fail(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax),
                   "cudaFuncSetAttribute");
@@ -54,6 +54,16 @@ cfd_status launch_one(DenseParams P, unsigned grid, cudaStream_t st) {
   launch_chained(fn, dim3(grid), kXThreads, smem, st, true, P);
   launch_end(family, st);
   return cuda_fail(cudaGetLastError(), "k_dense_exact launch");
+}
+
+template <typename TI, typename TO, int N, int AXIS, bool ITER, int MODE = kPlain>
+cfd_status launch_one(const DenseParams &P, unsigned grid, cudaStream_t st) {
+  if constexpr (AXIS != 2 || MODE == kDirect || MODE == kHaloDirect) {
+    return launch_staged<TI, TO, N, AXIS, ITER, MODE, 0>(P, grid, st);
+  } else {
+    return P.tma_kind ? launch_staged<TI, TO, N, AXIS, ITER, MODE, 1>(P, grid, st)
+                      : launch_staged<TI, TO, N, AXIS, ITER, MODE, 2>(P, grid, st);
+  }
 }
 
 // Ghost width 4 has the axis compiled in; other widths share one instantiation per type.

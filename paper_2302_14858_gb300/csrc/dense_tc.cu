@@ -1531,20 +1531,23 @@ void plan_tma(DenseParams &P, size_t elem, bool exact) {
   P.tma_zstep = d0;
 }
 
-// The exact form's x stages write their outputs by TMA (boxes of 8 values x 32 pencils) where the
-// tile's pencils are consecutive rows of an output aligned to 16 bytes.
-void plan_out_tma(DenseParams &P, size_t elem) {
+// The exact form's x stages write their outputs by TMA (boxes of 8 values x 32 pencils) where a tile's pencils
+// are consecutive rows of an output aligned to 16 bytes: every block's interior pencils are, whatever the
+// order of the block ids and the staging of the input.  The output is a tensor of rows of N values up to the
+// group's last block (blocks start at multiples of 8^3 values).  With rows
+// stored by the lanes the x stages of 448 x 16^3 and 64 x 32^3 blocks in alternating order (4 fields, two degrees)
+// took 0.268 ms against 0.140.
+void plan_out_tma(DenseParams &P, size_t elem, long long int_end) {
   P.out_box_bytes = 0;
-  if (P.axis != 2 || !P.tma_kind || !P.contig || !P.xvec) return;
+  if (P.axis != 2 || !P.xvec) return;
   if (P.n1 != P.N || P.n2 != P.N || P.int_lo1 != 0 || P.int_lo2 != 0 || P.int_hi1 != P.N || P.int_hi2 != P.N) return;
-  const unsigned long long rows = (unsigned long long)P.nblk * P.nf * P.nops * P.N * P.N;
+  const unsigned long long rows = (unsigned long long)int_end * P.nf * P.nops / P.N;
   if (rows >= (1ull << 31)) return;
   EncodeTiledFn enc = tensor_map_encoder();
   if (!enc) return;
-  char *base = static_cast<char *>(P.out) + (size_t)P.nf * P.nops * P.int0 * elem;
   const cuuint64_t gdim[2] = {(cuuint64_t)P.N, (cuuint64_t)rows}, gstr[1] = {(cuuint64_t)P.N * elem};
   const cuuint32_t box[2] = {8, 32}, estr[2] = {1, 1};
-  if (enc(&P.tmap_out, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, gdim,
+  if (enc(&P.tmap_out, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, P.out, gdim,
           gstr, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
           elem == 8 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -1592,7 +1595,7 @@ void set_launch_constants(DenseParams &P) {
 // with events on the stream, and keep the fastest.  Repeated launches of a stage are idempotent
 // (a stage never reads what it writes), and every candidate computes the same outputs.
 cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int L, size_t ein, bool f32,
-                        unsigned grid, cudaStream_t st) {
+                        unsigned grid, long long int_end, cudaStream_t st) {
   const bool exact = S == 4;
   auto launch = [&](DenseParams Q) -> cfd_status {
     if (exact) {
@@ -1616,7 +1619,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
     if (Q.direct) plan_direct(Q);  // (checked before the stage was made)
     else if (staging == 0) plan_tma(Q, ein, exact);
     else { Q.tma_kind = 0; Q.tma_boxes = 0; }
-    if (exact) plan_out_tma(Q, f32 ? 4 : 8);
+    if (exact) plan_out_tma(Q, f32 ? 4 : 8, int_end);
     return Q;
   };
   const int idx = ds->launch++;
@@ -1775,6 +1778,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
     base.out = out;
     base.seg_rows = N;
     base.kext = E;
+    long long int_end = 0;  // end of the group's last block
     {
       const std::vector<int> &gb = B->groups[gi];
       bool contig = true;
@@ -1784,6 +1788,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
       base.b0 = gb[0];
       base.ext0 = B->extpre[gb[0]];
       base.int0 = B->intpre[gb[0]];
+      int_end = B->intpre[gb.back()] + (long long)N * N * N;
     }
     base.nbr = B->d_nbr;
     base.halo_deg_mask = (B->s[0].present ? 1 : 0) | (B->s[1].present ? 2 : 0);
@@ -1797,7 +1802,7 @@ cfd_status dense_apply(cfd_blocks_s *B, const void *fields, int nf, unsigned mas
       P.tiles_per_job = (np + kTile - 1) / kTile;
       P.ntiles = P.tiles_per_job * P.nblk * P.nf;
       const unsigned grid = (unsigned)std::min(P.ntiles, sms);
-      return launch_stage(ds, P, G.Kp, S, L, ein, f32, grid, st);
+      return launch_stage(ds, P, G.Kp, S, L, ein, f32, grid, int_end, st);
     };
     // segments: (degree, mode, op); passes of at most 32 rows
     auto iterating = [&](int box) { return n_iter > 0 && !G.cyc[box]; };
@@ -2112,6 +2117,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
     if (upwind) group_signs += (size_t)base.nblk * 3 * N * N;
     base.seg_rows = N;
     base.kext = E;
+    long long int_end = 0;  // end of the group's last block
     {
       const std::vector<int> &gb = B->groups[gi];
       bool contig = true;
@@ -2121,6 +2127,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       base.b0 = gb[0];
       base.ext0 = B->extpre[gb[0]];
       base.int0 = B->intpre[gb[0]];
+      int_end = B->intpre[gb.back()] + (long long)N * N * N;
     }
     base.nbr = B->d_nbr;
     base.halo_deg_mask = 3;   // both halo slots pairs: S+ (columns E, E+1), S- (E+2, E+3)
@@ -2134,7 +2141,7 @@ cfd_status dense_biased(cfd_blocks_s *B, const void *fields, int nf, const void 
       P.tiles_per_job = (np + kTile - 1) / kTile;
       P.ntiles = P.tiles_per_job * P.nblk * P.nf;
       const unsigned grid = (unsigned)std::min(P.ntiles, sms);
-      return launch_stage(ds, P, G.Kp, S, L, ein_b, f32, grid, st);
+      return launch_stage(ds, P, G.Kp, S, L, ein_b, f32, grid, int_end, st);
     };
     for (int i = 0; i < naxes; ++i) {
       const int box = axes[i];

@@ -253,3 +253,85 @@ def test_chained_launches_keep_their_order(lib, nb, N, nf, graph):
     lib.cfd_sync_status(B)
     torch.cuda.synchronize()
     assert torch.equal(got, want) and torch.equal(h, f)
+
+
+def interleaved(g, nf, seed, np_t):
+    """Eight 16^3 and three 32^3 blocks, each size a periodic box of its own, in an order that keeps neither
+    size's blocks together: (n, dx, neighbours, per-block samples of nf + 3 fields)."""
+    from types import SimpleNamespace
+    parts = []
+    for k, (nb, N) in enumerate((((2, 2, 2), 16), ((1, 3, 1), 32))):
+        mesh = W.periodic_box_mesh(*nb, N, g)
+        L = [nb[a] * N * mesh.dx[0, a] for a in range(3)]
+        r = W.rng(seed + k)
+        fs = []
+        for _ in range(nf + 3):
+            s = W.sine_sum(r, 6, 1, 3)
+            s.k = 2 * np.pi * s.k / np.asarray(L)
+            fs.append(s)
+        parts.append((mesh, W.sample(mesh, fs, np_t)))
+    (a, fa), (b, fb) = parts
+    order = np.array([0, 8, 1, 2, 3, 9, 4, 5, 10, 6, 7])    # position -> block of (a, b)
+    where = np.argsort(order)
+    nbr = np.concatenate([np.asarray(a.neighbors), np.asarray(b.neighbors) + 8])
+    return SimpleNamespace(n=np.concatenate([a.n, b.n])[order], dx=np.concatenate([a.dx, b.dx])[order],
+                           neighbors=where[nbr][order].astype(np.int32), fields=[(fa + fb)[i] for i in order])
+
+
+@pytest.mark.parametrize("g,dtype,nf,n_iter,offset", [
+    (4, "f64", 2, 0, 0), (4, "f64", 1, 1, 0), (4, "f32", 3, 0, 0), (4, "f32", 2, 1, 0), (4, "f64", 2, 0, 1),
+    (5, "f64", 1, 0, 0), (6, "f32", 1, 0, 0),
+])
+def test_sizes_that_alternate_in_block_order(lib, g, dtype, nf, n_iter, offset):
+    """Block ids of one size that are not consecutive: inputs staged by element or 16-byte copies, offsets from
+    the tables, x outputs as row boxes of the whole output.  Apply against the banded solve, and (where the
+    biased windows take the ghost width) the upwinded shift term."""
+    import torch
+    from tests.helpers import SCHEMES
+    np_t, t_t = (np.float32, torch.float32) if dtype == "f32" else (np.float64, torch.float64)
+    m = interleaved(g, nf, 500 + g + n_iter, np_t)
+    dev = torch.device("cuda", 0)
+
+    def put(a):
+        hold = torch.zeros(a.size + 8, dtype=t_t, device=dev)
+        v = hold[offset:offset + a.size]
+        v.copy_(torch.from_numpy(np.ascontiguousarray(a, np_t)))
+        return v
+
+    fields = put(np.concatenate([b[:nf].reshape(-1) for b in m.fields]))
+    shift = put(np.concatenate([b[nf:].reshape(-1) for b in m.fields]))
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), desc("Q13_1_d2"))
+    lib.cfd_scheme_set_biased(s, SCHEMES["X2_d1"])
+    B = lib.cfd_blocks_bind(s, m.n, m.dx, m.neighbors, g, lib.CFD_F32 if dtype == "f32" else lib.CFD_F64)
+    tol = 2e-6 if dtype == "f32" else 1e-7
+    nint = sum(int(v) ** 3 for v in m.n)
+
+    def call(what, prec, nops):
+        buf = torch.full((nint * nf * nops + 8,), float("nan"), dtype=t_t, device=dev)
+        out = buf[offset:offset + nint * nf * nops]
+        if what == "apply":
+            need = lib.cfd_apply_workspace(B, nf, lib.CFD_OP_ALL, prec, n_iter)
+        else:
+            need = lib.cfd_biased_workspace(B, nf, prec, n_iter)
+        work = torch.empty(max(need, 256), dtype=torch.uint8, device=dev)
+        if what == "apply":
+            lib.cfd_apply(B, fields, nf, lib.CFD_OP_ALL, prec, n_iter, out, work)
+        elif what == "advect":
+            lib.cfd_advect(B, fields, nf, shift, prec, n_iter, out, work)
+        else:
+            lib.cfd_apply_biased(B, fields, nf, 7, 1, prec, n_iter, out, work)
+        lib.cfd_sync_status(B)
+        flat, at, per = out.double().cpu().numpy(), 0, {}
+        for v in m.n:  # [size][op]: the group's blocks and fields
+            k = nf * nops * int(v) ** 3
+            per.setdefault(int(v), []).append(flat[at:at + k].reshape(nf, nops, -1))
+            at += k
+        return {N: np.stack(v) for N, v in per.items()}
+
+    for what, nops in (("apply", 9),) + ((("advect", 1), ("biased", 3)) if g in (4, 6) else ()):
+        got, want = call(what, lib.CFD_TC_BF16_EXACT, nops), call(what, lib.CFD_FP64_BANDED, nops)
+        for N in got:
+            for q in range(nf):
+                for i in range(nops):
+                    e = rel_max(got[N][:, q, i], want[N][:, q, i])
+                    assert e < tol, (what, N, q, i, e)
