@@ -68,6 +68,7 @@ struct BiasedParams {
   int mode;                // 0 d[S+], 1 d[S-], 2 advect (beta_+ d[S+] + beta_- d[S-])
   int accum;               // 1: add into out
   int pass, last;
+  int cyclic;              // some block is its own neighbour along the axis
 };
 
 void build_biased_tables(const BiasedCoef &c, int N, int g, BiasedTables &T);
