@@ -90,21 +90,23 @@ struct PencilTab {
   int W;                 // points needed beyond the block on each side: max(h, M + 1)
   int anti;              // degree 1 with exactly antisymmetric coefficients: differences of pairs
   int unscaled;          // spacing differs between blocks: results are multiplied per block
-  double neg, nil;       // -1 and 0 (see stencil() in line.cu)
-  double factor;         // folded into the results (1, or 1/2 for one half of an averaged pair)
+  // scalars, copied as one run (kTabScalars): -1 and 0 (see stencil() in line.cu); the factor folded into the
+  // results (1, or 1/2 for one half of an averaged pair); scale of rows that keep their coefficients (1: folded)
+  // and its reciprocal; factor of the upper fixed value; cyclic system: a and the Sherman-Morrison factor
+  double neg, nil, factor, sc, isc, hhi, a, vfac;
   double clo[2 * kMaxH + 1];
-  double sc, isc;        // scale of rows that keep their coefficients (1: folded), and its reciprocal
   // closed system (rows 1..N-2; rows 0 and N-1 are the closures): row k
   //   z_k = sum_m rc[k][m + M] f_{k+m} - lo[k] z_{k-1},   x_k = pv[k] z_k - up[k] x_{k+1}
   double rc[kMaxN][2 * kMaxM + 1], lo[kMaxN], up[kMaxN], pv[kMaxN];
   // iterated system, rows k = -1..N at k + 1; the fixed values enter the first and last row
-  double irc[kMaxN + 2][2 * kMaxM + 1], ilo[kMaxN + 2], iup[kMaxN + 2], ipv[kMaxN + 2], hhi;
+  double irc[kMaxN + 2][2 * kMaxM + 1], ilo[kMaxN + 2], iup[kMaxN + 2], ipv[kMaxN + 2];
   // cyclic system: Thomas rows of the corner-modified matrix, its Sherman-Morrison vector
-  double yrc[kMaxN][2 * kMaxM + 1], ylo[kMaxN], yup[kMaxN], ypv[kMaxN], z[kMaxN], a, vfac;
+  double yrc[kMaxN][2 * kMaxM + 1], ylo[kMaxN], yup[kMaxN], ypv[kMaxN], z[kMaxN];
   // rows 1 and N-2 of the closed and of the iterated operator over the window (index j + W for point
   // j), and the coefficients of the fixed values: what the neighbours read (factor 1 always)
   double hrow[2][2][kMaxN + 2 * kMaxH + 2], hc[2][2];
 };
+constexpr int kTabScalars = 8;
 }  // namespace cfd
 
 struct cfd_scheme_s {

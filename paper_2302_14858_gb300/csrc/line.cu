@@ -5,19 +5,23 @@
 // other instruction hides behind that, so the kernel is written for few FP64 operations and enough
 // warps, not for few instructions:
 //   - the pencil sits in shared memory ([point][lane], 33 lanes wide: conflict-free along either
-//     index), rows run in rolled loops with few registers, 20 to 36 warps per SM;
+//     index), rows run in rolled loops with few registers, 16 to 24 warps per SM;
 //   - a row is its stencil (three differences and three FMAs for an odd stencil with M = 3, seven FMAs
 //     for an even one), one FMA forward and one back, and for an even stencil the pivot (line.h): 8 or
 //     10 operations, 11 before;
 //   - the passes of the hybrid iteration that only feed the neighbours compute the two values the
 //     neighbours read, as two rows of the dense operator (~2 N FMAs per pencil instead of a solve);
 //   - along x, pencils are rows: a warp loads and stores its 32 rows with consecutive lanes on
-//     consecutive points and turns them in shared memory.
+//     consecutive points and turns them in shared memory;
+//   - pencils and tables arrive by asynchronous copies, all in flight at once.
 // Mixed derivatives take the inner derivative from the d_j output (or one FP64 copy of it) and only
 // the ghost strips are solved again, where the version before solved the extended pencils for each of
-// the six ordered pairs.  128^3 as 512 blocks of 16^3, 4 fields, nine ops, one iteration: 8.41 -> 3.65 ms
-// (526 -> ~165 FP64 operations per point); 27 blocks of 16^3, one field: 447 -> 192 us in 15 launches
-// instead of 37 (there latency counts: loads go out eight at a time, rows four at a time).
+// the six ordered pairs.  128^3 as 512 blocks of 16^3, 4 fields, nine ops, one iteration: 8.41 -> 3.03 ms
+// (526 -> ~150 FP64 operations per point); 27 blocks of 16^3, one field: 447 -> 162 us in 15 launches
+// instead of 37.  Small launches are a chain of latencies: one op of 2^3 blocks of 8^3 takes 5.5 to 7.2 us
+// (6.3 to 9.0 with loads eight at a time and the table read through registers), of 16^3 8.7 to 10.1 us.
+#include <stddef.h>
+
 #include <algorithm>
 #include <type_traits>
 
@@ -36,7 +40,7 @@ __device__ __forceinline__ int dir_index(int dz, int dy, int dx) {
 
 constexpr int kPitch = 33;   // lanes per point of a warp's tile, padded
 constexpr int kLineWarps = 4;
-constexpr int kTabDoubles = (kMaxN + 2) * (2 * 3 + 1) + 4 * (kMaxN + 2) + 2 * kMaxH + 1;  // M <= 3
+constexpr int kTabDoubles = (kMaxN + 2) * (2 * 3 + 1) + 4 * (kMaxN + 2) + 2 * kMaxH + 1 + kTabScalars;  // M <= 3
 
 // Every operation of the solves is an FMA of three register operands: on GB300 that form issues every
 // 64 cycles per SM sub-partition, an add, a multiply or an FMA with a constant operand every 76
@@ -67,15 +71,26 @@ __device__ __forceinline__ void stencils(double (&r)[R], const double *c, int cw
       for (int u = 0; u < R; ++u) r[u] = fma(c[u * cw + M + m], f[u + M + m], m == -M ? nil : r[u]);
   }
 }
-// a closure row (half-width h <= kMaxH)
-__device__ __forceinline__ double closure_row(const double *c, const double *p, int h, bool anti, double neg, double nil) {
-  double s = nil;
-  if (anti) {
-    for (int m = h; m >= 1; --m) s = fma(c[h + m], fma(p[-m * kPitch], neg, p[m * kPitch]), s);
+// The two closure rows (half-width h), at points p and q: two chains side by side.
+template <bool anti>
+__device__ __forceinline__ void closure_rows(double &s, double &t, const double *c, const double *p, const double *q,
+                                             int h, double neg, double nil) {
+  s = t = nil;
+  if constexpr (anti) {
+#pragma unroll
+    for (int m = 5; m >= 1; --m) {
+      if (m > h) continue;
+      s = fma(c[h + m], fma(p[-m * kPitch], neg, p[m * kPitch]), s);
+      t = fma(c[h + m], fma(q[-m * kPitch], neg, q[m * kPitch]), t);
+    }
   } else {
-    for (int m = -h; m <= h; ++m) s = fma(c[h + m], p[m * kPitch], s);
+#pragma unroll
+    for (int m = -5; m <= 5; ++m) {
+      if (m < -h || m > h) continue;
+      s = fma(c[h + m], p[m * kPitch], s);
+      t = fma(c[h + m], q[m * kPitch], t);
+    }
   }
-  return s;
 }
 
 // Forward sweep over rows k0 .. k0 + n - 1 (n even): z_k = r_k - lo_k z_{k-1}, stored where point k - M
@@ -101,38 +116,55 @@ __device__ __forceinline__ double forward(const double *c, const double *lo, dou
   return z;
 }
 
-// 32 rows (one per lane, pointer `mine`, n elements each) with consecutive lanes on consecutive elements,
-// eight loads in flight: op(row, element, pointer of the row or null) returns what sink takes.
-template <typename P, typename Load, typename Sink>
-__device__ __forceinline__ void for_rows(P *mine, int n, Load load, Sink sink) {
-  const int lane = threadIdx.x & 31;
-  int r = 0, j = lane;
-  for (int i = 0; i < n; i += 8) {
-    double v[8];
-    int rr[8], jj[8];
+// 32 rows (one per lane, pointer `mine`, n elements each) with consecutive lanes on consecutive elements:
+// f(pointer of the row, row, element) for the rows that are not null, U of them side by side.
+template <int U, typename P, typename F>
+__device__ __forceinline__ void for_rows(P *mine, int n, F f) {
+  const int dr = 32 / n, dj = 32 - dr * n, lane = threadIdx.x & 31;
+  int r = lane / n, j = lane - r * n;
+  for (int i = 0; i < n; i += U) {
+    P *row[U];
+    int rr[U], jj[U];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      while (j >= n) { j -= n; ++r; }
+    for (int u = 0; u < U; ++u) {
       rr[u] = r & 31;
       jj[u] = j;
-      j += 32;
-      P *row = reinterpret_cast<P *>(__shfl_sync(0xffffffffu, (long long)mine, rr[u]));
-      v[u] = 0.0;
-      if (i + u < n && row) v[u] = load(row, rr[u], jj[u]);
+      row[u] = reinterpret_cast<P *>(__shfl_sync(0xffffffffu, (long long)mine, rr[u]));
+      if (i + u >= n) row[u] = nullptr;
+      r += dr;
+      j += dj;
+      if (j >= n) {
+        j -= n;
+        ++r;
+      }
     }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      P *row = reinterpret_cast<P *>(__shfl_sync(0xffffffffu, (long long)mine, rr[u]));
-      if (i + u < n && row) sink(row, rr[u], jj[u], v[u]);
-    }
+    f(row, rr, jj);
   }
+}
+
+// Copies that need no register until the wait: a launch of few warps has a whole pencil and its table in
+// flight at once (eight loads at a time took a memory latency per batch).
+__device__ __forceinline__ void copy_async(double *dst, const double *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async(double *dst, const float *src) {  // (into the low half: widened later)
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+
+// (double)f by integer instructions for zeros and normal values (a conversion holds the FP64 pipe for 64 cycles).
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = u & 0x7F800000u;
+  if ((e == 0 && (u << 1) != 0) || e == 0x7F800000u) return (double)f;
+  const unsigned hi = (u & 0x80000000u) | (e ? ((u & 0x7FFFFFFFu) >> 3) + (896u << 20) : 0u);
+  return __hiloint2double((int)hi, (int)(u << 29));
 }
 
 // T: field dtype.  M > 0: solve (interior half-width M); M = 0: a halo pass, which writes the two values
 // the neighbours read.  The table's part that the CTA needs is copied to shared memory first (read row by
-// row from memory it cost a miss per row: half the time of a small launch).
+// row from memory it cost a miss per row: half the time of a small launch).  Registers: with 80 allowed
+// (6 CTAs per SM) the 128^3 case takes 3.03 ms; left to itself the compiler takes 64 and spills, 3.21.
 template <typename T, int M>
-__global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant__ PencilArgs A) {
+__global__ void __launch_bounds__(kLineWarps * 32, 6) k_line(const __grid_constant__ PencilArgs A) {
   extern __shared__ double line_smem[];
   const PencilTask &K = A.task[blockIdx.y];
   const PencilTab &tab = *K.tab;
@@ -142,15 +174,45 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
   constexpr bool HALO = M == 0;
   constexpr int CW = 2 * M + 1;
   // shared: closed or iterated rows [N + 2][CW], lo, up [N + 2] each, closure; cyclic rows, lo, up, z
-  // (halo passes: the two operator rows); then a tile per warp
+  // (halo passes: the two operator rows), the scalars; then a tile per warp
   double *s_rc = line_smem, *s_lo = s_rc + (kMaxN + 2) * CW, *s_up = s_lo + kMaxN + 2, *s_clo = s_up + kMaxN + 2,
-         *s_z = s_clo + 2 * kMaxH + 1, *s_pv = s_z + kMaxN + 2;
+         *s_z = s_clo + 2 * kMaxH + 1, *s_pv = s_z + kMaxN + 2, *s_k = s_pv + kMaxN + 2;
   double *tile = line_smem + kTabDoubles + (threadIdx.x >> 5) * (L * kPitch);
   const int np = K.n1 * K.n2;
-  const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if ((long long)blockIdx.x * blockDim.x >= (long long)np * A.nblk * A.nf) return;  // (whole CTAs)
-  bool valid = id < (long long)np * A.nblk * A.nf;
-  const int job = valid ? (int)(id / np) : 0, p = valid ? (int)(id - (long long)job * np) : 0;
+  // (the entry points admit 65535 blocks x fields of a size: fewer than 2^27 pencils)
+  const int id = (int)(blockIdx.x * blockDim.x + threadIdx.x), npen = np * A.nblk * A.nf;
+  if ((int)(blockIdx.x * blockDim.x) >= npen) return;  // (whole CTAs)
+  bool valid = id < npen;
+  const int job = valid ? id / np : 0, p = valid ? id - job * np : 0;
+  // the table's part, in flight while the pencils are fetched; one barrier for both
+  {
+    const int t = threadIdx.x;
+    if (HALO) {
+      constexpr int HW = sizeof(tab.hrow[0][0]) / sizeof(double);
+      const double *h = &tab.hrow[A.pass > 0][0][0];
+      for (int i = t; i < 2 * HW; i += blockDim.x) copy_async(s_rc + i, h + i);
+      if (t < 4) copy_async(s_k + t, &tab.hc[0][0] + t);
+    } else {
+      const bool iter = !cyc && A.pass > 0;
+      const double(*rc)[2 * kMaxM + 1] = cyc ? tab.yrc : (iter ? tab.irc : tab.rc);
+      const double *lo = cyc ? tab.ylo : (iter ? tab.ilo : tab.lo);
+      const double *up = cyc ? tab.yup : (iter ? tab.iup : tab.up);
+      const double *pv = cyc ? tab.ypv : (iter ? tab.ipv : tab.pv);
+      const int rows = iter ? N + 2 : N;
+      for (int i = t; i < rows * CW; i += blockDim.x) copy_async(s_rc + i, &rc[i / CW][i % CW]);
+      if (t < rows) {
+        copy_async(s_lo + t, lo + t);
+        copy_async(s_up + t, up + t);
+        copy_async(s_pv + t, pv + t);
+        if (cyc) copy_async(s_z + t, &tab.z[t]);
+      } else if (t >= 64 && t <= 64 + 2 * kMaxH) {
+        copy_async(s_clo + t - 64, &tab.clo[t - 64]);
+      } else if (t >= 96 && t < 96 + kTabScalars) {
+        static_assert(offsetof(PencilTab, vfac) == offsetof(PencilTab, neg) + (kTabScalars - 1) * sizeof(double), "one run");
+        copy_async(s_k + t - 96, &tab.neg + (t - 96));
+      }
+    }
+  }
   const int lb = job / A.nf, q = job - lb * A.nf, b = A.blocks[lb];
   const int i1 = p / K.n2, i2 = p - i1 * K.n2;
   // transverse point relative to the block's own points
@@ -165,38 +227,20 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
   const int blo = look ? A.nbr[b * 26 + dir_index(-(ax == 0), -(ax == 1), -(ax == 2))] : 0;
   const int bhi = look ? A.nbr[b * 26 + dir_index(ax == 0, ax == 1, ax == 2)] : 0;
   if (K.only) valid = valid && (blo == b && bhi == b) == (K.only == 1);
-  // (copied while the pencils are fetched; one barrier for both)
-  if (HALO) {
-    const double *h = &tab.hrow[A.pass > 0][0][0];
-    constexpr int HW = sizeof(tab.hrow[0][0]) / sizeof(double);
-    for (int i = threadIdx.x; i < 2 * HW; i += blockDim.x) s_rc[i] = __ldg(h + i);
-  } else {
-    const double(*rc)[2 * kMaxM + 1] = cyc ? tab.yrc : (A.pass > 0 ? tab.irc : tab.rc);
-    const double *lo = cyc ? tab.ylo : (A.pass > 0 ? tab.ilo : tab.lo);
-    const double *up = cyc ? tab.yup : (A.pass > 0 ? tab.iup : tab.up);
-    const double *pv = cyc ? tab.ypv : (A.pass > 0 ? tab.ipv : tab.pv);
-    const int rows = !cyc && A.pass > 0 ? N + 2 : N;
-    for (int i = threadIdx.x; i < rows * CW; i += blockDim.x) s_rc[i] = __ldg(&rc[i / CW][i % CW]);
-    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-      s_lo[i] = __ldg(lo + i);
-      s_up[i] = __ldg(up + i);
-      s_pv[i] = __ldg(pv + i);
-      if (cyc) s_z[i] = __ldg(&tab.z[i]);
-    }
-    if (threadIdx.x <= 2 * kMaxH) s_clo[threadIdx.x] = __ldg(&tab.clo[threadIdx.x]);
-  }
-
   // ---- the pencil: points -W .. N+W-1 at tile entries 0 .. L-1
   if (!K.gather) {
     const T *src = static_cast<const T *>(A.field) + (long long)A.nf * A.extpre[b] + (long long)q * E * E * E +
                    (c1 + g) * stride(K.t1, E) + (c2 + g) * stride(K.t2, E) + (long long)(g - W) * stride(ax, E);
     if (ax == 2) {
-      for_rows(valid ? src : nullptr, L, [](const T *row, int, int k) { return (double)__ldg(row + k); },
-               [&](const T *, int r, int k, double v) { tile[k * kPitch + r] = v; });
+      for_rows<4>(valid ? src : nullptr, L, [&](const T *const(&row)[4], const int(&r)[4], const int(&k)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row[u]) copy_async(tile + k[u] * kPitch + r[u], row[u] + k[u]);
+      });
     } else if (valid) {
       const int s = stride(ax, E);
 #pragma unroll 8
-      for (int j = 0; j < L; ++j) tile[j * kPitch + lane] = (double)__ldg(src + (long long)j * s);
+      for (int j = 0; j < L; ++j) copy_async(tile + j * kPitch + lane, src + (long long)j * s);
     }
   } else {
     // own points of the inner derivative (FP64: an output slot, or the scratch copy), ghosts from its strip
@@ -204,25 +248,26 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
                                            ((long long)q * A.nops + K.in_op) * n3
                                      : A.region + K.in_off + (long long)job * n3;
     own += c1 * stride(K.t1, N) + c2 * stride(K.t2, N);
-    // (plain loads: the derivative was written by an earlier launch on the stream, but `out` is written here)
     if (ax == 2) {
-      for_rows(valid ? own : nullptr, N, [](const double *row, int, int k) { return row[k]; },
-               [&](const double *, int r, int k, double v) { tile[(W + k) * kPitch + r] = v; });
+      for_rows<4>(valid ? own : nullptr, N, [&](const double *const(&row)[4], const int(&r)[4], const int(&k)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (row[u]) copy_async(tile + (W + k[u]) * kPitch + r[u], row[u] + k[u]);
+      });
     } else if (valid) {
       const int s = stride(ax, N);
 #pragma unroll 8
-      for (int j = 0; j < N; ++j) tile[(W + j) * kPitch + lane] = own[(long long)j * s];
+      for (int j = 0; j < N; ++j) copy_async(tile + (W + j) * kPitch + lane, own + (long long)j * s);
     }
     if (valid) {  // strip layout: [2g ghost points along the axis][N][N] (t1, t2)
       const double *st = A.region + K.strip_off + (long long)job * (2 * g * N * N) + c1 * N + c2;
 #pragma unroll 4
       for (int j = 0; j < W; ++j) {
-        tile[j * kPitch + lane] = st[(long long)(g - W + j) * N * N];
-        tile[(W + N + j) * kPitch + lane] = st[(long long)(g + j) * N * N];
+        copy_async(tile + j * kPitch + lane, st + (long long)(g - W + j) * N * N);
+        copy_async(tile + (W + N + j) * kPitch + lane, st + (long long)(g + j) * N * N);
       }
     }
   }
-  __syncthreads();
   double *f0 = tile + W * kPitch + lane;  // point 0 of this lane's pencil
   const double scale = unscaled ? A.scale[(b * 2 + (K.deg - 1)) * 3 + (2 - ax)] : 1.0;
   // the neighbours' previous iterate at k^c = -2 and N+1 (their rows N-2 and 1)
@@ -237,6 +282,15 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       dhi /= scale;
     }
   }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  if (sizeof(T) == 4 && !K.gather) {
+#pragma unroll 8
+    for (int j = 0; j < L; ++j) {
+      double *e = tile + j * kPitch + lane;
+      *e = widen(*reinterpret_cast<const float *>(e));
+    }
+  }
 
   if constexpr (HALO) {
     if (!valid || cyc) return;
@@ -247,7 +301,7 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       int j = 0;
       constexpr int HW = sizeof(tab.hrow[0][0]) / sizeof(double);
       const double *c = s_rc + w * HW, *f = tile + lane;
-      double s0 = it ? fma(tab.hc[w][0], dlo, tab.hc[w][1] * dhi) : 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+      double s0 = it ? fma(s_k[2 * w], dlo, s_k[2 * w + 1] * dhi) : 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
       for (; j + 4 <= L; j += 4) {
         s0 = fma(c[j], f[j * kPitch], s0);
         s1 = fma(c[j + 1], f[(j + 1) * kPitch], s1);
@@ -265,7 +319,7 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
     auto solve = [&](auto anti_c, auto add_c, auto unscaled_c) {
     constexpr bool anti = decltype(anti_c)::value, ADD = decltype(add_c)::value, UNSCALED = decltype(unscaled_c)::value;
     // ---- solve
-    const double neg = __ldg(&tab.neg), nil = __ldg(&tab.nil), one = -neg;
+    const double neg = s_k[0], nil = s_k[1], factor = s_k[2], sc_k = s_k[3], isc = s_k[4], hhi = s_k[5], one = -neg;
     double *zrow = f0 - M * kPitch;
     const bool closed = !cyc && A.pass == 0;
     double x = 0.0, z = 0.0, x0 = 0.0;
@@ -281,23 +335,22 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
         x = fma(-s_up[k], x, scaled(zrow[k * kPitch], s_pv[k]));
         zrow[k * kPitch] = x;
       }
-      const double s = fma(-tab.a, xn, x) * tab.vfac;   // (x_0 - a x_{N-1}) vfac
+      const double s = fma(-s_k[6], xn, x) * s_k[7];   // (x_0 - a x_{N-1}) vfac
       for (int k = 0; k < N; ++k) zrow[k * kPitch] = fma(-s, s_z[k], zrow[k * kPitch]);
       top = -1;
       up = pv = nullptr;
     } else if (closed) {
-      x0 = closure_row(s_clo, f0, K.h, anti, neg, nil);
-      x = closure_row(s_clo, f0 + (N - 1) * kPitch, K.h, anti, neg, nil);
+      closure_rows<anti>(x0, x, s_clo, f0, f0 + (N - 1) * kPitch, K.h, neg, nil);
       // (the closure rows take a zero times their neighbour, so a NaN or an infinity reaches the whole pencil)
-      x = fma(nil, forward<M, anti>(s_rc + CW, s_lo + 1, f0, 1, N - 2, x0, neg, nil), scaled(x, tab.sc));
-      x0 = scaled(x0, tab.sc);
+      x = fma(nil, forward<M, anti>(s_rc + CW, s_lo + 1, f0, 1, N - 2, x0, neg, nil), scaled(x, sc_k));
+      x0 = scaled(x0, sc_k);
       top = N - 2;
       up = s_up;
       pv = s_pv;
     } else {
       // row -1 starts from the fixed value: z_{-2} enters as hlo / lo times it
-      z = forward<M, anti>(s_rc, s_lo, f0, -1, N + 2, scaled(tab.factor * dlo, tab.isc), neg, nil);
-      x = fma(-tab.hhi, dhi, scaled(z, s_pv[N + 1]));  // row N
+      z = forward<M, anti>(s_rc, s_lo, f0, -1, N + 2, scaled(factor * dlo, isc), neg, nil);
+      x = fma(-hhi, dhi, scaled(z, s_pv[N + 1]));  // row N
       top = N - 1;
       up = s_up + 1;
       pv = s_pv + 1;
@@ -365,17 +418,26 @@ __global__ void __launch_bounds__(kLineWarps * 32) k_line(const __grid_constant_
       __syncwarp();
       const double *row0 = tile + (W - M) * kPitch;
       if (K.sc_off >= 0)
-        for_rows(sc, N, [&](double *, int r, int k) { return row0[k * kPitch + r]; },
-                 [](double *row, int, int k, double v) { row[k] = v; });
-      if (K.out_op >= 0) {
-        for_rows(out, N,
-                 [&](T *row, int r, int k) { 
-                   double v = row0[k * kPitch + r];
-                   if constexpr (ADD) v = fma((double)row[k], one, v);
-                   return v;
-                 },
-                 [](T *row, int, int k, double v) { row[k] = (T)v; });
-      }
+        for_rows<4>(sc, N, [&](double *const(&row)[4], const int(&r)[4], const int(&k)[4]) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            if (row[u]) row[u][k[u]] = row0[k[u] * kPitch + r[u]];
+        });
+      if (K.out_op >= 0)
+        for_rows<8>(out, N, [&](T *const(&row)[8], const int(&r)[8], const int(&k)[8]) {
+          T old[8];
+          if constexpr (ADD) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) old[u] = row[u] ? row[u][k[u]] : T(0);
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            if (!row[u]) continue;
+            double v = row0[k[u] * kPitch + r[u]];
+            if constexpr (ADD) v = fma((double)old[u], one, v);
+            row[u][k[u]] = (T)v;
+          }
+        });
     }
     };
     using std::false_type;

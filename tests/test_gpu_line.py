@@ -121,3 +121,24 @@ def test_a_wider_stencil_of_the_other_degree_changes_nothing(lib, N, g, wide):
     d[wide - 1] = dict(d[wide - 1], closure=pad + list(c) + pad)
     got = run(lib, *d, mesh.n, mesh.dx, mesh.neighbors, g, flat, 1, ops, 1)
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("N,ops", [(8, ("dx", "dyy", "dz")), (16, ("dxx", "dy", "dzz")), (32, ("dx", "dz"))])
+def test_fp32_fields_are_widened_exactly(lib, N, ops):
+    """FP32 fields of every kind (normal, subnormal, zeros of either sign, the largest; one block with a NaN and
+    an infinity) give the FP32 rounding of what the same values give as FP64 fields."""
+    mesh = W.periodic_box_mesh(2, 2, 1, N, 4)
+    E = N + 8
+    r = W.rng(70 + N)
+    f = r.uniform(-1, 1, (4, 1, E ** 3)) * 2.0 ** r.integers(-12, 12, (4, 1, E ** 3))
+    f[1] *= 2.0 ** -140                               # subnormal in FP32, many to zero
+    f[2, 0, ::3] = np.where(r.uniform(size=len(f[2, 0, ::3])) < 0.5, -0.0, 3e38)
+    f[3, 0, E ** 3 // 2] = np.nan
+    f[3, 0, E ** 3 // 2 + 5] = np.inf
+    flat = f.astype(np.float32).reshape(-1)
+    d = (desc("Q13_1_d1"), desc("Q13_1_d2"))
+    dx = np.full((4, 3), 0.125)
+    with np.errstate(over="ignore", invalid="ignore"):
+        want = run(lib, *d, mesh.n, dx, mesh.neighbors, 4, flat.astype(np.float64), 1, ops, 0).astype(np.float32)
+    got = run(lib, *d, mesh.n, dx, mesh.neighbors, 4, flat, 1, ops, 0, f32=True).astype(np.float32)
+    assert np.array_equal(got, want, equal_nan=True)
