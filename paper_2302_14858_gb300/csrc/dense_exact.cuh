@@ -6,9 +6,11 @@
 //     D_ij / sigma_i = sum_t b_t 2^{-9-10t},   f_pj / tau_p = sum_s a_s 2^{-9-10s},  |a_s|, |b_t| <= 512,
 // each an integer that FP16 holds exactly.  A product of digits is below 2^18; the pairs of one level
 // k = s + t accumulate in the same FP32 TMEM columns, and levels k <= 3 (10 pairs) are kept.  A level
-// sum is bounded by 512 sum_j (|b_0| + .. + |b_k|); with the digits' mean of 256 that is below 2^24 for
-// levels 0-2, so these accumulators are exact integers, and a level-3 unit is 2^-48.  The dropped pairs
-// (three of level 4) and the 2^-40 roundings leave ~4 x 2^-40 sigma_i tau_p rms per output over K = 40
+// sum is bounded by 512 sum_j (|b_0| + .. + |b_k|), whatever the pencil: below 2^24 it is an exact integer.
+// Over every row of the Q13, P12 and X_2 operators (closed, iterated, cyclic; N = 16 and 32; up to eight spacings) the
+// largest bounds are 0.32, 0.65 and 0.92 of 2^24 for levels 1, 2 and 3; an operator whose digits are all near
+// 512 may exceed it and then rounds in units of 2 of that level (2^-37 and 2^-47 for levels 2 and 3).  The
+// dropped pairs (three of level 4) and the 2^-40 roundings leave ~4 x 2^-40 sigma_i tau_p rms per output over K = 40
 // columns; five base-256 digits with levels 0-4, the form before, left 4.5 x 2^-40 with 15 pairs.
 //
 // Measured (256^3 as 512 blocks of 32^3, 4 FP64 fields, nine ops: six launches, event times): five
@@ -147,13 +149,19 @@ __device__ __forceinline__ void release_levels(uint32_t t_empty) {
   if ((threadIdx.x & 31) == 0) mbar_arrive(t_empty);
 }
 
-// The levels of one output as a 64-bit integer in units of 2^-43 sigma tau: t1 = x0 2^10 + x1 exact
-// (|x0| < 2^21 - 2^14, see the row scale in exact_image), the two low levels joined in FP32 (their
-// sum rounds at 2^-24 of a level that is itself 2^-20 of the result's scale).
+// The levels of one output as a 64-bit integer in units of 2^-43 sigma tau, joined as integers: t1 = x0 2^10 + x1
+// (|x0| < 2^21 - 2^14, see the row scale in exact_image) and t2 = x2 2^5 + round(x3 2^-5), |t2| < 2^31 - 2^28.
+// The only rounding is the last level's, 2^-44 at most (the two low levels joined in FP32 rounded at 2^-24 of
+// their sum).  x0 and x3 2^-5 are below 2^22: adding 1.5 2^23 leaves their integer in the mantissa, at the cost of
+// an FP32 operation where a conversion takes eight.
 template <int C>
 __device__ __forceinline__ long long exact_y(const uint32_t (&acc)[kSl][C], int c) {
-  const int t1 = __float2int_rn(__uint_as_float(acc[0][c])) * 1024 + __float2int_rn(__uint_as_float(acc[1][c]));
-  const int t2 = __float2int_rn(fmaf(__uint_as_float(acc[2][c]), 32.0f, __uint_as_float(acc[3][c]) * 0.03125f));
+  constexpr float kBias = 12582912.0f;
+  constexpr uint32_t kBiasBits = 0x4B400000u;
+  const uint32_t x0 = __float_as_uint(__uint_as_float(acc[0][c]) + kBias);
+  const uint32_t x3 = __float_as_uint(fmaf(__uint_as_float(acc[3][c]), 0.03125f, kBias));
+  const int t1 = (int)(x0 * 1024u + (uint32_t)__float2int_rn(__uint_as_float(acc[1][c])) - kBiasBits * 1024u);
+  const int t2 = (int)((uint32_t)__float2int_rn(__uint_as_float(acc[2][c])) * 32u + x3 - kBiasBits);
   return ((long long)t1 << 15) + (long long)t2;
 }
 constexpr int kYUnit = 43, kFUnit = 48;  // result exponents: 2^(rowexp + etau - unit)
