@@ -237,10 +237,10 @@ __device__ __forceinline__ float to_float(double v) {
                            (hi & 0x80000000u));
   return a == 0 ? 0.0f : (float)v;
 }
-// A float as a double, exactly (zeros, and subnormals: below 1e-38, give zero).
+// A float as a double, exactly.
 __device__ __forceinline__ double to_double(float f) {
   const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
-  if (e == 0xFFu) return (double)f;
+  if (e == 0xFFu || (e == 0 && (u << 1) != 0)) return (double)f;
   return e == 0 ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xFFFFFu)), (int)(u << 29));
 }
 

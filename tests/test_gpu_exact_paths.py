@@ -335,3 +335,31 @@ def test_sizes_that_alternate_in_block_order(lib, g, dtype, nf, n_iter, offset):
                 for i in range(nops):
                     e = rel_max(got[N][:, q, i], want[N][:, q, i])
                     assert e < tol, (what, N, q, i, e)
+
+
+def test_dissipation_of_tiny_fields(lib):
+    """Fields near 2^-130: the FP32 dissipation sums are subnormal floats there and keep what those hold (2^-19 of
+    the fields), so the step is the ordinary one scaled, to a hundredth of what the dissipation contributes."""
+    import torch
+    from oracle import timestep as T
+    N, g, S = 16, 4, 2.0 ** -130
+    mesh = W.periodic_box_mesh(2, 2, 2, N, g)
+    E = N + 2 * g
+    flat = W.rng(41).uniform(-1, 1, (8, 2, E ** 3))
+    s = lib.cfd_scheme_create(desc("Q13_1_d1"), desc("Q13_1_d2"))
+    B = lib.cfd_blocks_bind(s, mesh.n, mesh.dx, mesh.neighbors, g, lib.CFD_F64)
+    dev, I = torch.device("cuda", 0), slice(g, g + N)
+
+    def step(scale, sigma):
+        u = [torch.from_numpy(flat[:, q].reshape(-1) * scale).to(dev) for q in range(2)]
+        work = torch.empty(lib.cfd_wave_lsrk_workspace(B, lib.CFD_TC_BF16_EXACT, 0), dtype=torch.uint8, device=dev)
+        lib.cfd_wave_lsrk_step(B, u[0], u[1], 0.1 * mesh.dx.min(), T.lsrk2s_rk4_float(), sigma, 4,
+                               lib.CFD_TC_BF16_EXACT, 0, work)
+        lib.cfd_sync_status(B)
+        return np.stack([v.cpu().numpy().reshape(8, E, E, E)[:, I, I, I] for v in u]) / scale
+
+    tiny, ordinary, without = step(S, 0.4), step(1.0, 0.4), step(1.0, 0.0)
+    for q in range(2):
+        effect = np.abs(ordinary[q] - without[q]).max()
+        assert effect > 0
+        assert np.abs(tiny[q] - ordinary[q]).max() < 1e-2 * effect, q
