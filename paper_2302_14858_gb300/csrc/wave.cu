@@ -228,11 +228,15 @@ __device__ __forceinline__ float to_float(double v) {
                            (hi & 0x80000000u));
   return a == 0 ? 0.0f : (float)v;
 }
-// A float as a double, exactly.
+// A float as a double, exactly, with integer instructions: subnormals are scaled up by 2^32 first.  (With a
+// conversion for them the compiler executes it always, and the step without shift at 128^3 took 629 us, not 600.)
 __device__ __forceinline__ double to_double(float f) {
-  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
-  if (e == 0xFFu || (e == 0 && (u << 1) != 0)) return (double)f;
-  return e == 0 ? 0.0 : __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u >> 3) & 0xFFFFFu)), (int)(u << 29));
+  const bool small = (__float_as_uint(f) & 0x7F800000u) == 0;
+  const unsigned u = __float_as_uint(small ? f * 0x1p32f : f), e = (u >> 23) & 0xFFu;
+  if (e == 0xFFu) return (double)f;
+  return e == 0 ? 0.0
+                : __hiloint2double((int)((u & 0x80000000u) | ((e + (small ? 864u : 896u)) << 20) | ((u >> 3) & 0xFFFFFu)),
+                                   (int)(u << 29));
 }
 
 // The right-hand side with FP32 stencil sums for N in {16, 32} and r = 4, the tensor-core steps' form.  A
