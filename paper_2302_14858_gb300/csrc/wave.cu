@@ -413,7 +413,7 @@ size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WaveLayout {
   size_t ext = 0, in = 0, apply = 0;
-  size_t total() const { return al(ext * 8) + al(in * 8) * 3 + al(3 * in * 8) + apply + 256; }
+  size_t total() const { return al(ext * 8) + al(in * 8) * 2 + al(3 * in * 8) + apply + 256; }
 };
 
 cfd_status wave_layout(cfd_blocks_s *B, cfd_precision prec, int n_iter, WaveLayout &L) {
@@ -453,7 +453,6 @@ extern "C" cfd_status cfd_wave_rk_step(cfd_blocks_t B, void *phi, void *K, doubl
   cudaStream_t st = (cudaStream_t)stream;
   char *base = (char *)(((uintptr_t)work + 255) & ~(uintptr_t)255);
   double *phis = (double *)base;  base += al(L.ext * 8);
-  base += al(L.in * 8);  // (unused: the size of the workspace is part of the interface)
   double *la = (double *)base;    base += al(L.in * 8);
   double *lb = (double *)base;    base += al(L.in * 8);
   double *lap = (double *)base;   base += al(3 * L.in * 8);
