@@ -107,10 +107,10 @@ cfd_status launch_exchange(cfd_blocks_s *B, void *fields, int nf, cudaStream_t s
       using T = decltype(tag);
       constexpr int V = decltype(vc)::value;
       dim3 grid((unsigned)((ghosts / V + 256 * kVPT - 1) / (256 * kVPT)), nblk * nf);
-      // Chained where the grid is about one wave (8 CTAs on each of 152 SMs), where launch latency counts: an
+      // Chained where the grid is about one wave (8 CTAs on each SM), where launch latency counts: an
       // exchange and d_x of one 32^3 block 10.2 -> 8.4 us.  Larger ones lose by starting in the tail of the
       // launch before (256^3, 4 fields, exchange and nine ops: 2.14 ms chained, 2.03 not).
-      const bool chained = (long long)grid.x * grid.y <= 8 * 152;
+      const bool chained = (long long)grid.x * grid.y <= 8ll * (B->num_sms > 0 ? B->num_sms : 148);
       launch_chained(k_exchange<T, decltype(nc)::value, decltype(gc)::value, V>, grid, 256, 0, st, chained,
                      static_cast<T *>(fields), nf, B->d_groups[gi], B->group_b0[gi], N, g, B->d_exch);
     };
