@@ -48,6 +48,13 @@ def arithmetic_name(prec: int, field_dtype: str) -> str:
             2: f"f16 digit slices, 10 exact-integer products in fp32, {io}",
             3: f"tf32, 1 product, fp32 accumulate, {io}"}[prec]
 
+
+def dense_kernel(prec: int) -> str:
+    """The tensor-core kernel of a precision and its arithmetic."""
+    return {1: "k_dense (tcgen05 GEMM, BF16 hi/lo split)", 2: "k_dense_exact (tcgen05 digit-slice GEMM)",
+            3: "k_dense (tcgen05 GEMM, TF32)"}[prec]
+
+
 WORKLOADS = {
     # one periodic 32^3 block (no interfaces: the undecomposed cyclic scheme), one field (8 sine modes,
     # integer k in [1, 12]), d_x only with the 6th-order tridiagonal Pade P^1_2: launch-bound
@@ -783,9 +790,9 @@ def main():
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         byts = algorithmic_bytes(nint, nf, nops, elem) * prof_steps
         achieved = byts / (tl * 1e-3) / 1e9
-        pairs = 10 if prec == PREC["tc_bf16_exact"] else 3
+        pairs = {"tc_bf16_exact": 10, "tc_bf16x3": 3, "tc_tf32": 1}[next(k for k, v in PREC.items() if v == prec)]
         tcf = tc_flops(mesh, nf, pairs) * prof_steps / (tl * 1e-3) / 1e12 if nops == 9 else None
-        roof = {"kernel": "k_dense_exact (tcgen05 digit-slice GEMM)", "bound": "hbm", "achieved": round(achieved, 1),
+        roof = {"kernel": dense_kernel(prec), "bound": "hbm", "achieved": round(achieved, 1),
                 "peak": hbm, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic_bytes_per_point_op": round(elem * (1 + nops) / nops, 3),
@@ -1107,7 +1114,7 @@ def run_advect(args, spec):
         ach = per_pf * units * prof_steps / (tdl * 1e-3) / 1e9
         nhl, thl = prof["dense_halo"]
         comb_b = (3 + 1 + 3 / nf) * elem * units * prof_steps
-        roof = {"kernel": "k_dense_exact (tcgen05 digit-slice GEMM, biased operators D+ and D-)", "bound": "hbm",
+        roof = {"kernel": dense_kernel(prec) + ", biased operators D+ and D-", "bound": "hbm",
                 "achieved": round(ach, 1), "peak": hbm, "unit": "GB/s", "frac": round(ach / hbm, 4),
                 "peak_source": "measured" if "hbm_gbs" in peaks else "fallback",
                 "algorithmic_bytes_per_point_field": round(per_pf, 2),

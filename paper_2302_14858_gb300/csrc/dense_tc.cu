@@ -364,8 +364,8 @@ __device__ __forceinline__ void digits_of(long long F, uint32_t (&out)[S]) {
 //
 // Persistent, one CTA of 16 warps per SM, warp-specialised:
 //   warps 0-7   producers: stage the next tile's pencils (TMA boxes, or
-//               cp.async), split the current one into 5 digit rows of A[buf]
-//               (two A buffers), publish the pencil scales (meta_full); then
+//               cp.async), split the current one into S digit rows of A[buf]
+//               (two for the hi/lo split, one for TF32; two A buffers), publish the pencil scales (meta_full); then
 //               thread 0 issues tcgen05.mma for every pass of the tile into
 //               one of three TMEM pass buffers (t_full on commit) and frees
 //               A[buf] with a last commit (a_empty);
@@ -1662,8 +1662,10 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
 // One halo pass of the hybrid iteration along the stage's axis: the four rows of every pencil that the
 // neighbours read, from the pencils (first iterate) or with the previous iterate's halo columns.
 //   exact: four of 16 operator rows through the tensor cores (dense_exact.cuh).  256^3, 4 FP64 fields,
-//     six passes: 0.95 ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
-//     coefficient and row where the digit split costs ~20 instructions per value for all rows;
+//     six passes: HALOMS ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
+//     coefficient and row where the digit split costs ~20 instructions per value for all rows.  The rows carry
+//     2^-40 of the pencil scale instead of 2^-46 of sum |c f|, as the final pass's own inputs do: errors of the
+//     outputs against 64 bits 1.2e-10 -> 1.1e-10 (2-norm, 256^3, nine ops, one iteration; n_iter 2 likewise);
 //   otherwise compensated FP32 on the CUDA cores (halo_rows.cu), whose cost does not depend on the form.
 static cfd_status halo_pass(DenseParams H, const DenseOp &op, const HaloRows &rows, bool exact, bool f32, int sms,
                             cudaStream_t st) {

@@ -15,9 +15,9 @@
 //   - each coefficient is an FP32 pair c = c_h + c_l, prepared on the host;
 //   - per row, c_h f_h is formed exactly (product and FMA residual) and added with TwoSum into
 //     a (sum, error) pair; c_h f_l + c_l f_h and the residuals go into the error word.
-// The result carries ~2^-46 relative to sum_j |c_j f_j|, more than the tensor-core digits keep
-// (2^-39 of the pencil scale), so the final pass sees the same halo values to its own
-// accuracy.  A NaN or an infinity in a pencil makes its four values NaN, as on the tensor-core
+// The result carries ~2^-46 relative to sum_j |c_j f_j|, far more than the two digits or the TF32 product of
+// the final pass keep.  (The exact form's own halo rows carry 2^-40 of the pencil scale; its outputs with
+// iteration are no further from 64 bits than with these, see halo_pass in dense_tc.cu.)  A NaN or an infinity in a pencil makes its four values NaN, as on the tensor-core
 // path.  The pencil addressing is the tensor-core stage's own.
 #include <cuda_runtime.h>
 

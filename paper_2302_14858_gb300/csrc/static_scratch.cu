@@ -8,8 +8,9 @@
 // Such callers can still bind the blocks once at start-up; this entry point
 // then needs no workspace argument and allocates nothing per call.
 //
-// The scratch it needs (the D_j intermediate of the mixed derivatives, on rows
-// extended along i) lives in one file-scope device array of fixed size.  Every
+// The scratch it needs (the ghost strips of the mixed derivatives' inner
+// derivative, and one copy of its own points where d_j is no FP64 output)
+// lives in one file-scope device array of fixed size.  Every
 // GPU that loads this library holds that array until the process exits.  Host
 // code cannot use the array's name as a device address, so the address is
 // looked up with cudaGetSymbolAddress once per device (on the first call made
