@@ -99,10 +99,10 @@ DEFAULT_WORKLOAD = "cfd256_b32_f4_fp64"
 MEASURED_TRAFFIC = {
     # 256^3 as 512 blocks of 32^3, 4 FP64 fields, 9 ops: one-pass capture of the 6 k_dense_exact
     # launches of a step at full size (profiles/launches_cfd256_b32_f4_tc_exact.md)
-    ("cfd256_b32_f4_fp64", "tc_bf16_exact", 0): 1414757547,
+    ("cfd256_b32_f4_fp64", "tc_bf16_exact", 0): 1414769024,
     # 448 x 16^3 + 64 x 32^3, 22 FP32 fields, 9 ops: one-pass capture of the 24 k_dense_exact launches
     # of a step at full size (profiles/launches_box448x16_64x32_f22_fp32_tc_exact.md)
-    ("box448x16_64x32_f22_fp32", "tc_bf16_exact", 0): 415434016,
+    ("box448x16_64x32_f22_fp32", "tc_bf16_exact", 0): 415397419,
 }
 
 

@@ -70,8 +70,9 @@ typedef enum cfd_status {
  *   - outputs that overflow become infinities; FP64 outputs below the normal
  *     range flush to zero, FP32 outputs round as IEEE.
  * With n_iter > 0 the values the neighbours read at their k^c nodes (the halo
- * rows of each iterate) come from a pass of the same arithmetic (BF16X3 and
- * TF32: from the CUDA cores in compensated FP32), then enter the final pass as
+ * rows of each iterate) come from a pass of the same arithmetic, 2^-40 of the
+ * pencil's scale (BF16X3 and TF32: from the CUDA cores in compensated FP32,
+ * ~2^-46 of sum_j |c_j f_j|), then enter the final pass as
  * four extra inputs of each pencil in the format above.
  */
 typedef enum cfd_precision {

@@ -17,10 +17,11 @@
 // BF16 digits with 15 pairs, 8 + 8 warps, one staging buffer 2.87 ms in all; this form with 8 epilogue
 // warps 2.69; with 16 epilogue warps and TMA stores of the x outputs 2.03 (S_x 0.37, S_y 0.45, S_z 0.48,
 // T_x 0.25, T_y 0.24 ms); direct outer stages, the operator's load behind the first tiles and a quarter of
-// the outputs converted by integers 1.79 (S 0.36 to 0.37, T 0.24 to 0.25).  A producer's value costs ~20
-// instructions against ~45 before, an output ~15 against ~28.  What bounds it now: T stages DRAM; S stages
-// DRAM (0.25 ms at the copy rate) and the FP64 pipe (48 conversions of 64 cycles per SM sub-partition and
-// tile, 0.17 ms) beside the integer work, no one of them alone.
+// the outputs converted by integers 1.79 (S 0.36 to 0.37, T 0.24 to 0.25); x stages compiled for one staging
+// and levels 0 and 3 made integers by an FP32 add 1.73 (S 0.34 to 0.35, T 0.23 to 0.24).  A producer's value
+// costs ~20 instructions against ~45 before, an output ~14 against ~28.  What bounds it now: T stages DRAM; S
+// stages DRAM (0.25 ms at the copy rate) and the FP64 pipe (48 conversions of 64 cycles per SM sub-partition
+// and tile, 0.17 ms) beside the integer work, no one of them alone.
 //
 // Roles (28 warps, one persistent CTA per SM):
 //   warps 0-7    producers: wait for a staged tile, split it into 4 digit rows of A[buf];
@@ -177,7 +178,8 @@ __device__ __forceinline__ float exact_f(const uint32_t (&acc)[kSl][C], int c) {
 
 // y 2^E for |y| < 2^53 and a result in the normal range (0 for y = 0): exact either way, by the FP64 pipe's
 // conversion (64 cycles per warp) or by integer instructions (some 30 more than the other way's few).  The
-// FP64 pipe is the busier: 0.23 of a 256^3 two-degree stage's 0.37 ms when it converts every output.
+// FP64 pipe is the busier: 0.23 of a 256^3 two-degree stage's 0.35 ms if it converted every output (0.17 with
+// three in four).
 template <bool INT>
 __device__ __forceinline__ double scaled_y(long long y, int E) {
   if constexpr (INT) {

@@ -1662,7 +1662,7 @@ cfd_status launch_stage(DenseState *ds, const DenseParams &P, int KP, int S, int
 // One halo pass of the hybrid iteration along the stage's axis: the four rows of every pencil that the
 // neighbours read, from the pencils (first iterate) or with the previous iterate's halo columns.
 //   exact: four of 16 operator rows through the tensor cores (dense_exact.cuh).  256^3, 4 FP64 fields,
-//     six passes: HALOMS ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
+//     six passes: 0.95 ms, against 2.02 ms in compensated FP32, which spends ~11 FP32 operations per
 //     coefficient and row where the digit split costs ~20 instructions per value for all rows.  The rows carry
 //     2^-40 of the pencil scale instead of 2^-46 of sum |c f|, as the final pass's own inputs do: errors of the
 //     outputs against 64 bits 1.2e-10 -> 1.1e-10 (2-norm, 256^3, nine ops, one iteration; n_iter 2 likewise);

@@ -17,9 +17,9 @@
 // Mixed derivatives take the inner derivative from the d_j output (or one FP64 copy of it) and only
 // the ghost strips are solved again, where the version before solved the extended pencils for each of
 // the six ordered pairs.  128^3 as 512 blocks of 16^3, 4 fields, nine ops, one iteration: 8.41 -> 3.03 ms
-// (526 -> ~150 FP64 operations per point); 27 blocks of 16^3, one field: 447 -> 162 us in 15 launches
-// instead of 37.  Small launches are a chain of latencies: one op of 2^3 blocks of 8^3 takes 5.5 to 7.2 us
-// (6.3 to 9.0 with loads eight at a time and the table read through registers), of 16^3 8.7 to 10.1 us.
+// (526 -> ~150 FP64 operations per point); 27 blocks of 16^3, one field: 447 -> 156 us in 15 launches
+// instead of 37.  Small launches are a chain of latencies: d_x and d_xx of 2^3 blocks of 8^3 take 6.0 and 7.1 us
+// (8.4 and 9.1 with loads eight at a time and the table through registers), of 16^3 8.4 and 10.0 (11.7, 13.1).
 #include <stddef.h>
 
 #include <algorithm>
